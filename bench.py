@@ -104,11 +104,11 @@ CAP = 1 << 24
 # again (tests/test_bench_counts.py fails until they are), and until then
 # the roofline reports no fraction.  Family codes: 0 oscillatory, 1 product
 # peak, 2 corner peak, 3 Gaussian, 4 C0.
-RULE_FP64_INST_D8 = {0: 5631.0, 1: 2476.0, 2: 4829.0, 3: 4136.0, 4: 4080.0}
-RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
-RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_region64.cuh", "gmq_families.cuh",
+RULE_FP64_INST_D8 = {0: 1779.0, 1: 1063.0, 2: 4829.0, 3: 1219.0, 4: 1163.0}
+RULE_FP64_FLOPS_D8 = {0: 2992.0, 1: 1649.0, 2: 6075.0, 3: 1895.0, 4: 1839.0}
+RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_region64.cuh", "gmq_families.cuh",
                        "gm_math_tables.cuh", "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "fcb577d59be93b60"
+RULE_COUNTS_SHA16 = "414fefa5b8798a8c"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -122,7 +122,7 @@ RULE_COUNTS_SHA16 = "fcb577d59be93b60"
 MIXED_FP32_OPS_D12 = {2: 116237.0, 3: 134179.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "c1f3307de3c65ba1"
+MIXED_COUNTS_SHA16 = "8ec0e6ec17be2d1d"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):
@@ -200,7 +200,8 @@ def eval_modes(ctx, stream):
     event-timed launches per family and mode on the context stream.  The
     default forms each node's S from per-axis terms (separable); node-wise
     evaluates f from every node's coordinates, as an integrand without that
-    form would be.  Both evaluate g at every node."""
+    form would be.  Both form the value of every node (products of per-axis
+    factors where the integrand has them)."""
     import torch
     from paper_2511_01573_gb300 import genz_inputs as G
     from paper_2511_01573_gb300 import gmq

@@ -633,11 +633,6 @@ __global__ void k_batch_advance(const BatchArgs B) {
   if (B.use_cond) cudaGraphSetConditional(B.cond, more ? 1u : 0u);
 }
 
-size_t batch_rule_smem(int dmax) {
-  const size_t pairs = sizeof(unsigned short) * (size_t)batch_pairs_offset(dmax + 1);
-  return (sizeof(double) * (size_t)batch_rule_doubles_max(dmax) + pairs + 15) & ~(size_t)15;
-}
-
 cudaError_t batch_launch_partition(const BatchArgs& B, cudaStream_t s) {
   k_batch_partition<<<B.count, 256, 0, s>>>(B);
   return cudaGetLastError();

@@ -119,27 +119,10 @@ __host__ __device__ inline int batch_lanes_for(const BatchArgs& B, long long n) 
 }
 
 
-// Doubles of the FP64 rule kernel's per-block region workspaces for T lanes
-// per region: 128 / T workspaces of the largest layout over dimensions
-// 1 .. dmax (gm_region64.cuh; flag masks included for every family); the
-// kernel sizes its shared memory for the largest over T.
-__host__ __device__ constexpr long long batch_rule_doubles(int dmax, int T) {
-  return (long long)sep_words_max(dmax, true, T > 1) * (kBatchRuleBlock / T);
-}
-__host__ __device__ constexpr long long batch_rule_doubles_max(int dmax) {
-  long long m = batch_rule_doubles(dmax, 1);
-  if (batch_rule_doubles(dmax, 4) > m) m = batch_rule_doubles(dmax, 4);
-  if (batch_rule_doubles(dmax, 32) > m) m = batch_rule_doubles(dmax, 32);
-  if (batch_rule_doubles(dmax, 128) > m) m = batch_rule_doubles(dmax, 128);
-  return m;
-}
-
 // Pair tables of every dimension 2 .. dmax, one after the other: the table
 // of dimension d starts at entry d (d - 1) (d - 2) / 6.
 __host__ __device__ constexpr int batch_pairs_offset(int d) { return d * (d - 1) * (d - 2) / 6; }
 
-// Shared memory of the FP64 rule kernel for the largest dimension.
-size_t batch_rule_smem(int dmax);
 cudaError_t batch_launch_partition(const BatchArgs& B, cudaStream_t s);
 // FP64 rule evaluation of the current list's regions of family FAM
 // (gm_batch_rule64.cuh; one launch per family present in the batch,

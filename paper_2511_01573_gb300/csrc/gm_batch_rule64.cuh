@@ -11,9 +11,31 @@
 #pragma once
 
 #include "gm_batch.cuh"
-#include "gm_region64.cuh"
+#include "gm_factor64.cuh"
 
 namespace gmq {
+
+// Doubles of the per-block region workspaces of family FAM: 128 / T
+// workspaces of the largest layout over dimensions 1 .. dmax, the largest
+// over T (T is chosen per sweep on the device).
+template <int FAM>
+__host__ __device__ constexpr long long batch_rule_doubles_max(int dmax) {
+  long long m = 0;
+  for (int T = 1; T <= kBatchRuleBlock; T *= T == 1 ? 4 : (T == 4 ? 8 : 4)) {
+    const long long w = (long long)region64_words_max(dmax, Fac<FAM>::kind, Sep<FAM>::kFlag, T > 1) *
+                        (kBatchRuleBlock / T);
+    if (w > m) m = w;
+  }
+  return m;
+}
+
+// Shared memory of the FP64 rule kernel of family FAM for the largest
+// dimension.
+template <int FAM>
+size_t batch_rule_smem(int dmax) {
+  const size_t pairs = sizeof(unsigned short) * (size_t)batch_pairs_offset(dmax + 1);
+  return (sizeof(double) * (size_t)batch_rule_doubles_max<FAM>(dmax) + pairs + 15) & ~(size_t)15;
+}
 
 template <int FAM, int T>
 __device__ __forceinline__ void batch_rule64_lanes(const BatchArgs& B, double* smem,
@@ -42,8 +64,8 @@ __device__ __forceinline__ void batch_rule64_lanes(const BatchArgs& B, double* s
       h = H[(int64_t)k * ld + r];
     };
     RegionSums o;
-    region_sums64<FAM, T>(it.P, d, pairs_all + batch_pairs_offset(d), ch, B.lam2, B.lam3,
-                          B.lam5, wsp, RPB, B.ratio, o);
+    region_sums<FAM, T>(it.P, d, pairs_all + batch_pairs_offset(d), ch, B.lam2, B.lam3, B.lam5,
+                        wsp, RPB, B.ratio, o);
     if (lane == 0)
       region_finish64(
           o, d, it.w7, it.w5, B.estimator ? it.nw : nullptr, it.vol_omega,
@@ -59,7 +81,7 @@ template <int FAM>
 __global__ void __launch_bounds__(kBatchRuleBlock) k_batch_rule64(const BatchArgs B) {
   extern __shared__ __align__(16) double smem[];
   const int dm = B.dmax;
-  unsigned short* pairs_all = reinterpret_cast<unsigned short*>(smem + batch_rule_doubles_max(dm));
+  unsigned short* pairs_all = reinterpret_cast<unsigned short*>(smem + batch_rule_doubles_max<FAM>(dm));
   for (int e = 2; e <= dm; ++e) {
     const int np = e * (e - 1) / 2;
     for (int p = threadIdx.x; p < np; p += blockDim.x) {
@@ -85,7 +107,7 @@ __global__ void __launch_bounds__(kBatchRuleBlock) k_batch_rule64(const BatchArg
 
 template <int FAM>
 cudaError_t batch_launch_rule64_family(const BatchArgs& B, int grid, cudaStream_t s) {
-  const size_t smem = batch_rule_smem(B.dmax);
+  const size_t smem = batch_rule_smem<FAM>(B.dmax);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_batch_rule64<FAM>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -98,7 +120,7 @@ cudaError_t batch_launch_rule64_family(const BatchArgs& B, int grid, cudaStream_
 template <int FAM>
 int batch_rule64_max_blocks_family(int dmax) {
   int nb = 0;
-  const size_t smem = batch_rule_smem(dmax);
+  const size_t smem = batch_rule_smem<FAM>(dmax);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_batch_rule64<FAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);

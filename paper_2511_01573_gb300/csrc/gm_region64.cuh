@@ -245,15 +245,6 @@ __host__ __device__ constexpr SepLayout sep_layout(int d, bool flag, bool lanes)
   return s;
 }
 
-// The largest workspace over dimensions 1 .. dmax (batched kernels, whose
-// regions have different dimensions).
-__host__ __device__ constexpr int sep_words_max(int dmax, bool flag, bool lanes) {
-  int m = 0;
-  for (int d = 1; d <= dmax; ++d)
-    if (sep_layout(d, flag, lanes).words > m) m = sep_layout(d, flag, lanes).words;
-  return m;
-}
-
 // The class sums and the fourth-difference argmax of one region by the T
 // lanes of the calling group (all of them call it).  ch(k, c, h) loads the
 // region's centre and half-width on axis k; pairs[p] = (j << 8) | k for the

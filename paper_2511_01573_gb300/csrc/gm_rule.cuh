@@ -8,24 +8,24 @@
 // region).  Each group
 //   1. reads its region's centres and half-widths from the structure-of-
 //      arrays list (consecutive threads read consecutive regions of one
-//      axis: coalesced) and builds the region's separable workspace in
-//      shared memory: the integrand's per-axis terms at the seven
-//      coordinate values of each axis, their prefix and suffix chains and
-//      the class-5 partial chains (gm_region64.cuh);
+//      axis: coalesced) and builds the region's workspace in shared memory:
+//      the factors of its coordinates and their class-5 partial products
+//      (gm_factor64.cuh), or, for integrands that do not factor, per-axis
+//      terms and partial chains of the inner sum (gm_region64.cuh);
 //   2. walks each class of nodes by index: a node's axes and signs are
 //      decoded from the bits of its index (centre; 4d axis nodes; 4 sign
 //      patterns per axis pair; the 2^d sign patterns of the last class are
-//      the bits of the index itself), its S combined from the workspace in
-//      one or two operations, so the FP64 work per node is the integrand's
-//      outer function and one accumulation;
+//      the bits of the index itself).  Every node's value is formed and
+//      added: one fused multiply-add of two factors, or the outer function
+//      of its inner sum and an add;
 //   3. combines the class sums over the T lanes, finds the split axis
 //      (argmax of the fourth differences) and writes I7, the error estimate,
 //      vol / vol(Omega) and the axis byte.
-// The per-region work is region_sums64 / region_finish64 of gm_region64.cuh,
-// whose fixed summation tree makes the results bit-identical for every T.
+// The per-region work is region_sums (gm_factor64.cuh) and region_finish64
+// (gm_region64.cuh), whose fixed summation tree makes the results bit-identical for every T.
 #pragma once
 
-#include "gm_region64.cuh"
+#include "gm_factor64.cuh"
 #include "gmq_common.cuh"
 #include "gmq_families.cuh"
 
@@ -43,11 +43,13 @@ inline size_t rule_smem_bytes(int d, int T, int real_bytes) {
   return (bytes + 15) & ~(size_t)15;
 }
 
-// Shared-memory bytes of the FP64 rule kernel: RB workspaces of the region
-// layout, the family parameters and the pair table.
-inline size_t rule64_smem_bytes(int d, int T, bool flag) {
+// Shared-memory bytes of the FP64 rule kernel: RB region workspaces, the
+// family parameters and the pair table.
+template <int FAM>
+inline size_t rule64_smem_bytes(int d, int T) {
   const int RB = kRuleBlock / T;
-  size_t bytes = sizeof(double) * (size_t)sep_layout(d, flag, T > 1).words * RB;
+  size_t bytes = sizeof(double) * RB *
+                 (size_t)region64_words(d, Fac<FAM>::kind, Sep<FAM>::kFlag, T > 1);
   bytes += sizeof(SmemParams<double>) + sizeof(unsigned short) * 128;
   return (bytes + 15) & ~(size_t)15;
 }
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(kRuleBlock) k_rule64(const RuleArgs A) {
   constexpr int RB = kRuleBlock / T;
   extern __shared__ __align__(16) double smem[];
   const int d = A.P.d;
-  const int words = sep_layout(d, Sep<FAM>::kFlag, T > 1).words;
+  const int words = region64_words(d, Fac<FAM>::kind, Sep<FAM>::kFlag, T > 1);
   double* wsp = smem;  // [words][RB] region workspaces
   SmemParams<double>* P = reinterpret_cast<SmemParams<double>*>(wsp + (size_t)words * RB);
   unsigned short* pairs = reinterpret_cast<unsigned short*>(P + 1);
@@ -94,8 +96,7 @@ __global__ void __launch_bounds__(kRuleBlock) k_rule64(const RuleArgs A) {
     h = H[(int64_t)k * ld];
   };
   RegionSums o;
-  region_sums64<FAM, T>(*P, d, pairs, ch, A.R.lam2, A.R.lam3, A.R.lam5, wsp + g, RB, A.R.ratio,
-                        o);
+  region_sums<FAM, T>(*P, d, pairs, ch, A.R.lam2, A.R.lam3, A.R.lam5, wsp + g, RB, A.R.ratio, o);
   if ((tid & (T - 1)) == 0)
     region_finish64(
         o, d, A.R.w7, A.R.w5, A.R.estimator ? A.R.nw : nullptr, A.R.vol_omega,
@@ -194,7 +195,7 @@ cudaError_t launch_rule64_t(const RuleArgs& A, cudaStream_t s) {
     k_rule64_nodewise<FAM, T><<<(unsigned)blocks, kRuleBlock, smem, s>>>(A);
     return cudaGetLastError();
   }
-  const size_t smem = rule64_smem_bytes(A.P.d, T, Sep<FAM>::kFlag);
+  const size_t smem = rule64_smem_bytes<FAM>(A.P.d, T);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_rule64<FAM, T>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
