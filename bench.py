@@ -94,21 +94,28 @@ def workload(args):
 
 CAP = 1 << 24
 
-# FP64 work of the rule kernel per region at d = 8 (401 nodes), per family:
-# FP64 thread-instructions (sm__thread_inst_executed_pipe_fp64_pred_on) and
-# flops (FMA = 2), from the ncu counters of a launch over 2^20 regions
-# (bench.py --probe-rule under ncu).  The counts are fixed by the integrand,
-# d and the compiled kernel: the four families take no data-dependent
-# branch.  They hold for the kernel sources whose fingerprint is
-# RULE_COUNTS_SHA16; when those sources change the counts must be taken
-# again (tests/test_bench_counts.py fails until they are), and until then
-# the roofline reports no fraction.  Family codes: 0 oscillatory, 1 product
-# peak, 2 corner peak, 3 Gaussian, 4 C0.
-RULE_FP64_INST_D8 = {0: 1779.0, 1: 1063.0, 2: 4829.0, 3: 1219.0, 4: 1163.0}
-RULE_FP64_FLOPS_D8 = {0: 2992.0, 1: 1649.0, 2: 6075.0, 3: 1895.0, 4: 1839.0}
-RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_region64.cuh", "gmq_families.cuh",
-                       "gm_math_tables.cuh", "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "414fefa5b8798a8c"
+# FP64 work of the rule at d = 8 (401 nodes) per region and family, as FP64
+# thread-instructions and flops (FMA = 2): what the separable form, which
+# evaluates the integrand's outer function at every node, spends on it (ncu,
+# sm__thread_inst_executed_pipe_fp64_pred_on over 2^20 regions).  A fixed unit
+# of work.  Family codes: 0 oscillatory, 1 product peak, 2 corner peak,
+# 3 Gaussian, 4 C0.
+RULE_FP64_INST_D8 = {0: 5631.0, 1: 2476.0, 2: 4829.0, 3: 4136.0, 4: 4080.0}
+RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
+
+# What the rule kernel executes on the FP64 pipe for it (the rest of its
+# arithmetic runs on the integer pipes), from the ncu counters of a launch over
+# 2^20 regions (bench.py --probe-rule under ncu).  The counts are fixed by the
+# integrand, d and the compiled kernel: the families take no data-dependent
+# branch on the benchmark's regions.  They hold for the kernel sources whose
+# fingerprint is RULE_COUNTS_SHA16; when those sources change the counts must
+# be taken again (tests/test_bench_counts.py fails until they are), and until
+# then the roofline reports no fraction.
+RULE_EXEC_FP64_INST_D8 = {0: 1779.0, 1: 1063.0, 2: 241.0, 3: 1219.0, 4: 1163.0}
+RULE_EXEC_FP64_FLOPS_D8 = {0: 2992.0, 1: 1649.0, 2: 231.0, 3: 1895.0, 4: 1839.0}
+RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_region64.cuh",
+                       "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
+RULE_COUNTS_SHA16 = "09ed4e24fb774ec5"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -1076,11 +1083,11 @@ def main():
     roof = None
     clocks = clk.summary()
     counts_current = rule_source_fingerprint() == RULE_COUNTS_SHA16
-    if rule["launches"] and all(f in RULE_FP64_INST_D8 for f in timed_fam_regions):
+    if rule["launches"] and all(f in RULE_EXEC_FP64_INST_D8 for f in timed_fam_regions):
         n_launch = rule["launches"]
         avg_s = rule["ms"] / 1000.0 / n_launch
-        inst = sum(RULE_FP64_INST_D8[f] * n for f, n in timed_fam_regions.items()) / n_launch
-        flops = sum(RULE_FP64_FLOPS_D8[f] * n for f, n in timed_fam_regions.items()) / n_launch
+        inst = sum(RULE_EXEC_FP64_INST_D8[f] * n for f, n in timed_fam_regions.items()) / n_launch
+        flops = sum(RULE_EXEC_FP64_FLOPS_D8[f] * n for f, n in timed_fam_regions.items()) / n_launch
         mhz = clocks.get("sm_mhz") or 2070.0
         peak_nominal = 2 * 152 * mhz * 1e6 / 1e9  # G FP64 lane-inst/s
         peak = probe64 / 1e9
@@ -1100,7 +1107,7 @@ def main():
                 "counts_match_source": counts_current,
                 "flops_view": {"achieved_gflops": flops / avg_s / 1e9,
                                "peak_gflops_measured_fma": 2 * probe_ops["fma"] / 1e9},
-                "inst_per_region": {G.FAMILY_NAMES[f]: RULE_FP64_INST_D8[f]
+                "inst_per_region": {G.FAMILY_NAMES[f]: RULE_EXEC_FP64_INST_D8[f]
                                     for f in sorted(timed_fam_regions)},
                 "regions_by_family": {G.FAMILY_NAMES[f]: n // args.steps
                                       for f, n in sorted(timed_fam_regions.items())}}

@@ -35,6 +35,7 @@
 // reversed order, as in gm_region64.cuh.
 #pragma once
 
+#include "gm_fixed64.cuh"
 #include "gm_region64.cuh"
 
 namespace gmq {
@@ -710,9 +711,9 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
 }
 
 // The class sums and the split axis of one region: from per-axis factors
-// where the integrand has them, from the separable form otherwise (the
-// corner peak and the polynomial; the cosine above d = 14; a region whose
-// factors lack exponent room).  Arguments as region_sums64; w points at the
+// where the integrand has them, in fixed point for the corner peak, from the
+// separable form otherwise (the polynomial; the cosine above d = 14; a region
+// whose factors or inner sums lack exponent room).  Arguments as region_sums64; w points at the
 // region's workspace of region64_words(d, ...) entries.
 template <int FAM, int T, class PT, class CH>
 __device__ __forceinline__ void region_sums(const PT& P, int d, const unsigned short* pairs,
@@ -725,6 +726,9 @@ __device__ __forceinline__ void region_sums(const PT& P, int d, const unsigned s
       region_sums64_rotation<FAM, T>(P, d, pairs, ch, lam2, lam3, lam5, w, ws, ratio, o);
       return;
     }
+  }
+  if constexpr (FAM == GMQ_CORNER_PEAK) {
+    if (region_sums64_corner<T>(P, d, pairs, ch, lam2, lam3, lam5, w, ws, ratio, o)) return;
   }
   region_sums64<FAM, T>(P, d, pairs, ch, lam2, lam3, lam5, w, ws, ratio, o);
 }
