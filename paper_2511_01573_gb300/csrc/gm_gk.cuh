@@ -12,15 +12,26 @@
 // index on ties), or the widest axis when every E_k is below 1e-11 of the
 // magnitude of the terms (prod h_k sum |wK f|).  d <= GMQ_GK_MAX_DIM.
 //
-// Mapping: one warp per region, four regions per 128-thread block.  The
-// node grid is walked by rows -- a row fixes the digits of axes 1..d-1 and
-// runs axis 0 over its 15 nodes -- lane l taking rows l, l + 32, ...; the
-// weight products of axes >= 1 and the E_k terms of axes >= 1 are formed
-// once per row (E_k += r_k[i_k] * (row sum of wK f), r = 1 - wG / wK), so
-// per node the FP64 work is the integrand and five operations.  Warp
-// butterflies combine the lanes' sums in a fixed order.
+// Mapping: a 128-thread block per region for d >= 4 (3375 rows and more), a
+// warp per region below.  The node grid is walked by rows -- a row fixes the
+// digits of axes 1..d-1 and runs axis 0 over its 15 nodes -- lane l of the L
+// lanes of a region taking rows l, l + L, ...  Butterflies, then a fixed
+// order over the warps, combine the lanes' sums.
+//
+// Bound: the FP64 pipe.  Integrands that are products of one factor per axis
+// (gm_factor64.cuh) hold wK e for the 15 nodes of every axis, relative to
+// the centre's value; a row is the product of its digits' entries, and each
+// node costs two fused multiply-adds (its terms of I_K and of E_0), about 20
+// fewer FP64 instructions than an evaluation of f with its weights.  Row sums
+// give the E_k of the other axes.  The nodes of I_G are the 7^d with odd
+// digits; they are walked on their own, because a lane that skips the term
+// saves nothing when another lane of its warp needs it.  f >= 0 for these
+// integrands, so sum |wK f| is I_K's sum.  d = 4, C0, 2500 regions: 6.57 ->
+// 0.71 ms.  Other integrands, and regions whose factors lack exponent room,
+// evaluate f at every node.
 #pragma once
 
+#include "gm_factor64.cuh"
 #include "gmq_common.cuh"
 #include "gmq_families.cuh"
 
@@ -40,42 +51,59 @@ struct GkArgs {
   const GkConst* K;  // device copy of the tables
 };
 
-constexpr int kGkWarps = 4;  // regions per block
+constexpr int kGkBlock = 128;
 
-template <int FAM>
-__global__ void __launch_bounds__(32 * kGkWarps) k_rule_gk(const GkArgs G) {
-  __shared__ GkConst K;
-  __shared__ SmemParams<double> P;
-  __shared__ double xt[kGkWarps][GMQ_GK_MAX_DIM * 15];  // node coordinates per axis
-  __shared__ double xs[kGkWarps][GMQ_GK_MAX_DIM][32];   // each lane's current node
-  const RuleArgs& A = G.A;
-  const int d = A.P.d;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  for (int i = tid; i < 60; i += blockDim.x) (&K.x[0])[i] = (&G.K->x[0])[i];
-  for (int j = tid; j < d; j += blockDim.x) {
-    P.a[j] = A.P.a[j];
-    P.u[j] = A.P.u[j];
-    P.b[j] = A.P.b[j];
+// Sums of one region: I_K, I_G, sum |wK f| and the directional terms,
+// without the factor prod h_k.
+struct GkSums {
+  double K = 0.0, G = 0.0, A = 0.0;
+  double E[GMQ_GK_MAX_DIM];
+};
+
+// Combine the sums of the region's 32 W lanes in a fixed order: every lane
+// of the region's first warp returns the total.  scratch: [W][9].
+template <int W>
+__device__ __forceinline__ void gk_combine(GkSums& s, double* scratch) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s.K += __shfl_xor_sync(0xffffffffu, s.K, off);
+    s.G += __shfl_xor_sync(0xffffffffu, s.G, off);
+    s.A += __shfl_xor_sync(0xffffffffu, s.A, off);
+#pragma unroll
+    for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] += __shfl_xor_sync(0xffffffffu, s.E[k], off);
   }
-  if (tid == 0) P.c0 = A.P.c0;
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * kGkWarps + w;
-  const bool active = r < A.n;
-  if (active)
-    for (int q = lane; q < d * 15; q += 32) {
-      const int k = q / 15, j = q - 15 * k;
-      xt[w][q] = fma(K.x[j], A.h[(int64_t)k * A.ld + r], A.c[(int64_t)k * A.ld + r]);
+  if constexpr (W > 1) {
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+      double* o = scratch + w * (3 + GMQ_GK_MAX_DIM);
+      o[0] = s.K;
+      o[1] = s.G;
+      o[2] = s.A;
+      for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) o[3 + k] = s.E[k];
     }
-  __syncthreads();
-  if (!active) return;  // the whole warp: its lanes share the region
+    __syncthreads();
+    if (w == 0) {
+      for (int v = 1; v < W; ++v) {
+        const double* o = scratch + v * (3 + GMQ_GK_MAX_DIM);
+        s.K += o[0];
+        s.G += o[1];
+        s.A += o[2];
+        for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] += o[3 + k];
+      }
+    }
+  }
+}
+
+// f at every node.  xt: node coordinates [d][15]; xs: this lane's current
+// node, entries 32 W apart.
+template <int FAM, int W>
+__device__ __forceinline__ void gk_sums_nodes(const SmemParams<double>& P, const GkConst& K, int d,
+                                              int lane, const double* xt, double* xs, GkSums& s) {
+  constexpr int L = 32 * W;
   int rows = 1;
   for (int k = 1; k < d; ++k) rows *= 15;
-  double SK = 0.0, SG = 0.0, SA = 0.0;
-  double E[GMQ_GK_MAX_DIM];
-#pragma unroll
-  for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) E[k] = 0.0;
-  auto X = [&](int j) -> double { return xs[w][j][lane]; };
-  for (int row = lane; row < rows; row += 32) {
+  auto X = [&](int j) -> double { return xs[j * L]; };
+  for (int row = lane; row < rows; row += L) {
     // digits of axes 1..d-1, their weight products and coordinates
     int q = row;
     double wr = 1.0, gr = 1.0;
@@ -87,12 +115,12 @@ __global__ void __launch_bounds__(32 * kGkWarps) k_rule_gk(const GkArgs G) {
         q /= 15;
         wr = wr * K.wk[dig[k]];
         gr = gr * K.wg[dig[k]];
-        xs[w][k][lane] = xt[w][k * 15 + dig[k]];
+        xs[k * L] = xt[k * 15 + dig[k]];
       }
     }
     double rk = 0.0, rg = 0.0, ra = 0.0, e0 = 0.0;
     for (int j = 0; j < 15; ++j) {
-      xs[w][0][lane] = xt[w][j];
+      xs[0] = xt[j];
       const double v = Family<FAM>::template eval<double>(P, d, X);
       const double t = __dmul_rn(__dmul_rn(K.wk[j], wr), v);  // wK-product * f
       rk = __dadd_rn(rk, t);
@@ -100,38 +128,165 @@ __global__ void __launch_bounds__(32 * kGkWarps) k_rule_gk(const GkArgs G) {
       ra = fma(__dmul_rn(K.wk[j], wr), fabs(v), ra);
       e0 = fma(K.r[j], t, e0);
     }
-    SK = __dadd_rn(SK, rk);
-    SG = __dadd_rn(SG, rg);
-    SA = __dadd_rn(SA, ra);
-    E[0] = __dadd_rn(E[0], e0);
+    s.K = __dadd_rn(s.K, rk);
+    s.G = __dadd_rn(s.G, rg);
+    s.A = __dadd_rn(s.A, ra);
+    s.E[0] = __dadd_rn(s.E[0], e0);
 #pragma unroll
     for (int k = 1; k < GMQ_GK_MAX_DIM; ++k)
-      if (k < d) E[k] = fma(K.r[dig[k]], rk, E[k]);
+      if (k < d) s.E[k] = fma(K.r[dig[k]], rk, s.E[k]);
   }
-  // combine the lanes (fixed butterfly order)
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    SK += __shfl_xor_sync(0xffffffffu, SK, off);
-    SG += __shfl_xor_sync(0xffffffffu, SG, off);
-    SA += __shfl_xor_sync(0xffffffffu, SA, off);
-#pragma unroll
-    for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) E[k] += __shfl_xor_sync(0xffffffffu, E[k], off);
+}
+
+// The same from per-axis factors, relative to F.  kt, gt: wK e and wG e
+// [d][15]; rt: r wK e of axis 0 [15].
+template <int W>
+__device__ __forceinline__ void gk_sums_factors(const GkConst& K, int d, int lane,
+                                                const double* kt, const double* gt,
+                                                const double* rt, GkSums& s) {
+  constexpr int L = 32 * W;
+  int rows = 1, grows = 1;
+  for (int k = 1; k < d; ++k) {
+    rows *= 15;
+    grows *= 7;
   }
+  for (int row = lane; row < rows; row += L) {
+    int q = row;
+    double kr = 1.0;
+    int dig[GMQ_GK_MAX_DIM];
+#pragma unroll
+    for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) {
+      if (k < d) {
+        dig[k] = q % 15;
+        q /= 15;
+        const double v = kt[k * 15 + dig[k]];
+        kr = k == 1 ? v : __dmul_rn(kr, v);
+      }
+    }
+    double rk = __dmul_rn(kt[0], kr), e0 = __dmul_rn(rt[0], kr);
+#pragma unroll
+    for (int j = 1; j < 15; ++j) {
+      rk = fma(kt[j], kr, rk);
+      e0 = fma(rt[j], kr, e0);
+    }
+    s.K = __dadd_rn(s.K, rk);
+    s.E[0] = __dadd_rn(s.E[0], e0);
+#pragma unroll
+    for (int k = 1; k < GMQ_GK_MAX_DIM; ++k)
+      if (k < d) s.E[k] = fma(K.r[dig[k]], rk, s.E[k]);
+  }
+  for (int row = lane; row < grows; row += L) {
+    int q = row;
+    double gr = 1.0;
+#pragma unroll
+    for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) {
+      if (k < d) {
+        const double v = gt[k * 15 + 2 * (q % 7) + 1];
+        q /= 7;
+        gr = k == 1 ? v : __dmul_rn(gr, v);
+      }
+    }
+    double rg = __dmul_rn(gt[1], gr);
+#pragma unroll
+    for (int j = 3; j < 15; j += 2) rg = fma(gt[j], gr, rg);
+    s.G = __dadd_rn(s.G, rg);
+  }
+  s.A = s.K;
+}
+
+// W warps per region, kGkBlock / (32 W) regions per block.
+template <int FAM, int W>
+__global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
+  using SF = Sep<FAM>;
+  constexpr int L = 32 * W, RB = kGkBlock / L;
+  constexpr bool kFactors = Fac<FAM>::kind == kReal;
+  constexpr int NT = GMQ_GK_MAX_DIM * 15;
+  __shared__ GkConst K;
+  __shared__ SmemParams<double> P;
+  __shared__ double xt[RB][NT];                      // node coordinates per axis
+  __shared__ double xs[RB][GMQ_GK_MAX_DIM * L];      // each lane's current node
+  __shared__ double ft[RB][kFactors ? 2 * NT + 15 : 1];
+  __shared__ int room[RB][GMQ_GK_MAX_DIM];
+  __shared__ double scratch[W * (3 + GMQ_GK_MAX_DIM)];
+  const RuleArgs& A = G.A;
+  const int d = A.P.d;
+  const int tid = threadIdx.x, w = tid / L, lane = tid % L;
+  for (int i = tid; i < 60; i += blockDim.x) (&K.x[0])[i] = (&G.K->x[0])[i];
+  for (int j = tid; j < d; j += blockDim.x) {
+    P.a[j] = A.P.a[j];
+    P.u[j] = A.P.u[j];
+    P.b[j] = A.P.b[j];
+  }
+  if (tid == 0) P.c0 = A.P.c0;
+  if (lane < GMQ_GK_MAX_DIM) room[w][lane] = 0;
+  __syncthreads();
+  const int64_t r = (int64_t)blockIdx.x * RB + w;
+  const bool active = r < A.n;
+  double* kt = ft[w];
+  double* gt = kt + NT;
+  double* rt = gt + NT;
+  if (active)
+    for (int q = lane; q < d * 15; q += L) {
+      const int k = q / 15, j = q - 15 * k;
+      const double c = A.c[(int64_t)k * A.ld + r];
+      const double x = fma(K.x[j], A.h[(int64_t)k * A.ld + r], c);
+      xt[w][q] = x;
+      if constexpr (kFactors) {
+        double e = Fac<FAM>::e(P, k, x, SF::phi(P, k, c));
+        atomicMax(&room[w][k], exp_magnitude(e));
+        if constexpr (SF::kFlag) {
+          if (SF::flag(P, k, x)) e = 0.0;
+        }
+        const double ke = __dmul_rn(K.wk[j], e);
+        kt[q] = ke;
+        gt[q] = __dmul_rn(K.wg[j], e);
+        if (k == 0) rt[j] = __dmul_rn(K.r[j], ke);
+      }
+    }
+  __syncthreads();
+  if (!active) return;  // the whole warp (W = 1): its lanes share the region
+  GkSums s;
+#pragma unroll
+  for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] = 0.0;
+  double F = 1.0;
+  bool factors = false;
+  if constexpr (kFactors) {
+    double S = 0.0;
+    int big = 0;
+    for (int k = 0; k < d; ++k) {
+      const double fc = SF::phi(P, k, A.c[(int64_t)k * A.ld + r]);
+      S = k ? (SF::kMul ? __dmul_rn(S, fc) : __dadd_rn(S, fc)) : fc;
+      big += room[w][k];
+    }
+    F = SF::g(d, S);
+    factors = big <= kFacExpRoom && exp_magnitude(F) <= kFacExpRoom;
+    if (factors)
+      gk_sums_factors<W>(K, d, lane, kt, gt, rt, s);
+    else
+      F = 1.0;
+  }
+  if (!factors) gk_sums_nodes<FAM, W>(P, K, d, lane, xt[w], xs[w] + lane, s);
+  gk_combine<W>(s, scratch);
   if (lane != 0) return;
+  s.K = __dmul_rn(F, s.K);
+  s.G = __dmul_rn(F, s.G);
+  s.A = __dmul_rn(F, s.A);
+#pragma unroll
+  for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] = __dmul_rn(F, s.E[k]);
   double hprod = 1.0, vol = 1.0;
   for (int k = 0; k < d; ++k) {
     const double hk = A.h[(int64_t)k * A.ld + r];
     hprod = __dmul_rn(hprod, hk);
     vol = __dmul_rn(vol, __dmul_rn(2.0, hk));
   }
-  const double ik = __dmul_rn(hprod, SK), ig = __dmul_rn(hprod, SG);
-  const double scale = __dmul_rn(hprod, SA);
+  const double ik = __dmul_rn(hprod, s.K), ig = __dmul_rn(hprod, s.G);
+  const double scale = __dmul_rn(hprod, s.A);
   int best = 0;
-  double eb = __dmul_rn(hprod, fabs(E[0]));
+  double eb = __dmul_rn(hprod, fabs(s.E[0]));
 #pragma unroll
   for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) {
     if (k < d) {
-      const double ek = __dmul_rn(hprod, fabs(E[k]));
+      const double ek = __dmul_rn(hprod, fabs(s.E[k]));
       if (ek > eb) {
         eb = ek;
         best = k;
@@ -159,12 +314,20 @@ __global__ void __launch_bounds__(32 * kGkWarps) k_rule_gk(const GkArgs G) {
   A.axis[r] = (uint8_t)(ax | (bad ? 0x80 : 0));
 }
 
+template <int FAM, int W>
+cudaError_t launch_rule_gk_warps(const GkArgs& G, cudaStream_t s) {
+  constexpr int RB = kGkBlock / (32 * W);
+  const int64_t blocks = (G.A.n + RB - 1) / RB;
+  if (blocks == 0) return cudaSuccess;
+  k_rule_gk<FAM, W><<<(unsigned)blocks, kGkBlock, 0, s>>>(G);
+  return cudaGetLastError();
+}
+
+// A block per region from d = 4 on: 3375 rows are 27 turns of 128 lanes (225
+// rows of d = 3 would leave the last of two turns 3/4 empty).
 template <int FAM>
 cudaError_t launch_rule_gk_family(const GkArgs& G, cudaStream_t s) {
-  const int64_t blocks = (G.A.n + kGkWarps - 1) / kGkWarps;
-  if (blocks == 0) return cudaSuccess;
-  k_rule_gk<FAM><<<(unsigned)blocks, 32 * kGkWarps, 0, s>>>(G);
-  return cudaGetLastError();
+  return G.A.P.d >= 4 ? launch_rule_gk_warps<FAM, 4>(G, s) : launch_rule_gk_warps<FAM, 1>(G, s);
 }
 
 #define GMQ_DEFINE_GK_FAMILY(FAMV) \

@@ -58,3 +58,43 @@ def test_factors_without_exponent_room(oracle, gpu_ctx, fam, scale, d):
     # the whole domain as well: the widest spread of factors
     c, h = np.concatenate([c, np.full((1, d), 0.5)]), np.concatenate([h, np.full((1, d), 0.5)])
     _check(oracle, gpu_ctx, fam, a, u, c, h, 3e-12)
+
+
+@pytest.mark.parametrize("fam,scale", [(G.GAUSSIAN, 1.0), (G.GAUSSIAN, 60.0), (G.C0, 1.0),
+                                       (G.C0, 300.0), (G.DISCONTINUOUS, 1.0),
+                                       (G.PRODUCT_PEAK, 1.0)])
+@pytest.mark.parametrize("d,n", [(1, 5), (2, 33), (3, 6), (4, 3), (5, 1)])
+def test_gauss_kronrod_factors(oracle, gpu_ctx, fam, scale, d, n):
+    """The Gauss-Kronrod rule from per-axis factors: a warp per region up to
+    d = 3, a block from d = 4, with and without exponent room."""
+    a, u = G.seed_uniform(17 + d, fam, d, 0.5 * scale, 3.0 * scale)
+    if fam == G.DISCONTINUOUS:
+        u = 0.4 + 0.6 * u
+    c, h = G.random_boxes(800 + d, n, d)
+    c, h = np.concatenate([c, np.full((1, d), 0.5)]), np.concatenate([h, np.full((1, d), 0.5)])
+    ref = oracle.rule_gk_regions(fam, a, u, c, h)
+    ik, err, vf, ax = (x.cpu().numpy() for x in gpu_ctx.eval_rule_gk(fam, a, u, _soa(c), _soa(h)))
+    assert np.all(np.abs(ik - ref["ik"]) <= 1e-12 * ref["scale"] + 1e-300)
+    assert np.all(np.abs(err - ref["err"]) <= 1e-12 * ref["scale"] + 1e-300)
+    clear = ~ref["axis_tie"].astype(bool)
+    assert np.array_equal((ax.astype(np.int32) & 0x7F)[clear], ref["axis"][clear])
+
+
+@pytest.mark.parametrize("fam,scale", [(G.GAUSSIAN, 1.0), (G.GAUSSIAN, 60.0), (G.C0, 1.0),
+                                       (G.C0, 300.0), (G.DISCONTINUOUS, 1.0),
+                                       (G.PRODUCT_PEAK, 1.0)])
+@pytest.mark.parametrize("d,n", [(1, 65), (2, 64), (3, 63), (8, 9), (9, 7)])
+def test_adjoint_factors(oracle, gpu_ctx, fam, scale, d, n):
+    """gmq_rule_grad from per-axis factors, with and without exponent room: the
+    bounds of the adjoint tests (1e-12 of the largest component), and three of
+    them for steep parameters, as above."""
+    a, u = G.seed_uniform(19 + d, fam, d, 0.5 * scale, 3.0 * scale)
+    if fam == G.DISCONTINUOUS:
+        u = 0.4 + 0.6 * u
+    c, h = G.random_boxes(900 + d, n, d)
+    go, qo = oracle.rule_grad(fam, a, u, c, h)
+    g, q = gpu_ctx.rule_grad(fam, a, u, _soa(c), _soa(h))
+    scale_g = np.max(np.abs(go)) + abs(qo)
+    bound = 1e-12 if scale == 1.0 else 3e-12
+    assert abs(q - qo) <= bound * scale_g
+    assert np.all(np.abs(np.asarray(g) - go) <= bound * scale_g)
