@@ -7,13 +7,16 @@
 // (a_1..a_d, u_1..u_d) is the same rule applied to df/dtheta:
 //   dQ/dtheta_k = sum_r vol_r sum_i w_i df/dtheta_k(x_i).
 // k_rule_grad_sep (the default) forms the gradient from per-axis, per-row
-// sums of w_i g'(S_i) over the separable form; k_rule_grad
+// sums of w_i g'(S_i), with the node values as products of per-axis factors
+// where the integrand has them and over the separable form otherwise;
+// k_rule_grad
 // (GMQ_EVAL_NODEWISE) evaluates f and its 2d parameter derivatives at every
 // node from a node-coordinate table.  Both run a thread per region, write
 // the region's contributions (and its I7) to a [2d+1][n] array, and the
 // per-row pairwise-tree sums give Q and its gradient.
 #pragma once
 
+#include "gm_factor64.cuh"
 #include "gm_rule.cuh"
 
 namespace gmq {
@@ -291,27 +294,236 @@ inline size_t grad_sep_smem_bytes(int d, bool flag) {
          sizeof(SmemParams<double>) + 16;
 }
 
+// Integrands that are products of per-axis factors (kReal of
+// gm_factor64.cuh): D = +-f, so with F = f(centre) every node adds one product
+// of factors to each sum it belongs to -- two fused multiply-adds a node
+// where the separable form evaluates f and adds it four times -- and the sign,
+// F and the rule's weights multiply the sums at the end.  Bound by the FP64
+// pipe; four d = 6 Gaussian rows to 1e-7 with their gradients, forward pass
+// included: 17.4 -> 9.0 ms (of it the forward pass 1.44x).
 template <int FAM>
-__global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs A) {
+constexpr double grad_factor_sign() {
+  return FAM == GMQ_GAUSSIAN || FAM == GMQ_C0 ? -1.0 : 1.0;
+}
+
+// The gradient from the per-axis, per-row sums of a region: row(j, Hr) fills
+// the seven sums of axis j; hall: the sum over all nodes.
+template <int FAM, class CH, class Row>
+__device__ __forceinline__ void grad_rows(const GradArgs& A, const SmemParams<double>& P, int64_t r,
+                                          double vol, const CH& ch, double hall, const Row& rows) {
+  const int d = A.P.d;
+  const double lam2 = A.R.lam2, lam3 = A.R.lam3, lam5 = A.R.lam5;
+  for (int j = 0; j < d; ++j) {
+    double c, h;
+    ch(j, c, h);
+    double Hr[7];
+    rows(j, Hr);
+    double ga = 0.0, gu = 0.0;
+#pragma unroll
+    for (int row = 0; row < 7; ++row) {
+      const double lam = row == kXC ? 0.0
+                         : row == kXP2 ? lam2 : row == kXM2 ? -lam2
+                         : row == kXP3 ? lam3 : row == kXM3 ? -lam3
+                         : row == kXP5 ? lam5 : -lam5;
+      const double x = row == kXC ? c : fma(lam, h, c);
+      double ca, cu;
+      SepGrad<FAM>::coef(P, j, x, ca, cu);
+      ga = fma(Hr[row], ca, ga);
+      gu = fma(Hr[row], cu, gu);
+    }
+    if constexpr (FAM == GMQ_OSCILLATORY) {
+      // base 2 pi u_1: dS/du_1 = 2 pi at every node
+      if (j == 0) gu = fma(2.0 * M_PI, hall, gu);
+    }
+    A.out[(int64_t)j * A.ldo + r] = __dmul_rn(vol, ga);
+    A.out[(int64_t)(d + j) * A.ldo + r] = __dmul_rn(vol, gu);
+  }
+}
+
+// One region from factors; false (and nothing written to A.out): the factors
+// lack exponent room.
+template <int FAM>
+__device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const SmemParams<double>& P,
+                                                    double* w, int64_t r) {
+  using SF = Sep<FAM>;
+  using FF = Fac<FAM>;
+  const int d = A.P.d;
+  const int pa = sep_a(d), pb = sep_b(d), pc = sep_c(d);
+  const int nlo = 1 << pa, nb = pb ? 1 << pb : 0, nc = pc ? 1 << pc : 0;
+  // per-region entries: factors of lambda2, lambda3 [2d each], class-5 chains,
+  // pair sums per axis and sign [2d], sign-pattern sums per part
+  const int e2 = 0, e3 = 2 * d, eA = 4 * d, eB = eA + nlo, eC = eB + nb, eG = eC + nc;
+  const int eTL = eG + 2 * d, eTB = eTL + nlo, eTC = eTB + nb;
+  auto W = [&](int e) -> double& { return w[(long long)e * kGradSepBlock]; };
+  const double* C = A.c + r;
+  const double* H = A.h + r;
+  auto ch = [&](int k, double& c, double& h) {
+    c = C[(int64_t)k * A.ld];
+    h = H[(int64_t)k * A.ld];
+  };
+  const double lam2 = A.R.lam2, lam3 = A.R.lam3, lam5 = A.R.lam5;
+  unsigned zc = 0u, z5 = 0u;
+  if constexpr (SF::kFlag) {
+    for (int k = 0; k < d; ++k) {
+      double c, h;
+      ch(k, c, h);
+      zc |= (unsigned)SF::flag(P, k, c) << k;
+    }
+  }
+  double S = 0.0, s2 = 0.0, s3 = 0.0, vol = 1.0;
+  int room = 0;
+  for (int k = 0; k < d; ++k) {
+    double c, h;
+    ch(k, c, h);
+    vol = __dmul_rn(vol, __dmul_rn(2.0, h));
+    const double fc = SF::phi(P, k, c);
+    S = k ? (SF::kMul ? __dmul_rn(S, fc) : __dadd_rn(S, fc)) : fc;
+    const double x2p = fma(lam2, h, c), x2m = fma(-lam2, h, c);
+    const double x3p = fma(lam3, h, c), x3m = fma(-lam3, h, c);
+    const double x5p = fma(lam5, h, c), x5m = fma(-lam5, h, c);
+    double p2 = FF::e(P, k, x2p, fc), m2 = FF::e(P, k, x2m, fc);
+    double p3 = FF::e(P, k, x3p, fc), m3 = FF::e(P, k, x3m, fc);
+    const double p5 = FF::e(P, k, x5p, fc), m5 = FF::e(P, k, x5m, fc);
+    room += max(max(exp_magnitude(p2), exp_magnitude(m2)),
+                max(max(exp_magnitude(p3), exp_magnitude(m3)),
+                    max(exp_magnitude(p5), exp_magnitude(m5))));
+    if constexpr (SF::kFlag) {
+      z5 |= ((unsigned)SF::flag(P, k, x5p) << k) | ((unsigned)SF::flag(P, k, x5m) << (k + 16));
+      if (SF::flag(P, k, x3p)) p3 = 0.0;
+      if (SF::flag(P, k, x3m)) m3 = 0.0;
+    }
+    W(e3 + 2 * k) = p3;
+    W(e3 + 2 * k + 1) = m3;
+    if constexpr (SF::kFlag) {  // an axis node is 0 with any other axis' centre flagged
+      const bool off = (zc & ~(1u << k)) != 0u;
+      if (off || SF::flag(P, k, x2p)) p2 = 0.0;
+      if (off || SF::flag(P, k, x2m)) m2 = 0.0;
+      if (off) p3 = m3 = 0.0;
+    }
+    W(e2 + 2 * k) = p2;
+    W(e2 + 2 * k + 1) = m2;
+    s2 = __dadd_rn(s2, __dadd_rn(p2, m2));
+    s3 = __dadd_rn(s3, __dadd_rn(p3, m3));
+    W(eG + 2 * k) = 0.0;
+    W(eG + 2 * k + 1) = 0.0;
+    const int e0 = k < pa ? eA : (k < pa + pb ? eB : eC);
+    const int i = k < pa ? k : (k < pa + pb ? k - pa : k - pa - pb);
+    if (i == 0) {
+      W(e0) = p5;
+      W(e0 + 1) = m5;
+    } else {
+      const int n = 1 << i;
+      for (int t = 0; t < n; ++t) {
+        const double v = W(e0 + t);
+        W(e0 + t + n) = __dmul_rn(v, m5);
+        W(e0 + t) = __dmul_rn(v, p5);
+      }
+    }
+  }
+  const double F = SF::g(d, S);
+  if (room > kFacExpRoom || exp_magnitude(F) > kFacExpRoom) return false;
+  // class 4: each node to its two axis slots
+  double s4 = 0.0;
+  for (int j = 0; j < d - 1; ++j) {
+    const double j0 = W(e3 + 2 * j), j1 = W(e3 + 2 * j + 1);
+    double g0 = 0.0, g1 = 0.0;
+    for (int k = j + 1; k < d; ++k) {
+      if constexpr (SF::kFlag) {
+        if (zc & ~((1u << j) | (1u << k))) continue;
+      }
+      const double k0 = W(e3 + 2 * k), k1 = W(e3 + 2 * k + 1);
+      g0 = fma(j0, k1, fma(j0, k0, g0));
+      g1 = fma(j1, k1, fma(j1, k0, g1));
+      W(eG + 2 * k) = fma(j1, k0, fma(j0, k0, W(eG + 2 * k)));
+      W(eG + 2 * k + 1) = fma(j1, k1, fma(j0, k1, W(eG + 2 * k + 1)));
+    }
+    W(eG + 2 * j) = __dadd_rn(W(eG + 2 * j), g0);
+    W(eG + 2 * j + 1) = __dadd_rn(W(eG + 2 * j + 1), g1);
+    s4 = __dadd_rn(s4, __dadd_rn(g0, g1));
+  }
+  // class 5: pattern m = lo + 2^a q to the sums of its parts; four entries of
+  // A and their sums in registers while q runs
+  for (int t = 0; t < nb; ++t) W(eTB + t) = 0.0;
+  for (int t = 0; t < nc; ++t) W(eTC + t) = 0.0;
+  const unsigned dmask = (1u << d) - 1u;
+  const int nq = 1 << (d - pa);
+  double s5 = 0.0;
+  for (int lo = 0; lo < nlo; lo += 4) {
+    double a[4], t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = lo + i < nlo ? W(eA + lo + i) : 0.0;
+      t[i] = 0.0;
+    }
+    for (int q = 0; q < nq; ++q) {
+      double bc = 1.0;
+      if (pb) bc = W(eB + (q & (nb - 1)));
+      if (pc) bc = __dmul_rn(bc, W(eC + (q >> pb)));
+      double U = 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        double v = a[i];
+        if constexpr (SF::kFlag) {
+          const unsigned m = (unsigned)(lo + i) | ((unsigned)q << pa);
+          if (((((~m) & z5) | (m & (z5 >> 16))) & dmask) != 0u) v = 0.0;
+        }
+        t[i] = fma(v, bc, t[i]);
+        U = fma(v, bc, U);
+      }
+      if (pb) W(eTB + (q & (nb - 1))) = __dadd_rn(W(eTB + (q & (nb - 1))), U);
+      if (pc) W(eTC + (q >> pb)) = __dadd_rn(W(eTC + (q >> pb)), U);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (lo + i < nlo) {
+        W(eTL + lo + i) = t[i];
+        s5 = __dadd_rn(s5, t[i]);
+      }
+  }
+  const double* w7 = A.R.w7;
+  const double f0 = SF::kFlag && zc ? 0.0 : 1.0;
+  const double hC = __dmul_rn(w7[0], f0);
+  const double T23 = fma(w7[1], s2, __dmul_rn(w7[2], s3));
+  const double T4 = __dmul_rn(w7[3], s4), T5 = __dmul_rn(w7[4], s5);
+  const double vF = __dmul_rn(vol, F);
+  const double all = __dadd_rn(__dadd_rn(hC, T23), __dadd_rn(T4, T5));
+  grad_rows<FAM>(A, P, r, __dmul_rn(grad_factor_sign<FAM>(), vF), ch, all,
+                 [&](int j, double* Hr) {
+    // sum over the sign patterns with bit j set (-lambda5 on axis j)
+    const int e0 = j < pa ? eTL : (j < pa + pb ? eTB : eTC);
+    const int n = j < pa ? nlo : (j < pa + pb ? nb : nc);
+    const int i = j < pa ? j : (j < pa + pb ? j - pa : j - pa - pb);
+    double hm5 = 0.0;
+    for (int t = 0; t < n; ++t)
+      if ((t >> i) & 1) hm5 = __dadd_rn(hm5, W(e0 + t));
+    hm5 = __dmul_rn(w7[4], hm5);
+    double p3 = W(e3 + 2 * j), m3 = W(e3 + 2 * j + 1);
+    if constexpr (SF::kFlag) {
+      if (zc & ~(1u << j)) p3 = m3 = 0.0;
+    }
+    Hr[kXP2] = __dmul_rn(w7[1], W(e2 + 2 * j));
+    Hr[kXM2] = __dmul_rn(w7[1], W(e2 + 2 * j + 1));
+    Hr[kXP3] = fma(w7[3], W(eG + 2 * j), __dmul_rn(w7[2], p3));
+    Hr[kXM3] = fma(w7[3], W(eG + 2 * j + 1), __dmul_rn(w7[2], m3));
+    Hr[kXP5] = __dsub_rn(T5, hm5);
+    Hr[kXM5] = hm5;
+    // the centre row: the classes 1 to 4 that leave axis j alone
+    Hr[kXC] = __dsub_rn(__dadd_rn(hC, __dadd_rn(T23, T4)),
+                        __dadd_rn(__dadd_rn(Hr[kXP2], Hr[kXM2]), __dadd_rn(Hr[kXP3], Hr[kXM3])));
+  });
+  A.out[(int64_t)(2 * d) * A.ldo + r] = __dmul_rn(vF, all);
+  return true;
+}
+
+// One region over the separable form.
+template <int FAM>
+__device__ __forceinline__ void grad_region_sep(const GradArgs& A, const SmemParams<double>& P,
+                                                double* w, int64_t r) {
   using SF = Sep<FAM>;
   using SG = SepGrad<FAM>;
   constexpr int RB = kGradSepBlock;
-  extern __shared__ __align__(16) double smem[];
   const int d = A.P.d;
   const SepLayout Ly = sep_layout(d, SF::kFlag, false);
-  const int words = grad_sep_words(d, SF::kFlag);
-  SmemParams<double>* P = reinterpret_cast<SmemParams<double>*>(smem + (size_t)words * RB);
-  const int tid = threadIdx.x;
-  for (int j = tid; j < d; j += RB) {
-    P->a[j] = A.P.a[j];
-    P->u[j] = A.P.u[j];
-    P->b[j] = A.P.b[j];
-  }
-  if (tid == 0) P->c0 = A.P.c0;
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * RB + tid;
-  if (r >= A.n) return;
-  double* w = smem + tid;
   auto W = [&](int e) -> double& { return w[(long long)e * RB]; };
   const int eHA = Ly.words, eG4 = eHA + 4 * d, eTL = eG4 + 2 * d;
   const int pa = sep_a(d), pb = sep_b(d), pc = sep_c(d);
@@ -349,10 +561,10 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
     double c, h;
     ch(k, c, h);
     const double xp = fma(lam3, h, c), xm = fma(-lam3, h, c);
-    const double fc = SF::phi(*P, k, c), fp = SF::phi(*P, k, xp), fm = SF::phi(*P, k, xm);
+    const double fc = SF::phi(P, k, c), fp = SF::phi(P, k, xp), fm = SF::phi(P, k, xm);
     if constexpr (SF::kFlag) {
-      zc |= (unsigned)SF::flag(*P, k, c) << k;
-      z3 |= ((unsigned)SF::flag(*P, k, xp) << k) | ((unsigned)SF::flag(*P, k, xm) << (k + 16));
+      zc |= (unsigned)SF::flag(P, k, c) << k;
+      z3 |= ((unsigned)SF::flag(P, k, xp) << k) | ((unsigned)SF::flag(P, k, xm) << (k + 16));
     }
     W(Ly.phiC + k) = fc;
     if (k == d - 1) {
@@ -370,12 +582,12 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
   double hC, T23 = 0.0, T4 = 0.0, T5 = 0.0;          // sums of w D
   {
     double f, D;
-    node(SF::kBase ? op(SF::base(*P), suf) : suf, zc != 0u, f, D);
+    node(SF::kBase ? op(SF::base(P), suf) : suf, zc != 0u, f, D);
     s1 = f;
     hC = __dmul_rn(w7[0], D);
   }
   // left to right: the axis nodes and the pair-node prefixes L
-  double pre = SF::kBase ? SF::base(*P) : 0.0;
+  double pre = SF::kBase ? SF::base(P) : 0.0;
   bool hp = SF::kBase;
   for (int k = 0; k < d; ++k) {
     double c, h;
@@ -386,11 +598,11 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
     for (int rr = 0; rr < 4; ++rr) {
       const double lam = rr < 2 ? (rr ? -lam2 : lam2) : (rr == 2 ? lam3 : -lam3);
       const double x = fma(lam, h, c);
-      const double ph = SF::phi(*P, k, x);
+      const double ph = SF::phi(P, k, x);
       const double lp = hp ? op(pre, ph) : ph;
       if (rr >= 2) W(Ly.L + 2 * k + (rr - 2)) = lp;
       bool zero = false;
-      if constexpr (SF::kFlag) zero = ((zc & ~(1u << k)) != 0u) || SF::flag(*P, k, x);
+      if constexpr (SF::kFlag) zero = ((zc & ~(1u << k)) != 0u) || SF::flag(P, k, x);
       double f, D;
       node(hs ? op(lp, sk) : lp, zero, f, D);
       const double hw = __dmul_rn(w7[rr < 2 ? 1 : 2], D);
@@ -413,13 +625,13 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
       double c, h;
       ch(j0 + i, c, h);
       const double xp = fma(lam5, h, c), xm = fma(-lam5, h, c);
-      const double fp = SF::phi(*P, j0 + i, xp), fm = SF::phi(*P, j0 + i, xm);
+      const double fp = SF::phi(P, j0 + i, xp), fm = SF::phi(P, j0 + i, xm);
       if constexpr (SF::kFlag)
-        z5 |= ((unsigned)SF::flag(*P, j0 + i, xp) << (j0 + i)) |
-              ((unsigned)SF::flag(*P, j0 + i, xm) << (j0 + i + 16));
+        z5 |= ((unsigned)SF::flag(P, j0 + i, xp) << (j0 + i)) |
+              ((unsigned)SF::flag(P, j0 + i, xm) << (j0 + i + 16));
       if (i == 0) {
-        W(e0) = with_base ? op(SF::base(*P), fp) : fp;
-        W(e0 + 1) = with_base ? op(SF::base(*P), fm) : fm;
+        W(e0) = with_base ? op(SF::base(P), fp) : fp;
+        W(e0 + 1) = with_base ? op(SF::base(P), fm) : fm;
       } else {
         const int n = 1 << i;
         for (int t = 0; t < n; ++t) {
@@ -509,9 +721,8 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
     ch(k, c, h);
     vol = __dmul_rn(vol, __dmul_rn(2.0, h));
   }
-  for (int j = 0; j < d; ++j) {
-    double c, h;
-    ch(j, c, h);
+  grad_rows<FAM>(A, P, r, vol, ch, __dadd_rn(__dadd_rn(hC, T23), __dadd_rn(T4, T5)),
+                 [&](int j, double* Hr) {
     // sum of w D over the sign patterns with bit j set (-lambda5 on axis j)
     double hm5 = 0.0;
     if (j < pa) {
@@ -527,7 +738,6 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
     const double a0 = W(eHA + 4 * j), a1 = W(eHA + 4 * j + 1);
     const double a2 = W(eHA + 4 * j + 2), a3 = W(eHA + 4 * j + 3);
     const double g0 = W(eG4 + 2 * j), g1 = W(eG4 + 2 * j + 1);
-    double Hr[7];
     Hr[kXC] = __dadd_rn(__dadd_rn(hC, __dsub_rn(T23, __dadd_rn(__dadd_rn(a0, a1),
                                                                  __dadd_rn(a2, a3)))),
                         __dsub_rn(T4, __dadd_rn(g0, g1)));
@@ -537,33 +747,36 @@ __global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs 
     Hr[kXM3] = __dadd_rn(a3, g1);
     Hr[kXP5] = __dsub_rn(T5, hm5);
     Hr[kXM5] = hm5;
-    double ga = 0.0, gu = 0.0;
-#pragma unroll
-    for (int row = 0; row < 7; ++row) {
-      const double lam = row == kXC ? 0.0
-                         : row == kXP2 ? lam2 : row == kXM2 ? -lam2
-                         : row == kXP3 ? lam3 : row == kXM3 ? -lam3
-                         : row == kXP5 ? lam5 : -lam5;
-      const double x = row == kXC ? c : fma(lam, h, c);
-      double ca, cu;
-      SG::coef(*P, j, x, ca, cu);
-      ga = fma(Hr[row], ca, ga);
-      gu = fma(Hr[row], cu, gu);
-    }
-    if constexpr (FAM == GMQ_OSCILLATORY) {
-      // base 2 pi u_1: dS/du_1 = 2 pi at every node
-      if (j == 0)
-        gu = fma(2.0 * M_PI, __dadd_rn(__dadd_rn(hC, T23), __dadd_rn(T4, T5)), gu);
-    }
-    A.out[(int64_t)j * A.ldo + r] = __dmul_rn(vol, ga);
-    A.out[(int64_t)(d + j) * A.ldo + r] = __dmul_rn(vol, gu);
-  }
+  });
   double t7 = __dmul_rn(w7[0], s1);
   t7 = fma(w7[1], s2, t7);
   t7 = fma(w7[2], s3, t7);
   t7 = fma(w7[3], s4, t7);
   t7 = fma(w7[4], s5, t7);
   A.out[(int64_t)(2 * d) * A.ldo + r] = __dmul_rn(vol, t7);
+}
+
+template <int FAM>
+__global__ void __launch_bounds__(kGradSepBlock) k_rule_grad_sep(const GradArgs A) {
+  constexpr int RB = kGradSepBlock;
+  extern __shared__ __align__(16) double smem[];
+  const int d = A.P.d;
+  const int words = grad_sep_words(d, Sep<FAM>::kFlag);
+  SmemParams<double>* P = reinterpret_cast<SmemParams<double>*>(smem + (size_t)words * RB);
+  const int tid = threadIdx.x;
+  for (int j = tid; j < d; j += RB) {
+    P->a[j] = A.P.a[j];
+    P->u[j] = A.P.u[j];
+    P->b[j] = A.P.b[j];
+  }
+  if (tid == 0) P->c0 = A.P.c0;
+  __syncthreads();
+  const int64_t r = (int64_t)blockIdx.x * RB + tid;
+  if (r >= A.n) return;
+  if constexpr (Fac<FAM>::kind == kReal) {
+    if (grad_region_factors<FAM>(A, *P, smem + tid, r)) return;
+  }
+  grad_region_sep<FAM>(A, *P, smem + tid, r);
 }
 
 template <int FAM>
