@@ -111,11 +111,12 @@ RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
 # fingerprint is RULE_COUNTS_SHA16; when those sources change the counts must
 # be taken again (tests/test_bench_counts.py fails until they are), and until
 # then the roofline reports no fraction.
-RULE_EXEC_FP64_INST_D8 = {0: 1779.0, 1: 1063.0, 2: 241.0, 3: 1219.0, 4: 1163.0}
-RULE_EXEC_FP64_FLOPS_D8 = {0: 2992.0, 1: 1649.0, 2: 231.0, 3: 1895.0, 4: 1839.0}
-RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_region64.cuh",
-                       "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "09ed4e24fb774ec5"
+RULE_EXEC_FP64_INST_D8 = {0: 476.0, 1: 533.0, 2: 241.0, 3: 424.0, 4: 328.0}
+RULE_EXEC_FP64_FLOPS_D8 = {0: 665.0, 1: 802.0, 2: 231.0, 3: 497.0, 4: 433.0}
+RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
+                       "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
+                       "gmq_common.cuh")
+RULE_COUNTS_SHA16 = "d52de4cfdf21e372"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -129,7 +130,7 @@ RULE_COUNTS_SHA16 = "09ed4e24fb774ec5"
 MIXED_FP32_OPS_D12 = {2: 116237.0, 3: 134179.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "8ec0e6ec17be2d1d"
+MIXED_COUNTS_SHA16 = "8fbdf1b590534d87"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):

@@ -370,34 +370,33 @@ __device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const Sme
       zc |= (unsigned)SF::flag(P, k, c) << k;
     }
   }
-  double S = 0.0, s2 = 0.0, s3 = 0.0, vol = 1.0;
+  Centre<FAM> top;
+  double s2 = 0.0, s3 = 0.0, vol = 1.0;
   int room = 0;
   for (int k = 0; k < d; ++k) {
     double c, h;
     ch(k, c, h);
     vol = __dmul_rn(vol, __dmul_rn(2.0, h));
     const double fc = SF::phi(P, k, c);
-    S = k ? (SF::kMul ? __dmul_rn(S, fc) : __dadd_rn(S, fc)) : fc;
-    const double x2p = fma(lam2, h, c), x2m = fma(-lam2, h, c);
-    const double x3p = fma(lam3, h, c), x3m = fma(-lam3, h, c);
-    const double x5p = fma(lam5, h, c), x5m = fma(-lam5, h, c);
-    double p2 = FF::e(P, k, x2p, fc), m2 = FF::e(P, k, x2m, fc);
-    double p3 = FF::e(P, k, x3p, fc), m3 = FF::e(P, k, x3m, fc);
-    const double p5 = FF::e(P, k, x5p, fc), m5 = FF::e(P, k, x5m, fc);
+    top.add(P, k, c, fc);
+    double p2 = FF::e(P, k, c, h, fc, lam2), m2 = FF::e(P, k, c, h, fc, -lam2);
+    double p3 = FF::e(P, k, c, h, fc, lam3), m3 = FF::e(P, k, c, h, fc, -lam3);
+    const double p5 = FF::e(P, k, c, h, fc, lam5), m5 = FF::e(P, k, c, h, fc, -lam5);
     room += max(max(exp_magnitude(p2), exp_magnitude(m2)),
                 max(max(exp_magnitude(p3), exp_magnitude(m3)),
                     max(exp_magnitude(p5), exp_magnitude(m5))));
     if constexpr (SF::kFlag) {
-      z5 |= ((unsigned)SF::flag(P, k, x5p) << k) | ((unsigned)SF::flag(P, k, x5m) << (k + 16));
-      if (SF::flag(P, k, x3p)) p3 = 0.0;
-      if (SF::flag(P, k, x3m)) m3 = 0.0;
+      z5 |= ((unsigned)SF::flag(P, k, fma(lam5, h, c)) << k) |
+            ((unsigned)SF::flag(P, k, fma(-lam5, h, c)) << (k + 16));
+      if (SF::flag(P, k, fma(lam3, h, c))) p3 = 0.0;
+      if (SF::flag(P, k, fma(-lam3, h, c))) m3 = 0.0;
     }
     W(e3 + 2 * k) = p3;
     W(e3 + 2 * k + 1) = m3;
     if constexpr (SF::kFlag) {  // an axis node is 0 with any other axis' centre flagged
       const bool off = (zc & ~(1u << k)) != 0u;
-      if (off || SF::flag(P, k, x2p)) p2 = 0.0;
-      if (off || SF::flag(P, k, x2m)) m2 = 0.0;
+      if (off || SF::flag(P, k, fma(lam2, h, c))) p2 = 0.0;
+      if (off || SF::flag(P, k, fma(-lam2, h, c))) m2 = 0.0;
       if (off) p3 = m3 = 0.0;
     }
     W(e2 + 2 * k) = p2;
@@ -420,7 +419,7 @@ __device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const Sme
       }
     }
   }
-  const double F = SF::g(d, S);
+  const double F = top.value(d);
   if (room > kFacExpRoom || exp_magnitude(F) > kFacExpRoom) return false;
   // class 4: each node to its two axis slots
   double s4 = 0.0;

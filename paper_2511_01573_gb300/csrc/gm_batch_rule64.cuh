@@ -37,6 +37,10 @@ size_t batch_rule_smem(int dmax) {
   return (sizeof(double) * (size_t)batch_rule_doubles_max<FAM>(dmax) + pairs + 15) & ~(size_t)15;
 }
 
+// Dynamic shared memory from which a launch opts in: the 48 KB that need no
+// opt-in hold the kernel's static arrays (at most 4 KB) too.
+constexpr size_t kBatchOptInSmem = 44 * 1024;
+
 template <int FAM, int T>
 __device__ __forceinline__ void batch_rule64_lanes(const BatchArgs& B, double* smem,
                                                    const unsigned short* pairs_all) {
@@ -108,7 +112,7 @@ __global__ void __launch_bounds__(kBatchRuleBlock) k_batch_rule64(const BatchArg
 template <int FAM>
 cudaError_t batch_launch_rule64_family(const BatchArgs& B, int grid, cudaStream_t s) {
   const size_t smem = batch_rule_smem<FAM>(B.dmax);
-  if (smem > 48 * 1024) {
+  if (smem > kBatchOptInSmem) {
     cudaError_t e = cudaFuncSetAttribute(k_batch_rule64<FAM>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -121,7 +125,7 @@ template <int FAM>
 int batch_rule64_max_blocks_family(int dmax) {
   int nb = 0;
   const size_t smem = batch_rule_smem<FAM>(dmax);
-  if (smem > 48 * 1024)
+  if (smem > kBatchOptInSmem)
     cudaFuncSetAttribute(k_batch_rule64<FAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_rule64<FAM>, kBatchRuleBlock,

@@ -8,32 +8,38 @@
 // design counts FP64 instructions.  With S = S_0 + Delta_j (+ Delta_k) an
 // exponential node is f = F e_j (e_k): F = f(centre), e = exp(-Delta) one of
 // six factors per axis (c +- lambda h for three generators), formed once per
-// region, and every node's value is one product that the accumulating fused
-// multiply-add forms on the way: 401 nodes at d = 8 cost 368 fused
-// multiply-adds and 48 exponentials instead of 401 exponentials, 401 chain
-// steps and 401 adds.  The product peak's factors are ratios of its
-// per-axis denominators (a reciprocal each); the cosine's are rotations
-// (cos Delta, sin Delta), two fused multiply-adds per node.  Measured at d = 8,
-// 2^20 regions, one thread per region: C0 8.14 -> 2.23 ms (4080 -> 1163 FP64
-// instructions a region), Gaussian 8.25 -> 2.34, product peak 4.71 -> 2.00,
-// cosine 10.99 -> 3.31 ms, the FP64 pipe 88-91 % active.
+// region, and every node's value is one product, formed and added in one go:
+// 401 nodes at d = 8 cost 368 products and 49 exponentials instead of 401
+// exponentials, 401 chain steps and 401 adds.  The product peak's factors are
+// ratios of its per-axis denominators (a reciprocal each); the cosine's are
+// rotations (cos Delta, sin Delta), two products per node.  Exponentials, sines
+// and class sums run in fixed point on the integer pipes (gmq_families.cuh,
+// Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
+// the outer function at every node: C0 8.14 -> 1.00 ms (4080 -> 328 FP64
+// instructions a region), Gaussian 8.25 -> 1.14, product peak 4.71 -> 1.21,
+// cosine 10.99 -> 1.95; with factors and FP64 sums and functions they took 2.23,
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (41-76 % active) is the
+// coordinates, the chains and the weights; twelve warps an SM (eight for the
+// cosine), as many as the workspaces in shared memory let.
 //
 // Accuracy: F is a common factor of every node, so its error scales the
 // region's value and is not amplified by the rule's weights of both signs
-// (sum |w| is 5.8 at d = 8); the factors carry an error near 2^-53 each.
+// (sum |w| is 5.8 at d = 8), and it is formed beyond FP64 (Centre); the factors
+// carry an error near 2^-53 each.  Against quad precision I7 is within 0.5 to 1.1
+// times, the error estimate within 0.1 to 1 times the separable form's error.
 // Factors may over- or underflow where f does not (a factor is relative to
 // the centre): regions whose factors' exponents do not leave room are
 // evaluated by region_sums64, decided from the region alone, so that every
 // lane mapping takes the same path.
 //
-// Summation order (fixed, the same for T = 1, 4, 32, 128 lanes): classes 2
-// and 3 one leaf per axis (the sum of its two nodes); class 4 one leaf per
-// pair of axes (its four nodes left to right by fused multiply-add); class 5
-// leaves of max(8, 2^d / 128) consecutive sign patterns, left to right by
-// fused multiply-add.  Leaves are combined by the adjacent-pairwise tree.
-// The lane mapping only places leaves: T lanes own consecutive leaves in bit
-// reversed order, as in gm_region64.cuh.
+// Classes 4 and 5 (368 of the 401 nodes at d = 8) add their products in fixed
+// point on the integer pipes (Limbs below); classes 2 and 3 stay in FP64, one
+// leaf per axis (the sum of its two nodes) of the adjacent-pairwise tree, which
+// T lanes share in bit-reversed order as in gm_region64.cuh.  Integer sums are
+// exact and the tree is fixed, so every lane mapping gives the same bits.
 #pragma once
+
+#include <type_traits>
 
 #include "gm_fixed64.cuh"
 #include "gm_region64.cuh"
@@ -49,24 +55,41 @@ struct Fac {
   static constexpr int kind = kNone;
 };
 
-// e(P, j, x, fc): the factor of x on axis j relative to the centre, whose
-// phi is fc
+// e(P, j, c, h, fc, lam): the factor of coordinate c + lam h on axis j relative
+// to the centre's, whose phi is fc.  low(P, j, c, fc): the rounding error of
+// fc.  Coordinates enter as differences from the centre where f is continuous:
+// fewer operations, and no rounding of c + lam h in between.
 template <>
 struct Fac<GMQ_C0> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double x, double fc) {
-    return gexp(fma(-P.a[j], fabs(__dsub_rn(x, P.u[j])), fc));
+  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
+                                             double lam) {
+    const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
+    return gexp(fma(-P.a[j], fabs(t), fc));
+  }
+  template <class PT>
+  __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
+    return fma(P.a[j], fabs(__dsub_rn(c, P.u[j])), -fc);
   }
 };
 
+// b ((t + lam h)^2 - t^2) = lam^2 b h^2 + lam 2 b h t, t = c - u
 template <>
 struct Fac<GMQ_GAUSSIAN> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double x, double fc) {
-    const double t = __dsub_rn(x, P.u[j]);
-    return gexp(fma(-__dmul_rn(P.b[j], t), t, fc));
+  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double,
+                                             double lam) {
+    const double t = __dsub_rn(c, P.u[j]);
+    const double bh = __dmul_rn(P.b[j], h);
+    const double q = __dmul_rn(__dadd_rn(t, t), bh);
+    return gexp(fma(-lam, q, -__dmul_rn(__dmul_rn(lam, lam), __dmul_rn(bh, h))));
+  }
+  template <class PT>
+  __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
+    const double t = __dsub_rn(c, P.u[j]), t2 = __dmul_rn(t, t);
+    return fma(P.b[j], fma(t, t, -t2), fma(P.b[j], t2, -fc));
   }
 };
 
@@ -74,8 +97,13 @@ template <>
 struct Fac<GMQ_DISCONTINUOUS> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double x, double fc) {
-    return gexp(fma(P.a[j], x, -fc));
+  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
+                                             double lam) {
+    return gexp(fma(P.a[j], fma(lam, h, c), -fc));
+  }
+  template <class PT>
+  __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
+    return fma(P.a[j], c, -fc);
   }
 };
 
@@ -83,32 +111,94 @@ template <>
 struct Fac<GMQ_PRODUCT_PEAK> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double x, double fc) {
-    return __dmul_rn(fc, gm_rcp(Sep<GMQ_PRODUCT_PEAK>::phi(P, j, x)));
+  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
+                                             double lam) {
+    const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
+    return __dmul_rn(fc, gm_rcp(fma(t, t, P.b[j])));
   }
 };
 
 template <>
 struct Fac<GMQ_OSCILLATORY> {
   static constexpr int kind = kRotation;
+  template <class PT>
+  __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
+    return fma(P.a[j], c, -fc);
+  }
+};
+
+// F = f(centre) from the axes' phi in order.  Its error is common to every
+// node, so the inner sum is kept to 2^-58 in fixed point, roundings of phi
+// included (for |S| < 16 and every |phi| < 16; in FP64 otherwise), and the
+// product peak's product as a sum of two doubles.
+template <int FAM>
+struct Centre {
+  double S, lo = 0.0;
+  i64 v = 0;
+  bool fixed = true;
+  template <class PT>
+  __device__ __forceinline__ void add(const PT& P, int k, double c, double fc) {
+    using SF = Sep<FAM>;
+    if constexpr (SF::kMul) {
+      if (k == 0) {
+        S = fc;
+      } else {
+        const double p = __dmul_rn(S, fc);
+        lo = fma(lo, fc, fma(S, fc, -p));
+        S = p;
+      }
+    } else {
+      if (k == 0) {
+        S = SF::kBase ? __dadd_rn(SF::base(P), fc) : fc;
+        if (SF::kBase) take(SF::base(P));
+      } else {
+        S = __dadd_rn(S, fc);
+      }
+      take(fc);
+      v += to_fixed(Fac<FAM>::low(P, k, c, fc), 58);
+    }
+  }
+  __device__ __forceinline__ void take(double x) {
+    v += to_fixed(x, 58);
+    fixed = fixed && small(x);
+  }
+  __device__ __forceinline__ static bool small(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x40300000u;  // |x| < 16
+  }
+  __device__ __forceinline__ double value(int d) const {
+    if constexpr (Sep<FAM>::kMul) {
+      const double r = Sep<FAM>::g(d, S);
+      return fma(-__dmul_rn(r, lo), r, r);
+    } else {
+      if (!fixed || !small(S)) return Sep<FAM>::g(d, S);
+      return exp_fixed(FAM == GMQ_DISCONTINUOUS ? v : -v);
+    }
+  }
+  __device__ __forceinline__ void sincos(double& sn, double& cs) const {
+    if (!fixed || !small(S))
+      gm_sincos(S, &sn, &cs);
+    else
+      sincos_fixed(v, &sn, &cs);
+  }
 };
 
 // Workspace of one region (entries `ws` doubles apart): the lambda3 factors
-// E3 [2d] and the class-5 chains A, B, C; with T > 1 lanes also phi at the
+// E3 [2d], for kReal their axes' exponents [d], and the class-5 chains A, B, C; with T > 1 lanes also phi at the
 // centre [d], the factors of lambda2 and lambda5 [2d each] and F [2].  For
 // kReal, chains over axes [0, a), [a, a + b), [a + b, d) of the factors of
 // c +- lambda5 h.  For kRotation every factor is two entries (cosine, sine
 // of the + sign; - is its conjugate) and every chain entry is two, A's
 // chains headed by F.
 struct FacLayout {
-  int e3, A, B, C, phiC, e2, e5, F, words;
+  int e3, x3, A, B, C, phiC, e2, e5, F, words;
 };
 
 __host__ __device__ constexpr FacLayout fac_layout(int d, int kind, bool lanes) {
   FacLayout s{};
   const int m = kind == kRotation ? 2 : 1;
   s.e3 = 0;
-  s.A = 2 * d * m;
+  s.x3 = 2 * d;
+  s.A = kind == kRotation ? 2 * d : 3 * d;
   s.B = s.A + m * (1 << sep_a(d));
   s.C = s.B + (sep_b(d) ? m * (1 << sep_b(d)) : 0);
   int w = s.C + (sep_c(d) ? m * (1 << sep_c(d)) : 0);
@@ -161,6 +251,123 @@ __device__ __forceinline__ int exp_magnitude(double v) {
   return e < 0 ? -e : e;
 }
 
+// The factor e of an axis' coordinate, or -0 where the discontinuous family's
+// f is 0 (a flagged coordinate): every product with it is then 0, it bounds no
+// table's exponent, and its sign tells it from a factor that underflowed.
+template <int FAM, class PT>
+__device__ __forceinline__ double factor(const PT& P, int k, double c, double h, double fc,
+                                         double lam) {
+  if constexpr (Sep<FAM>::kFlag) {
+    if (Sep<FAM>::flag(P, k, fma(lam, h, c))) return -0.0;
+  }
+  return Fac<FAM>::e(P, k, c, h, fc, lam);
+}
+__device__ __forceinline__ int factor_room(double e) {
+  return __double2hiint(e) == (int)0x80000000u ? 0 : exp_magnitude(e);
+}
+
+// Class sums as sums of products of two 53-bit fixed-point numbers.  A number
+// is v 2^(53 - E) rounded, in two signed limbs h 2^27 + l (|h| <= 2^26, |l| <=
+// 2^26); 2^E bounds the table it comes from, so its error is at most 2^-54 of
+// the table's largest entry, an FP64 rounding of that entry.  A product is
+// h h' 2^54 + (h l' + l h') 2^27, three multiply-adds to 64 bits (12 cycles of
+// an SM quarter against 76 for an FP64 instruction); l l', below 2^-54 of the
+// largest product and of either sign, is left out.  Sums are exact integers:
+// no order of the nodes and no lane mapping changes a bit.
+struct Limbs {
+  int h, l;
+};
+
+__device__ __forceinline__ Limbs limbs_split(i64 q) {
+  Limbs r;
+  r.l = ((int)q << 5) >> 5;
+  r.h = (int)((q - r.l) >> 27);
+  return r;
+}
+__device__ __forceinline__ double limbs_pack(Limbs v) { return __hiloint2double(v.h, v.l); }
+__device__ __forceinline__ Limbs limbs_unpack(double w) {
+  Limbs r;
+  r.h = __double2hiint(w);
+  r.l = __double2loint(w);
+  return r;
+}
+// |v| <= 2^E
+__device__ __forceinline__ double limbs_of(double v, int E) {
+  return limbs_pack(limbs_split(to_fixed(v, 53 - E)));
+}
+
+constexpr int kLimbRun = 512;  // products that a LimbAcc takes before it may overflow
+
+struct LimbAcc {
+  i64 hh = 0, mid = 0;
+  __device__ __forceinline__ void add(Limbs a, Limbs b) {
+    hh += (i64)a.h * b.h;
+    mid += (i64)a.h * b.l;
+    mid += (i64)a.l * b.h;
+  }
+  __device__ __forceinline__ void sub(Limbs a, Limbs b) {
+    hh -= (i64)a.h * b.h;
+    mid -= (i64)a.h * b.l;
+    mid -= (i64)a.l * b.h;
+  }
+  // a b as a number of the same kind (53 bits, rounded down)
+  __device__ __forceinline__ static Limbs product(Limbs a, Limbs b) {
+    const i64 mid = (i64)a.h * b.l + (i64)a.l * b.h;
+    return limbs_split((((i64)a.h * b.h) << 1) + (mid >> 26));
+  }
+};
+
+// 128-bit total of LimbAccs, in units of 2^27 products' last places.
+struct LimbSum {
+  i64 hi = 0;
+  u64 lo = 0;
+  __device__ __forceinline__ void add(i64 h, u64 l) {
+    lo += l;
+    hi += h + (lo < l ? 1 : 0);
+  }
+  __device__ __forceinline__ void take(LimbAcc& a) {
+    add(a.hh >> 37, (u64)a.hh << 27);
+    add(a.mid >> 63, (u64)a.mid);
+    a.hh = 0;
+    a.mid = 0;
+  }
+  // times 2^(E - 79): E the sum of the two tables' bounds
+  __device__ __forceinline__ double value(int E) const {
+    const double v = fma((double)hi, 0x1p64, (double)lo);
+    return __dmul_rn(v, __hiloint2double((944 + max(E, -900)) << 20, 0));  // 2^(E - 79)
+  }
+};
+
+template <int T>
+__device__ __forceinline__ void lanes_add(LimbSum& x, unsigned mask) {
+  if constexpr (T > 32) {
+    __shared__ i64 sh[T];
+    __shared__ u64 sl[T];
+    const int l = threadIdx.x & (T - 1);
+#pragma unroll
+    for (int off = T / 2; off >= 32; off >>= 1) {
+      __syncthreads();
+      sh[l] = x.hi;
+      sl[l] = x.lo;
+      __syncthreads();
+      x.add(sh[l ^ off], sl[l ^ off]);
+    }
+  }
+  constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+  for (int off = W / 2; off > 0; off >>= 1) {
+    const i64 h = __shfl_xor_sync(mask, x.hi, off, W);
+    const u64 l = __shfl_xor_sync(mask, x.lo, off, W);
+    x.add(h, l);
+  }
+}
+
+// Exponent E with v < 2^E; a zero (a flagged factor), below every factor with
+// room, gets one that leaves its fixed-point value 0.
+__device__ __forceinline__ int exp_bound(double v) {
+  return max(((__double2hiint(v) >> 20) & 0x7ff) - 1022, -900);
+}
+
 // The leaves that a lane of T owns when a tree has 2^lg leaf positions:
 // [p0, p0 + cnt), bit-reversed as the butterfly of lanes_tree expects; with
 // fewer leaves than lanes, lane l < 2^lg owns one.
@@ -181,47 +388,29 @@ __device__ __forceinline__ void lane_leaves(int lane, int lg, int& p0, int& cnt)
   }
 }
 
-// Sum of `n` leaves, leaf(p) the value of leaf p, over a tree of 2^lg >= n
-// positions by the T lanes of a group.
-template <int T, class Leaf>
-__device__ __forceinline__ double leaf_sum(int n, int lg, int lane, unsigned mask, Leaf leaf) {
-  PairTree t;
-  int p0, cnt;
-  lane_leaves<T>(lane, lg, p0, cnt);
-  const int p1 = min(p0 + cnt, n);
-  for (int p = p0; p < p1; ++p) t.push(leaf(p));
-  bool present;
-  const double x = t.flush(present);
-  return lanes_tree<T>(x, present, mask);
-}
-
-// log2 of the leaf positions of class 5 (leaves of at least 8 patterns, at
-// most 128 leaves) and of the pairs of axes (<= 120) and axes (<= 16)
-__device__ __forceinline__ int fac_lg5(int d) { return d <= 3 ? 0 : min(7, d - 3); }
 __device__ __forceinline__ int lg_ceil(int n) { return n <= 1 ? 0 : 32 - __clz(n - 1); }
 
-// Class 5 of the real factors: pattern m = (m_A, hi), value A[m_A] *
-// (B[hi] or B[.] C[.]); a leaf runs over whole stretches of m_A.
-// zero(m): the discontinuous family's nodes that are 0.
-template <bool kFlag, class WF, class Zero>
-__device__ __forceinline__ double fac_leaf5(const WF& W, const FacLayout& Ly, int pa, int pb,
-                                            int pc, int m0, int cs, const Zero& zero) {
-  const int am = (1 << pa) - 1;
-  const int run = min(cs, 1 << pa);
-  double x = 0.0;
-  for (int s = 0; s < cs; s += run) {
-    const int m = m0 + s, hi = m >> pa, ea = Ly.A + (m & am);
-    double bc = 1.0;
-    if (pb) bc = W(Ly.B + (hi & ((1 << pb) - 1)));
-    if (pc) bc = __dmul_rn(bc, W(Ly.C + (hi >> pb)));
-#pragma unroll 4
-    for (int q = 0; q < run; ++q) {
-      double a = W(ea + q);
-      if (kFlag && zero(m + q)) a = 0.0;
-      x = (s | q) ? fma(a, bc, x) : __dmul_rn(a, bc);
+// Class 5 of the real factors by one thread: pattern m = (m_A, hi), value
+// A[m_A] B[hi] (A[m_A] (B[.] C[.]) above d = 8); CH entries of A stay in
+// registers while hi runs, so a product costs one shared-memory read in CH.
+template <int CH, class WF>
+__device__ __forceinline__ void fac_class5(const WF& W, const FacLayout& Ly, int pa, int pb, int pc,
+                                           LimbSum& sum) {
+  const int nA = 1 << pa, nhi = 1 << (pb + pc), bm = (1 << pb) - 1;
+  for (int lo = 0; lo < nA; lo += CH) {
+    Limbs a[CH];
+#pragma unroll
+    for (int i = 0; i < CH; ++i) a[i] = limbs_unpack(W(Ly.A + lo + i));
+    LimbAcc acc;
+    for (int hi = 0; hi < nhi; ++hi) {
+      Limbs b = limbs_unpack(W(Ly.B + (hi & bm)));
+      if (pc) b = LimbAcc::product(b, limbs_unpack(W(Ly.C + (hi >> pb))));
+#pragma unroll
+      for (int i = 0; i < CH; ++i) acc.add(a[i], b);
+      if (((hi + 1) & (kLimbRun / CH - 1)) == 0) sum.take(acc);
     }
+    sum.take(acc);
   }
-  return x;
 }
 
 // Class sums and split axis of one region from per-axis factors (kReal);
@@ -233,85 +422,67 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
                                                    double lam5, double* w, int ws, double ratio,
                                                    RegionSums& o) {
   using SF = Sep<FAM>;
-  using FF = Fac<FAM>;
   const int lane = (T == 1) ? 0 : (int)(threadIdx.x & (unsigned)(T - 1));
   const unsigned mask = group_mask<T>();
   const FacLayout Ly = fac_layout(d, kReal, T > 1);
   const int pa = sep_a(d), pb = sep_b(d), pc = sep_c(d);
   auto W = [&](int e) -> double& { return w[(long long)e * ws]; };
-  auto op = [](double x, double y) -> double {
-    if constexpr (SF::kMul)
-      return __dmul_rn(x, y);
-    else
-      return __dadd_rn(x, y);
-  };
-  // flag masks of the discontinuous family (x_j > u_j): centre; c +- lambda3
-  // h and c +- lambda5 h (+ in bits 0..15, - in bits 16..31)
-  unsigned zc = 0u, z3 = 0u, z5 = 0u;
+  unsigned zc = 0u;  // discontinuous family: the axes whose centre is flagged
   double F, s2, s3, dbest = -1.0;  // class sums and differences relative to F
   int kbest = 0, room = 0;
+  unsigned top5 = 0;  // bit k: axis k's larger lambda5 factor is the - one
   // first axis and length of the chain part that axis k belongs to
   auto part = [&](int k, int& e0, int& i) {
     e0 = k < pa ? Ly.A : (k < pa + pb ? Ly.B : Ly.C);
     i = k < pa ? k : (k < pa + pb ? k - pa : k - pa - pb);
   };
   // sums of an axis's node pairs and its fourth difference
-  auto axis = [&](int k, double p2, double m2, double p3, double m3, bool fp2, bool fm2,
-                  double& q2, double& q3) {
+  auto axis = [&](int k, double p2, double m2, double p3, double m3, double& q2, double& q3) {
     double f0 = 1.0;
     if constexpr (SF::kFlag) {
       if (zc & ~(1u << k)) p2 = m2 = p3 = m3 = 0.0;
       if (zc) f0 = 0.0;
-      if (fp2) p2 = 0.0;
-      if (fm2) m2 = 0.0;
-      if ((z3 >> k) & 1u) p3 = 0.0;
-      if ((z3 >> (k + 16)) & 1u) m3 = 0.0;
     }
     q2 = __dadd_rn(p2, m2);
     q3 = __dadd_rn(p3, m3);
     const double two_f0 = f0 + f0;
     const double D = fabs(__dsub_rn(__dsub_rn(q2, two_f0),
                                     __dmul_rn(ratio, __dsub_rn(q3, two_f0))));
-    if (D > dbest) {
+    // D >= 0: the order of the bit patterns
+    if (__double_as_longlong(D) > __double_as_longlong(dbest)) {
       dbest = D;
       kbest = k;
     }
   };
-  if constexpr (T == 1) {
-    if constexpr (SF::kFlag) {
-      for (int k = 0; k < d; ++k) {
-        double c, h;
-        ch(k, c, h);
-        zc |= (unsigned)SF::flag(P, k, c) << k;
-      }
+  if constexpr (SF::kFlag) {
+    for (int k = 0; k < d; ++k) {
+      double c, h;
+      ch(k, c, h);
+      zc |= (unsigned)SF::flag(P, k, c) << k;
     }
+  }
+  if constexpr (T == 1) {
     PairTree t2, t3;
-    double S = 0.0;
+    Centre<FAM> top;
     for (int k = 0; k < d; ++k) {
       double c, h;
       ch(k, c, h);
       const double fc = SF::phi(P, k, c);
-      S = k ? op(S, fc) : fc;
-      const double x2p = fma(lam2, h, c), x2m = fma(-lam2, h, c);
-      const double x3p = fma(lam3, h, c), x3m = fma(-lam3, h, c);
-      const double x5p = fma(lam5, h, c), x5m = fma(-lam5, h, c);
-      const double p2 = FF::e(P, k, x2p, fc), m2 = FF::e(P, k, x2m, fc);
-      const double p3 = FF::e(P, k, x3p, fc), m3 = FF::e(P, k, x3m, fc);
-      const double p5 = FF::e(P, k, x5p, fc), m5 = FF::e(P, k, x5m, fc);
-      room += max(max(exp_magnitude(p2), exp_magnitude(m2)),
-                  max(max(exp_magnitude(p3), exp_magnitude(m3)),
-                      max(exp_magnitude(p5), exp_magnitude(m5))));
+      top.add(P, k, c, fc);
+      const double p2 = factor<FAM>(P, k, c, h, fc, lam2);
+      const double m2 = factor<FAM>(P, k, c, h, fc, -lam2);
+      const double p3 = factor<FAM>(P, k, c, h, fc, lam3);
+      const double m3 = factor<FAM>(P, k, c, h, fc, -lam3);
+      const double p5 = factor<FAM>(P, k, c, h, fc, lam5);
+      const double m5 = factor<FAM>(P, k, c, h, fc, -lam5);
+      room += max(max(factor_room(p2), factor_room(m2)),
+                  max(max(factor_room(p3), factor_room(m3)),
+                      max(factor_room(p5), factor_room(m5))));
       W(Ly.e3 + 2 * k) = p3;
       W(Ly.e3 + 2 * k + 1) = m3;
-      bool fp2 = false, fm2 = false;
-      if constexpr (SF::kFlag) {
-        fp2 = SF::flag(P, k, x2p);
-        fm2 = SF::flag(P, k, x2m);
-        z3 |= ((unsigned)SF::flag(P, k, x3p) << k) | ((unsigned)SF::flag(P, k, x3m) << (k + 16));
-        z5 |= ((unsigned)SF::flag(P, k, x5p) << k) | ((unsigned)SF::flag(P, k, x5m) << (k + 16));
-      }
+      top5 |= (unsigned)(__double_as_longlong(m5) > __double_as_longlong(p5)) << k;
       double q2, q3;
-      axis(k, p2, m2, p3, m3, fp2, fm2, q2, q3);
+      axis(k, p2, m2, p3, m3, q2, q3);
       t2.push(q2);
       t3.push(q3);
       // the part's class-5 chains, by doubling
@@ -329,7 +500,7 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
         }
       }
     }
-    F = SF::g(d, S);
+    F = top.value(d);
     bool pr;
     s2 = t2.flush(pr);
     s3 = t3.flush(pr);
@@ -343,22 +514,10 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
       double c, h;
       ch(k, c, h);
       const double lam = r < 2 ? lam2 : (r < 4 ? lam3 : lam5);
-      const double x = fma((r & 1) ? -lam : lam, h, c);
       const double fc = SF::phi(P, k, c);
-      const double e = FF::e(P, k, x, fc);
+      const double e = factor<FAM>(P, k, c, h, fc, (r & 1) ? -lam : lam);
       W((r < 2 ? Ly.e2 : (r < 4 ? Ly.e3 : Ly.e5)) + 2 * k + (r & 1)) = e;
       if (r == 0) W(Ly.phiC + k) = fc;
-    }
-    if constexpr (SF::kFlag) {
-      for (int k = 0; k < d; ++k) {
-        double c, h;
-        ch(k, c, h);
-        zc |= (unsigned)SF::flag(P, k, c) << k;
-        z3 |= ((unsigned)SF::flag(P, k, fma(lam3, h, c)) << k) |
-              ((unsigned)SF::flag(P, k, fma(-lam3, h, c)) << (k + 16));
-        z5 |= ((unsigned)SF::flag(P, k, fma(lam5, h, c)) << k) |
-              ((unsigned)SF::flag(P, k, fma(-lam5, h, c)) << (k + 16));
-      }
     }
     group_sync<T>(mask);
     // 2. lanes over the tasks: F (and its room, by the lane that forms it)
@@ -366,16 +525,20 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     const int nA = 1 << pa, nB = pb ? 1 << pb : 0, nC = pc ? 1 << pc : 0;
     for (int t = lane; t < 1 + nA + nB + nC; t += T) {
       if (t == 0) {
-        double S = W(Ly.phiC);
-        for (int k = 1; k < d; ++k) S = op(S, W(Ly.phiC + k));
-        const double Fv = SF::g(d, S);
+        Centre<FAM> top;
+        for (int k = 0; k < d; ++k) {
+          double c, h;
+          ch(k, c, h);
+          top.add(P, k, c, W(Ly.phiC + k));
+        }
+        const double Fv = top.value(d);
         for (int k = 0; k < d; ++k) {
           int m = 0;
 #pragma unroll
           for (int s = 0; s < 2; ++s)
-            m = max(m, max(exp_magnitude(W(Ly.e2 + 2 * k + s)),
-                           max(exp_magnitude(W(Ly.e3 + 2 * k + s)),
-                               exp_magnitude(W(Ly.e5 + 2 * k + s)))));
+            m = max(m, max(factor_room(W(Ly.e2 + 2 * k + s)),
+                           max(factor_room(W(Ly.e3 + 2 * k + s)),
+                               factor_room(W(Ly.e5 + 2 * k + s)))));
           big += m;
         }
         W(Ly.F) = Fv;
@@ -412,16 +575,9 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     lane_leaves<T>(lane, lg_ceil(d), p0, cnt);
     const int p1 = min(p0 + cnt, d);
     for (int k = p0; k < p1; ++k) {
-      bool fp2 = false, fm2 = false;
-      if constexpr (SF::kFlag) {
-        double c, h;
-        ch(k, c, h);
-        fp2 = SF::flag(P, k, fma(lam2, h, c));
-        fm2 = SF::flag(P, k, fma(-lam2, h, c));
-      }
       double q2, q3;
-      axis(k, W(Ly.e2 + 2 * k), W(Ly.e2 + 2 * k + 1), W(Ly.e3 + 2 * k), W(Ly.e3 + 2 * k + 1), fp2,
-           fm2, q2, q3);
+      axis(k, W(Ly.e2 + 2 * k), W(Ly.e2 + 2 * k + 1), W(Ly.e3 + 2 * k), W(Ly.e3 + 2 * k + 1), q2,
+           q3);
       t2.push(q2);
       t3.push(q3);
     }
@@ -441,38 +597,113 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     const double x2 = t2.flush(pr2), x3 = t3.flush(pr3);
     s2 = lanes_tree<T>(x2, pr2, mask);
     s3 = lanes_tree<T>(x3, pr3, mask);
+    for (int k = 0; k < d; ++k)
+      top5 |= (unsigned)(__double_as_longlong(W(Ly.e5 + 2 * k + 1)) >
+                         __double_as_longlong(W(Ly.e5 + 2 * k))) << k;
   }
-  // class 4: one leaf per pair j < k, signs ++, +-, -+, --
+  // the tables as limbs: the lambda3 factors, an exponent for each axis, and
+  // the chains, whose largest entry is the product of the larger factors
+  const int nA = 1 << pa, nB = pb ? 1 << pb : 0, nC = pc ? 1 << pc : 0;
+  const int EA = exp_bound(W(Ly.A + (int)(top5 & (unsigned)(nA - 1))));
+  const int EB = pb ? exp_bound(W(Ly.B + (int)((top5 >> pa) & (unsigned)(nB - 1)))) : 0;
+  const int EC = pc ? exp_bound(W(Ly.C + (int)(top5 >> (pa + pb)))) : 0;
+  if constexpr (T > 1) group_sync<T>(mask);  // every lane has read the doubles
+  int M1 = -4096, M2 = -4096;                // the two largest exponents of E3's axes
+  for (int k = lane; k < d; k += T) {
+    const double p3 = W(Ly.e3 + 2 * k), m3 = W(Ly.e3 + 2 * k + 1);
+    const int E = max(exp_bound(p3), exp_bound(m3));
+    W(Ly.e3 + 2 * k) = limbs_of(p3, E);
+    W(Ly.e3 + 2 * k + 1) = limbs_of(m3, E);
+    W(Ly.x3 + k) = __hiloint2double(E, 0);
+    M2 = max(M2, min(M1, E));
+    M1 = max(M1, E);
+  }
+  for (int q = lane; q < nA + nB + nC; q += T)
+    W(Ly.A + q) = limbs_of(W(Ly.A + q), q < nA ? EA : (q < nA + nB ? EB : EC));
+  if constexpr (T > 1) group_sync<T>(mask);
+  if constexpr (T > 1 || SF::kFlag) {
+    // (a flagged centre leaves the pairs that move its axis)
+    M1 = M2 = -4096;
+    const unsigned move = zc & (zc - 1u);  // the flagged axes but the lowest
+    const int first = zc ? __ffs((int)zc) - 1 : -1;
+    for (int k = 0; k < d; ++k) {
+      const int E = __double2hiint(W(Ly.x3 + k));
+      if (k == first) {
+        M2 = max(M2, M1);
+        M1 = E;
+      } else if (first < 0) {
+        M2 = max(M2, min(M1, E));
+        M1 = max(M1, E);
+      } else if (move == 0u || ((move >> k) & 1u)) {
+        if (k < first)
+          M1 = max(M1, E);
+        else
+          M2 = max(M2, E);
+      }
+    }
+  }
+  // class 4: the four nodes of the pairs j < k, a pair's exact sum cut to 2^-55
+  // of the largest product that two axes can have
+  LimbSum s5;
+  LimbAcc acc;
+  i64 s4 = 0;
   const int np = d * (d - 1) / 2;
-  const double s4 = leaf_sum<T>(np, lg_ceil(np), lane, mask, [&](int p) -> double {
+  for (int p = lane; p < np; p += T) {
     const unsigned pr = pairs[p];
     const int j = (int)(pr >> 8), k = (int)(pr & 255u);
-    double j0 = W(Ly.e3 + 2 * j), j1 = W(Ly.e3 + 2 * j + 1);
-    double k0 = W(Ly.e3 + 2 * k), k1 = W(Ly.e3 + 2 * k + 1);
+    const Limbs j0 = limbs_unpack(W(Ly.e3 + 2 * j)), j1 = limbs_unpack(W(Ly.e3 + 2 * j + 1));
+    const Limbs k0 = limbs_unpack(W(Ly.e3 + 2 * k)), k1 = limbs_unpack(W(Ly.e3 + 2 * k + 1));
     if constexpr (SF::kFlag) {
-      if (zc & ~((1u << j) | (1u << k))) j0 = j1 = 0.0;
-      if ((z3 >> j) & 1u) j0 = 0.0;
-      if ((z3 >> (j + 16)) & 1u) j1 = 0.0;
-      if ((z3 >> k) & 1u) k0 = 0.0;
-      if ((z3 >> (k + 16)) & 1u) k1 = 0.0;
+      if (zc & ~((1u << j) | (1u << k))) continue;
     }
-    return fma(j1, k1, fma(j1, k0, fma(j0, k1, __dmul_rn(j0, k0))));
-  });
+    LimbAcc pair;
+    pair.add(j0, k0);
+    pair.add(j0, k1);
+    pair.add(j1, k0);
+    pair.add(j1, k1);
+    const int sh = M1 + M2 - __double2hiint(W(Ly.x3 + j)) - __double2hiint(W(Ly.x3 + k));
+    s4 += ((pair.hh << 1) + (pair.mid >> 26)) >> min(sh, 63);
+  }
   // class 5
-  const int lg5 = fac_lg5(d), cs = 1 << (d - lg5);
-  const unsigned dmask = (1u << d) - 1u;
-  const double s5 = leaf_sum<T>(1 << lg5, lg5, lane, mask, [&](int p) -> double {
-    return fac_leaf5<SF::kFlag>(W, Ly, pa, pb, pc, p * cs, cs, [&](int m) -> bool {
-      return ((((unsigned)~m & z5) | ((unsigned)m & (z5 >> 16))) & dmask) != 0u;
-    });
-  });
+  const Limbs one{1 << 26, 0};
+  if constexpr (T == 1) {
+    if (pb == 0) {  // d = 1
+      for (int q = 0; q < nA; ++q) acc.add(limbs_unpack(W(Ly.A + q)), one);
+      s5.take(acc);
+    } else if (nA >= 8) {
+      fac_class5<8>(W, Ly, pa, pb, pc, s5);
+    } else if (nA >= 4) {
+      fac_class5<4>(W, Ly, pa, pb, pc, s5);
+    } else {
+      fac_class5<2>(W, Ly, pa, pb, pc, s5);
+    }
+  } else {
+    int run = 0;
+    for (int m = lane; m < (1 << d); m += T) {
+      const int hi = m >> pa;
+      Limbs b = pb ? limbs_unpack(W(Ly.B + (hi & (nB - 1)))) : one;
+      if (pc) b = LimbAcc::product(b, limbs_unpack(W(Ly.C + (hi >> pb))));
+      acc.add(limbs_unpack(W(Ly.A + (m & (nA - 1)))), b);
+      if (++run == kLimbRun) {
+        s5.take(acc);
+        run = 0;
+      }
+    }
+    s5.take(acc);
+    LimbSum t4;
+    t4.add(s4 >> 63, (u64)s4);
+    lanes_add<T>(t4, mask);
+    s4 = (i64)t4.lo;
+    lanes_add<T>(s5, mask);
+  }
   double f0 = F;
   if constexpr (SF::kFlag) f0 = zc ? 0.0 : F;
   o.s1 = f0;
   o.s2 = __dmul_rn(F, s2);
   o.s3 = __dmul_rn(F, s3);
-  o.s4 = __dmul_rn(F, s4);
-  o.s5 = __dmul_rn(F, s5);
+  const double scale4 = __hiloint2double((970 + max(M1 + M2, -900)) << 20, 0);  // 2^(M1 + M2 - 53)
+  o.s4 = __dmul_rn(F, __dmul_rn((double)s4, scale4));
+  o.s5 = __dmul_rn(F, s5.value(EA + EB + EC));
   o.f0 = f0;
   o.dbest = __dmul_rn(fabs(F), dbest);
   o.kbest = kbest;
@@ -510,7 +741,8 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
     q3 = __dadd_rn(p3, m3);
     const double D = fabs(__dsub_rn(__dsub_rn(q2, two_f0),
                                     __dmul_rn(ratio, __dsub_rn(q3, two_f0))));
-    if (D > dbest) {
+    // D >= 0: the order of the bit patterns
+    if (__double_as_longlong(D) > __double_as_longlong(dbest)) {
       dbest = D;
       kbest = k;
     }
@@ -521,13 +753,13 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
     ry = fma(x, s, __dmul_rn(y, c));
   };
   if constexpr (T == 1) {
-    double S = SF::base(P);
+    Centre<FAM> top;
     for (int k = 0; k < d; ++k) {
       double c, h;
       ch(k, c, h);
-      S = __dadd_rn(S, SF::phi(P, k, c));
+      top.add(P, k, c, SF::phi(P, k, c));
     }
-    gm_sincos(S, &Fs, &Fc);
+    top.sincos(Fs, Fc);
     PairTree t2, t3;
     for (int k = 0; k < d; ++k) {
       double c, h;
@@ -582,10 +814,14 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
     group_sync<T>(mask);
     // 2. F, then the class-5 chains (A's headed by F)
     if (lane == 0) {
-      double S = SF::base(P);
-      for (int k = 0; k < d; ++k) S = __dadd_rn(S, W(Ly.phiC + k));
+      Centre<FAM> top;
+      for (int k = 0; k < d; ++k) {
+        double c, h;
+        ch(k, c, h);
+        top.add(P, k, c, W(Ly.phiC + k));
+      }
       double sn, cs;
-      gm_sincos(S, &sn, &cs);
+      top.sincos(sn, cs);
       W(Ly.F) = cs;
       W(Ly.F + 1) = sn;
     }
@@ -652,59 +888,124 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
     s2 = lanes_tree<T>(x2, pr2, mask);
     s3 = lanes_tree<T>(x3, pr3, mask);
   }
-  // class 4: F turned by j (both signs), then the four nodes of the pair
-  const int np = d * (d - 1) / 2;
-  const double s4 = leaf_sum<T>(np, lg_ceil(np), lane, mask, [&](int p) -> double {
-    const unsigned pr = pairs[p];
-    const int j = (int)(pr >> 8), k = (int)(pr & 255u);
-    const double cj = W(Ly.e3 + 2 * j), nj = W(Ly.e3 + 2 * j + 1);
-    const double ck = W(Ly.e3 + 2 * k), nk = W(Ly.e3 + 2 * k + 1);
-    double px, py, mx, my;
-    rotate(Fc, Fs, cj, nj, px, py);
-    rotate(Fc, Fs, cj, -nj, mx, my);
-    double x = __dmul_rn(px, ck);
-    x = fma(-py, nk, x);
-    x = fma(px, ck, x);
-    x = fma(py, nk, x);
-    x = fma(mx, ck, x);
-    x = fma(-my, nk, x);
-    x = fma(mx, ck, x);
-    return fma(my, nk, x);
-  });
+  // the chains as limbs (every entry is at most 1)
+  const int nA = 1 << pa, nB = pb ? 1 << pb : 0, nC = pc ? 1 << pc : 0;
+  for (int e = lane; e < 2 * (nA + nB + nC); e += T) W(Ly.A + e) = limbs_of(W(Ly.A + e), 0);
+  if constexpr (T > 1) group_sync<T>(mask);
+  LimbSum s4, s5;
+  LimbAcc acc;
+  int run = 0;
   // class 5: Re(A B) (Re(A (B C)) above d = 8)
-  const int lg5 = fac_lg5(d), cs = 1 << (d - lg5);
-  const int am = (1 << pa) - 1, run = min(cs, 1 << pa);
-  const double s5 = leaf_sum<T>(1 << lg5, lg5, lane, mask, [&](int p) -> double {
-    double x = 0.0;
-    for (int s = 0; s < cs; s += run) {
-      const int m = p * cs + s, hi = m >> pa, ea = Ly.A + 2 * (m & am);
-      double bx = 1.0, by = 0.0;
-      if (pb) {
-        const int eb = Ly.B + 2 * (hi & ((1 << pb) - 1));
-        bx = W(eb);
-        by = W(eb + 1);
+  auto bc_of = [&](int hi, Limbs& x, Limbs& y) {
+    if (!pb) {
+      x = Limbs{1 << 26, 0};
+      y = Limbs{0, 0};
+      return;
+    }
+    const int eb = Ly.B + 2 * (hi & (nB - 1));
+    x = limbs_unpack(W(eb));
+    y = limbs_unpack(W(eb + 1));
+    if (pc) {
+      const int ec = Ly.C + 2 * (hi >> pb);
+      const Limbs u = limbs_unpack(W(ec)), v = limbs_unpack(W(ec + 1));
+      LimbAcc r, i;
+      r.add(x, u);
+      r.sub(y, v);
+      i.add(x, v);
+      i.add(y, u);
+      x = limbs_split((r.hh << 1) + (r.mid >> 26));
+      y = limbs_split((i.hh << 1) + (i.mid >> 26));
+    }
+  };
+  if constexpr (T == 1) {
+    auto walk = [&](auto entries) {  // so many entries of A in registers
+      constexpr int N = decltype(entries)::value;
+      for (int lo = 0; lo < nA; lo += N) {
+        Limbs ax[N], ay[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          ax[i] = limbs_unpack(W(Ly.A + 2 * (lo + i)));
+          ay[i] = limbs_unpack(W(Ly.A + 2 * (lo + i) + 1));
+        }
+        for (int hi = 0; hi < (1 << (pb + pc)); ++hi) {
+          Limbs bx, by;
+          bc_of(hi, bx, by);
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            acc.add(ax[i], bx);
+            acc.sub(ay[i], by);
+          }
+          if (((hi + 1) & (kLimbRun / (2 * N) - 1)) == 0) s5.take(acc);
+        }
+        s5.take(acc);
       }
-      if (pc) {
-        const int ec = Ly.C + 2 * (hi >> pb);
-        double rx, ry;
-        rotate(bx, by, W(ec), W(ec + 1), rx, ry);
-        bx = rx;
-        by = ry;
-      }
-#pragma unroll 4
-      for (int q = 0; q < run; ++q) {
-        const double ax = W(ea + 2 * q), ay = W(ea + 2 * q + 1);
-        x = (s | q) ? fma(ax, bx, x) : __dmul_rn(ax, bx);
-        x = fma(-ay, by, x);
+    };
+    if (nA >= 4)
+      walk(std::integral_constant<int, 4>());
+    else
+      walk(std::integral_constant<int, 2>());
+  } else {
+    for (int m = lane; m < (1 << d); m += T) {
+      Limbs bx, by;
+      bc_of(m >> pa, bx, by);
+      const int ea = Ly.A + 2 * (m & (nA - 1));
+      acc.add(limbs_unpack(W(ea)), bx);
+      acc.sub(limbs_unpack(W(ea + 1)), by);
+      if ((run += 2) == kLimbRun) {
+        s5.take(acc);
+        run = 0;
       }
     }
-    return x;
-  });
+    s5.take(acc);
+  }
+  // a pair needs F turned by its first axis, formed in FP64 once per axis and
+  // sign and kept in the chains' place (4 d <= 2 (2^a + 2^b + 2^c) for every d)
+  if constexpr (T > 1) group_sync<T>(mask);  // the chains and lambda3's doubles have been read
+  const int J = Ly.A;
+  for (int k = lane; k < d; k += T) {
+    const double c3 = W(Ly.e3 + 2 * k), n3 = W(Ly.e3 + 2 * k + 1);
+    double x, y;
+    rotate(Fc, Fs, c3, n3, x, y);
+    W(J + 4 * k) = limbs_of(x, 0);
+    W(J + 4 * k + 1) = limbs_of(y, 0);
+    rotate(Fc, Fs, c3, -n3, x, y);
+    W(J + 4 * k + 2) = limbs_of(x, 0);
+    W(J + 4 * k + 3) = limbs_of(y, 0);
+    W(Ly.e3 + 2 * k) = limbs_of(c3, 0);
+    W(Ly.e3 + 2 * k + 1) = limbs_of(n3, 0);
+  }
+  if constexpr (T > 1) group_sync<T>(mask);
+  // class 4: the four nodes of the pairs j < k, real part of J (c +- i n)
+  const int np = d * (d - 1) / 2;
+  run = 0;
+  for (int p = lane; p < np; p += T) {
+    const unsigned pr = pairs[p];
+    const int j = (int)(pr >> 8), k = (int)(pr & 255u);
+    const Limbs ck = limbs_unpack(W(Ly.e3 + 2 * k)), nk = limbs_unpack(W(Ly.e3 + 2 * k + 1));
+#pragma unroll
+    for (int sj = 0; sj < 2; ++sj) {
+      const Limbs x = limbs_unpack(W(J + 4 * j + 2 * sj));
+      const Limbs y = limbs_unpack(W(J + 4 * j + 2 * sj + 1));
+      acc.add(x, ck);
+      acc.sub(y, nk);
+      acc.add(x, ck);
+      acc.add(y, nk);
+    }
+    if ((run += 8) == kLimbRun) {
+      s4.take(acc);
+      run = 0;
+    }
+  }
+  s4.take(acc);
+  if constexpr (T > 1) {
+    lanes_add<T>(s4, mask);
+    lanes_add<T>(s5, mask);
+  }
   o.s1 = Fc;
   o.s2 = s2;
   o.s3 = s3;
-  o.s4 = s4;
-  o.s5 = s5;
+  o.s4 = s4.value(0);
+  o.s5 = s5.value(0);
   o.f0 = Fc;
   o.dbest = dbest;
   o.kbest = kbest;

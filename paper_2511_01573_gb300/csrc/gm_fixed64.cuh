@@ -27,21 +27,6 @@
 
 namespace gmq {
 
-typedef unsigned long long u64;
-typedef long long i64;
-
-__device__ __forceinline__ u64 wide_mul(unsigned a, unsigned b) { return (u64)a * b; }
-
-// round(x 2^q) for |x| < 2^(62 - q), by integer operations
-__device__ __forceinline__ i64 to_fixed(double x, int q) {
-  const int hi = __double2hiint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
-  const int sh = e - 1075 + q;
-  const i64 v = sh >= 0 ? m << (sh & 15) : (sh > -56 ? ((m >> (-sh - 1)) + 1) >> 1 : 0);
-  return hi < 0 ? -v : v;
-}
-
 // 2^64 / s for s = v / 2^58 in (1 + 2^-9, 4).  An FP32 reciprocal of the
 // leading bits gives y0 (23 bits, relative error below 2^-20); e = 1 - s y0
 // follows exactly from the low 64 bits of v Y0, and y0 (1 + e + e^2) leaves
@@ -56,17 +41,6 @@ __device__ __forceinline__ u64 fixed_rcp(i64 v) {
   const i64 c = ((e >> 17) + (i64)((u64)((i64)eh * eh) >> 34)) >> 4;  // 2^60 (e + e^2)
   const i64 t = (i64)((u64)c * y0);                                   // 2^83 y0 (e + e^2)
   return ((u64)y0 << 41) + (u64)(t >> 19);
-}
-
-// Upper 64 bits of a^2 and a b, up to two units below the exact ones.
-__device__ __forceinline__ u64 fixed_sqr(u64 a) {
-  const unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
-  return wide_mul(h, h) + (wide_mul(h, l) >> 31);
-}
-__device__ __forceinline__ u64 fixed_mul(u64 a, u64 b) {
-  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
-  const unsigned bh = (unsigned)(b >> 32), bl = (unsigned)b;
-  return wide_mul(ah, bh) + (wide_mul(ah, bl) >> 32) + (wide_mul(al, bh) >> 32);
 }
 
 // u[i]^e, e >= 1, by the binary powering of ipow; N values side by side, so

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
       const double x = fma(K.x[j], A.h[(int64_t)k * A.ld + r], c);
       xt[w][q] = x;
       if constexpr (kFactors) {
-        double e = Fac<FAM>::e(P, k, x, SF::phi(P, k, c));
+        double e = Fac<FAM>::e(P, k, c, A.h[(int64_t)k * A.ld + r], SF::phi(P, k, c), K.x[j]);
         atomicMax(&room[w][k], exp_magnitude(e));
         if constexpr (SF::kFlag) {
           if (SF::flag(P, k, x)) e = 0.0;
@@ -251,14 +251,14 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
   double F = 1.0;
   bool factors = false;
   if constexpr (kFactors) {
-    double S = 0.0;
+    Centre<FAM> top;
     int big = 0;
     for (int k = 0; k < d; ++k) {
-      const double fc = SF::phi(P, k, A.c[(int64_t)k * A.ld + r]);
-      S = k ? (SF::kMul ? __dmul_rn(S, fc) : __dadd_rn(S, fc)) : fc;
+      const double c = A.c[(int64_t)k * A.ld + r];
+      top.add(P, k, c, SF::phi(P, k, c));
       big += room[w][k];
     }
-    F = SF::g(d, S);
+    F = top.value(d);
     factors = big <= kFacExpRoom && exp_magnitude(F) <= kFacExpRoom;
     if (factors)
       gk_sums_factors<W>(K, d, lane, kt, gt, rt, s);
