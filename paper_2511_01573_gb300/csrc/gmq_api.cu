@@ -57,6 +57,7 @@ struct gmq_context {
   char* scratch = nullptr;
   size_t scratch_bytes = 0;
   DevStatus* h_status = nullptr;  // pinned, large enough for a BatchState too
+  cudaEvent_t status_ev = nullptr;  // a sweep's status has reached h_status
   std::vector<gmq_sweep> trace;
   int64_t launches = 0;
   // final partition of the last integration (GMQ_KEEP_PARTITION)
@@ -296,21 +297,34 @@ int auto_splits(int d, int64_t cap) {
   return s;
 }
 
-// Threads per region for a sweep of n regions: one thread per region once
-// there are enough regions to give every SM about eight warps; otherwise
-// split each region's nodes over 4 or 32 lanes.
-// Lanes per region for a sweep of n regions: enough threads to fill the
-// GPU (about 256 per SM), a thread per region when the list alone does;
-// a 128-thread block per region (FP64 only) for very short lists of
-// regions with many nodes.
+// Lanes per region for a sweep of n regions (a launch choice: FP64 results do
+// not depend on it).
+// FP64: what a region costs on the FP64 pipe outside its nodes (centre, volume,
+// weights) is paid once per warp, so few lanes per region waste least; more
+// lanes shorten the chain of one region while warps are few.  Measured, rule
+// call in us for 4 / 1 lanes (d = 8, C0 and corner peak): n = 8192: 81 / 111 and
+// 89 / 103, 16384: 114 / 111 and 101 / 106; for 32 / 4 lanes: n = 512: 61 / 75
+// and 64 / 72, 2048: 77 / 75 and 77 / 73, 8192: 143 / 81; d = 10: n = 2048 (the
+// cosine) 98 / 117, 4096: 134 / 115; a block per region only pays for a region
+// or less per SM.
+// Mixed: the register walk of one lane (3 <= d <= 12) wins over 32 lanes from
+// some 2000 regions on at 401 nodes (d = 8, C0: n = 512: 68 / 62, 2048: 69 /
+// 75, 32768: 72 / 302), at once below 130 nodes (d = 5: 58 / 70 at 2048) and
+// from about 5000 at 1245 nodes (d = 10: 93 / 97 at 2048, 92 / 159 at 8192; the
+// corner peak 139 / 98 and 141 / 171); 4 lanes never do (111 to 265 us).
 int choose_lanes(int req, int64_t n, int d, int sms, int precision) {
   if (req) return req;
   const int64_t nodes = num_nodes(d);
-  const int64_t want = (int64_t)sms * 256;
-  if (n >= want || nodes < 16) return 1;
-  if (n * 4 >= want || nodes < 128) return 4;
-  if (n * 32 >= want || nodes < 1024 || precision != GMQ_FP64) return 32;
-  return 128;
+  if (precision != GMQ_FP64) {
+    if (d < 3 || d > 12) {
+      const int64_t want = (int64_t)sms * 256;
+      return n >= want || nodes < 16 ? 1 : (n * 4 >= want || nodes < 128 ? 4 : 32);
+    }
+    return nodes < 256 || n * 256 >= (int64_t)sms * 8 * nodes ? 1 : 32;
+  }
+  if (n >= (int64_t)sms * 96 || nodes < 16) return 1;
+  if (n >= (int64_t)sms * (nodes < 1024 ? 8 : 20) || nodes < 128) return 4;
+  return n > sms || nodes < 1024 ? 32 : 128;
 }
 
 cudaError_t launch_rule(int fam, int precision, int T, const RuleArgs& A, cudaStream_t s) {
@@ -743,10 +757,16 @@ gmq_status gmq_create(gmq_context** out, int device, size_t pool_bytes_hint) {
     delete ctx;
     return GMQ_ERR_CUDA;
   }
+  if (cudaEventCreateWithFlags(&ctx->status_ev, cudaEventDisableTiming) != cudaSuccess) {
+    cudaFreeHost(ctx->h_status);
+    delete ctx;
+    return GMQ_ERR_CUDA;
+  }
   if (pool_bytes_hint > 0) {
     char* base = nullptr;
     gmq_status st = ensure_pool(ctx, pool_bytes_hint, &base);
     if (st != GMQ_OK) {
+      cudaEventDestroy(ctx->status_ev);
       cudaFreeHost(ctx->h_status);
       delete ctx;
       return st;
@@ -765,6 +785,7 @@ gmq_status gmq_destroy(gmq_context* ctx) {
     if (ctx->scratch) cudaFree(ctx->scratch);
     if (ctx->gscratch) cudaFree(ctx->gscratch);
     if (ctx->gk_dev) cudaFree(ctx->gk_dev);
+    if (ctx->status_ev) cudaEventDestroy(ctx->status_ev);
     if (ctx->h_status) cudaFreeHost(ctx->h_status);
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
     if (ctx->ev_made)
@@ -1001,12 +1022,18 @@ gmq_status gmq_integrate(gmq_context* ctx, const gmq_problem* prob, const gmq_op
     prof_begin(ctx, kKClassify);
     GMQ_CK(launch_classify(S, strm));
     prof_end(ctx, kKClassify, n);
+    // the split does not change the status: the host reads it and prepares the
+    // next sweep while the split still runs
+    GMQ_CK(cudaMemcpyAsync(ctx->h_status, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, strm));
+    GMQ_CK(cudaEventRecord(ctx->status_ev, strm));
     prof_begin(ctx, kKSplit);
     GMQ_CK(launch_split(S, strm));
     prof_end(ctx, kKSplit, n);
     ctx->launches += 4;
-    GMQ_CK(cudaMemcpyAsync(ctx->h_status, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, strm));
-    GMQ_CK(cudaStreamSynchronize(strm));
+    if (ctx->prof_on)
+      GMQ_CK(cudaStreamSynchronize(strm));
+    else
+      GMQ_CK(cudaEventSynchronize(ctx->status_ev));
     prof_collect(ctx);
     const DevStatus h = *ctx->h_status;
 
@@ -1054,6 +1081,7 @@ gmq_status gmq_integrate(gmq_context* ctx, const gmq_problem* prob, const gmq_op
     std::swap(cA, cB);
     std::swap(hA, hB);
   }
+  GMQ_CK(cudaStreamSynchronize(strm));  // the last sweep's split has done with the pool
   out->iterations = iters;
   out->status = status;
   // final partition: the leaves recorded so far plus the last sweep's list

@@ -145,4 +145,34 @@ __device__ __forceinline__ double block_tree_sum(double v, double* scratch) {
   return tot;
 }
 
+// Two block_tree_sums at once for kQuad-thread blocks (8 warps): the even
+// lanes of a warp build the tree of a, the odd ones that of b, from the second
+// level on (at the first, lane pairs exchange the operand they do not keep).
+// The same additions as two calls -- a + b == b + a -- with half of the FP64
+// instructions, which is what bounds the kernels that sum per region (an FP64
+// instruction takes ~76 cycles of an SM quarter, whatever its active lanes).
+// scratch: >= 18 doubles of shared memory; both totals in every thread.
+__device__ __forceinline__ void block_tree_sum2(double a, double b, double* scratch, double& ta,
+                                                double& tb) {
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const bool odd = lane & 1u;
+  const double o = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+  double v = (odd ? b : a) + o;
+#pragma unroll
+  for (int off = 2; off < 32; off <<= 1) v = v + __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if (lane < 2) scratch[2 * warp + lane] = v;
+  __syncthreads();
+  if (warp == 0) {
+    double w = scratch[lane & 15u];
+#pragma unroll
+    for (int off = 2; off < 16; off <<= 1) w = w + __shfl_xor_sync(0xffffffffu, w, off);
+    if (lane < 2) scratch[16 + lane] = w + 0.0;  // as with the empty upper half (-0 gives 0)
+  }
+  __syncthreads();
+  ta = scratch[16];
+  tb = scratch[17];
+  __syncthreads();
+}
+
 }  // namespace gmq

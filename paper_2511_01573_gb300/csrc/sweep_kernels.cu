@@ -48,36 +48,42 @@ __device__ double tree_sum_global(const double* v, int64_t count, double* scratc
 // the kTile-thread form.
 constexpr int kQuad = kTile / 4;
 
-__device__ __forceinline__ double tile_sum4(const double* v, int64_t base, int64_t count,
-                                            double* scratch) {
-  const int64_t i = base + 4 * (int64_t)threadIdx.x;
-  const double a = i < count ? v[i] : 0.0, b = i + 1 < count ? v[i + 1] : 0.0;
-  const double c = i + 2 < count ? v[i + 2] : 0.0, d = i + 3 < count ? v[i + 3] : 0.0;
-  return block_tree_sum((a + b) + (c + d), scratch);
+__device__ __forceinline__ double quad_sum(const double* v, int64_t i, int64_t count) {
+  double q[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) q[k] = i + k < count ? __ldcg(v + i + k) : 0.0;
+  return (q[0] + q[1]) + (q[2] + q[3]);
 }
 
-// tree_sum_global for blocks of kQuad threads; the partials were written by
-// other blocks of this launch (read through L2).
-__device__ double tree_sum_global4(const double* v, int64_t count, double* scratch,
-                                   double* tile_sums) {
+// The trees over two arrays of tile sums by one block of kQuad threads; the
+// partials were written by other blocks of this launch (read through L2).
+__device__ void tree_sums_global4(const double* va, const double* vb, int64_t count,
+                                  double* scratch, double (*tile_sums)[kTile], double& ta,
+                                  double& tb) {
+  const int64_t t4 = 4 * (int64_t)threadIdx.x;
   if (count <= kTile) {
-    const int64_t i = 4 * (int64_t)threadIdx.x;
-    double q[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q[k] = i + k < count ? __ldcg(v + i + k) : 0.0;
-    return block_tree_sum((q[0] + q[1]) + (q[2] + q[3]), scratch);
+    block_tree_sum2(quad_sum(va, t4, count), quad_sum(vb, t4, count), scratch, ta, tb);
+    return;
   }
   const int64_t nt = (count + kTile - 1) / kTile;  // <= kTile by construction
   for (int64_t t = 0; t < nt; ++t) {
-    const int64_t i = t * kTile + 4 * (int64_t)threadIdx.x;
-    double q[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q[k] = i + k < count ? __ldcg(v + i + k) : 0.0;
-    const double s = block_tree_sum((q[0] + q[1]) + (q[2] + q[3]), scratch);
-    if (threadIdx.x == 0) tile_sums[t] = s;
+    double a, b;
+    block_tree_sum2(quad_sum(va, t * kTile + t4, count), quad_sum(vb, t * kTile + t4, count),
+                    scratch, a, b);
+    if (threadIdx.x == 0) {
+      tile_sums[0][t] = a;
+      tile_sums[1][t] = b;
+    }
   }
   __syncthreads();
-  return tile_sum4(tile_sums, 0, nt, scratch);
+  double q[2][4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    q[0][k] = t4 + k < nt ? tile_sums[0][t4 + k] : 0.0;
+    q[1][k] = t4 + k < nt ? tile_sums[1][t4 + k] : 0.0;
+  }
+  block_tree_sum2((q[0][0] + q[0][1]) + (q[0][2] + q[0][3]),
+                  (q[1][0] + q[1][1]) + (q[1][2] + q[1][3]), scratch, ta, tb);
 }
 
 // Exclusive scan of in[0..count) (int) into out (long long) by one block of
@@ -134,11 +140,30 @@ __device__ __forceinline__ void load4(const double* v, int64_t i, int64_t n, dou
   }
 }
 
+// x <= y without an FP64 compare for x, y that are not negative (and +0 for
+// zero); false when either is NaN, as the compare.  Negative values and -0 take
+// the compare itself.
+__device__ __forceinline__ bool le_bits(double x, double y) {
+  const long long bx = __double_as_longlong(x), by = __double_as_longlong(y);
+  if ((bx | by) < 0) return x <= y;
+  return bx <= by && by <= 0x7ff0000000000000ll;
+}
+
+// e <= guard |i7|: the product is formed only where the exponents leave it
+// open.  For normal values guard |i7| < 2^(eg + ei + 2) with eg, ei the
+// unbiased exponents, so an e with a larger exponent cannot be under it.
+__device__ __forceinline__ bool under_guard(double e, double i7, double guard) {
+  const int xe = (__double2hiint(e) >> 20) & 0x7ff, xi = (__double2hiint(i7) >> 20) & 0x7ff;
+  const int xg = (__double2hiint(guard) >> 20) & 0x7ff;
+  if (__double2hiint(e) >= 0 && xe > 0 && xi < 0x7ff && xe > xi + xg - 1023 + 2) return false;
+  return e <= __dmul_rn(guard, fabs(i7));
+}
+
 }  // namespace
 
 __global__ void __launch_bounds__(kQuad) k_sum_status(const SweepArgs S) {
   __shared__ double scratch[33];
-  __shared__ double tile_sums[kTile];
+  __shared__ double tile_sums[2][kTile];
   __shared__ int is_last;
   if (S.st->flags & kDone) return;
   // a tile of kTile regions per block, 4 consecutive regions per thread
@@ -146,8 +171,8 @@ __global__ void __launch_bounds__(kQuad) k_sum_status(const SweepArgs S) {
   double a[4], b[4];
   load4(S.i7, r, S.n, a);
   load4(S.err, r, S.n, b);
-  const double ta = block_tree_sum((a[0] + a[1]) + (a[2] + a[3]), scratch);
-  const double tb = block_tree_sum((b[0] + b[1]) + (b[2] + b[3]), scratch);
+  double ta, tb;
+  block_tree_sum2((a[0] + a[1]) + (a[2] + a[3]), (b[0] + b[1]) + (b[2] + b[3]), scratch, ta, tb);
   if (threadIdx.x == 0) {
     S.blk_a[blockIdx.x] = ta;
     S.blk_b[blockIdx.x] = tb;
@@ -158,8 +183,8 @@ __global__ void __launch_bounds__(kQuad) k_sum_status(const SweepArgs S) {
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  const double A = tree_sum_global4(S.blk_a, gridDim.x, scratch, tile_sums);
-  const double B = tree_sum_global4(S.blk_b, gridDim.x, scratch, tile_sums);
+  double A, B;
+  tree_sums_global4(S.blk_a, S.blk_b, gridDim.x, scratch, tile_sums, A, B);
   if (threadIdx.x == 0) {
     DevStatus* st = S.st;
     st->ticket_sum = 0u;
@@ -182,7 +207,7 @@ __global__ void __launch_bounds__(kQuad) k_sum_status(const SweepArgs S) {
 
 __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
   __shared__ double scratch[33];
-  __shared__ double tile_sums[kTile];
+  __shared__ double tile_sums[2][kTile];
   __shared__ long long wsum[32];
   __shared__ int wcnt[kQuad / 32];
   __shared__ int is_last;
@@ -214,8 +239,7 @@ __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
     if (r + k < S.n) {
       const double thr = (S.classifier == GMQ_LOCAL_REL) ? __dmul_rn(S.rel_tol, fabs(i7[k]))
                                                          : __dmul_rn(budget, vf[k]);
-      const double guard = __dmul_rn(S.guard, fabs(i7[k]));
-      const bool retire = (e[k] <= thr) || (e[k] <= guard) || (ax[k] & 0x80);
+      const bool retire = le_bits(e[k], thr) || under_guard(e[k], i7[k], S.guard) || (ax[k] & 0x80);
       fl[k] = retire ? 0 : 1;
       split += fl[k];
       if (retire) {
@@ -234,8 +258,9 @@ __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
   }
   const int wsplit = __reduce_add_sync(0xffffffffu, split);
   if ((threadIdx.x & 31) == 0) wcnt[threadIdx.x >> 5] = wsplit;
-  const double ta = block_tree_sum((ri[0] + ri[1]) + (ri[2] + ri[3]), scratch);  // syncs
-  const double tb = block_tree_sum((re[0] + re[1]) + (re[2] + re[3]), scratch);
+  double ta, tb;
+  block_tree_sum2((ri[0] + ri[1]) + (ri[2] + ri[3]), (re[0] + re[1]) + (re[2] + re[3]), scratch,
+                  ta, tb);  // syncs
   if (threadIdx.x == 0) {
     int cnt = 0;
     for (int w = 0; w < kQuad / 32; ++w) cnt += wcnt[w];
@@ -250,8 +275,8 @@ __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
   if (!is_last) return;
   __threadfence();
   const long long total = block_exclusive_scan_any(S.blk_count, S.blk_off, gridDim.x, wsum);
-  const double A = tree_sum_global4(S.blk_a, gridDim.x, scratch, tile_sums);
-  const double B = tree_sum_global4(S.blk_b, gridDim.x, scratch, tile_sums);
+  double A, B;
+  tree_sums_global4(S.blk_a, S.blk_b, gridDim.x, scratch, tile_sums, A, B);
   if (threadIdx.x == 0) {
     DevStatus* st = S.st;
     st->ticket_cls = 0u;
@@ -279,20 +304,28 @@ __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
   }
 }
 
-__global__ void __launch_bounds__(kTile) k_split(const SweepArgs S) {
-  __shared__ int wcount[32];
+// A quarter of a tile per block of kQuad threads, one region per thread: 1024
+// threads a block with this kernel's registers left one block on an SM and
+// HBM half idle.
+__global__ void __launch_bounds__(kQuad) k_split(const SweepArgs S) {
+  __shared__ int wcount[kQuad / 32];
   if (S.st->flags & kDone) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t r = (int64_t)blockIdx.x * kTile + tid;
+  const int quarter = (int)(blockIdx.x & 3u);
+  const int64_t tile = blockIdx.x >> 2, r0 = tile * kTile;
+  // split regions of the tile's earlier quarters
+  int wpre = 0;
+  for (int q = 0; q < quarter; ++q)
+    wpre += __syncthreads_count(r0 + q * kQuad + tid < S.n && S.flags[r0 + q * kQuad + tid]);
+  const int64_t r = r0 + quarter * kQuad + tid;
   const int f = (r < S.n) ? (int)S.flags[r] : 0;
   const unsigned bal = __ballot_sync(0xffffffffu, f);
   if (lane == 0) wcount[warp] = __popc(bal);
   __syncthreads();
-  int wpre = 0;
   for (int w = 0; w < warp; ++w) wpre += wcount[w];
   if (r >= S.n) return;
   // split regions before r in the whole list
-  const long long pos = S.blk_off[blockIdx.x] + wpre + __popc(bal & ((1u << lane) - 1u));
+  const long long pos = S.blk_off[tile] + wpre + __popc(bal & ((1u << lane) - 1u));
   if (!f) {
     if (S.keep) {
       // retired: append to the final-partition list after the earlier
@@ -427,7 +460,7 @@ cudaError_t launch_classify(const SweepArgs& S, cudaStream_t s) {
 cudaError_t launch_split(const SweepArgs& S, cudaStream_t s) {
   const int64_t blocks = (S.n + kTile - 1) / kTile;
   if (blocks == 0) return cudaSuccess;
-  k_split<<<(unsigned)blocks, kTile, 0, s>>>(S);
+  k_split<<<(unsigned)(4 * blocks), kQuad, 0, s>>>(S);
   return cudaGetLastError();
 }
 

@@ -535,8 +535,8 @@ class Context:
         ld = self._ld(center, halfw)
         cap = 2 * n if cap_out is None else cap_out
         dev = center.device
-        co = torch.zeros((d, max(cap, 1)), dtype=torch.float64, device=dev)
-        ho = torch.zeros((d, max(cap, 1)), dtype=torch.float64, device=dev)
+        co = torch.empty((d, max(cap, 1)), dtype=torch.float64, device=dev)
+        ho = torch.empty((d, max(cap, 1)), dtype=torch.float64, device=dev)
         flags = torch.empty(max(n, 1), dtype=torch.uint8, device=dev)
         ns = C.c_int64()
         ri = C.c_double()
@@ -548,6 +548,9 @@ class Context:
             C.byref(ri), C.byref(re_))
         _check("gmq_classify_split", code, ok=(OK, CAP_REACHED))
         k = int(ns.value)
+        if code == CAP_REACHED:  # nothing was split: no column of the outputs was written
+            co.zero_()
+            ho.zero_()
         return dict(status=code, n_split=k, ret_i=ri.value, ret_e=re_.value, flags=flags[:n],
                     center=co[:, :2 * k], halfw=ho[:, :2 * k])
 
