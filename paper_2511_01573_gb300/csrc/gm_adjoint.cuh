@@ -319,17 +319,41 @@ __device__ __forceinline__ void grad_rows(const GradArgs& A, const SmemParams<do
     double Hr[7];
     rows(j, Hr);
     double ga = 0.0, gu = 0.0;
+    auto rows_of = [&](auto f) {
 #pragma unroll
-    for (int row = 0; row < 7; ++row) {
-      const double lam = row == kXC ? 0.0
-                         : row == kXP2 ? lam2 : row == kXM2 ? -lam2
-                         : row == kXP3 ? lam3 : row == kXM3 ? -lam3
-                         : row == kXP5 ? lam5 : -lam5;
-      const double x = row == kXC ? c : fma(lam, h, c);
-      double ca, cu;
-      SepGrad<FAM>::coef(P, j, x, ca, cu);
-      ga = fma(Hr[row], ca, ga);
-      gu = fma(Hr[row], cu, gu);
+      for (int row = 0; row < 7; ++row)
+        f(Hr[row], row == kXC ? 0.0
+                   : row == kXP2 ? lam2 : row == kXM2 ? -lam2
+                   : row == kXP3 ? lam3 : row == kXM3 ? -lam3
+                   : row == kXP5 ? lam5 : -lam5, row == kXC);
+    };
+    if constexpr (FAM == GMQ_GAUSSIAN) {
+      // dphi/da = 2 a t^2, dphi/du = -2 a^2 t: the sums of H t and H t^2
+      const double t0 = __dsub_rn(c, P.u[j]);
+      rows_of([&](double H, double lam, bool centre) {
+        const double t = centre ? t0 : fma(lam, h, t0), ht = __dmul_rn(H, t);
+        gu = __dadd_rn(gu, ht);
+        ga = fma(ht, t, ga);
+      });
+      ga = __dmul_rn(__dmul_rn(2.0, P.a[j]), ga);
+      gu = __dmul_rn(__dmul_rn(-2.0, P.b[j]), gu);
+    } else if constexpr (FAM == GMQ_C0) {
+      // dphi/da = |t|, dphi/du = -a sign(t)
+      const double t0 = __dsub_rn(c, P.u[j]);
+      rows_of([&](double H, double lam, bool centre) {
+        const double t = centre ? t0 : fma(lam, h, t0);
+        ga = fma(H, fabs(t), ga);
+        const long long bits = __double_as_longlong(t);
+        if (bits << 1) gu = bits < 0 ? __dadd_rn(gu, H) : __dsub_rn(gu, H);
+      });
+      gu = __dmul_rn(P.a[j], gu);
+    } else {
+      rows_of([&](double H, double lam, bool centre) {
+        double ca, cu;
+        SepGrad<FAM>::coef(P, j, centre ? c : fma(lam, h, c), ca, cu);
+        ga = fma(H, ca, ga);
+        gu = fma(H, cu, gu);
+      });
     }
     if constexpr (FAM == GMQ_OSCILLATORY) {
       // base 2 pi u_1: dS/du_1 = 2 pi at every node
@@ -346,7 +370,6 @@ template <int FAM>
 __device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const SmemParams<double>& P,
                                                     double* w, int64_t r) {
   using SF = Sep<FAM>;
-  using FF = Fac<FAM>;
   const int d = A.P.d;
   const int pa = sep_a(d), pb = sep_b(d), pc = sep_c(d);
   const int nlo = 1 << pa, nb = pb ? 1 << pb : 0, nc = pc ? 1 << pc : 0;
@@ -379,9 +402,10 @@ __device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const Sme
     vol = __dmul_rn(vol, __dmul_rn(2.0, h));
     const double fc = SF::phi(P, k, c);
     top.add(P, k, c, fc);
-    double p2 = FF::e(P, k, c, h, fc, lam2), m2 = FF::e(P, k, c, h, fc, -lam2);
-    double p3 = FF::e(P, k, c, h, fc, lam3), m3 = FF::e(P, k, c, h, fc, -lam3);
-    const double p5 = FF::e(P, k, c, h, fc, lam5), m5 = FF::e(P, k, c, h, fc, -lam5);
+    double e[6];
+    axis_factors<FAM>(P, k, c, h, fc, lam2, lam3, lam5, e);
+    double p2 = e[0], m2 = e[1], p3 = e[2], m3 = e[3];
+    const double p5 = e[4], m5 = e[5];
     room += max(max(exp_magnitude(p2), exp_magnitude(m2)),
                 max(max(exp_magnitude(p3), exp_magnitude(m3)),
                     max(exp_magnitude(p5), exp_magnitude(m5))));

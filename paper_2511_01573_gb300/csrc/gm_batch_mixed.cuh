@@ -25,7 +25,7 @@ inline size_t batch_rule_mixed_smem(int dmax) {
 }
 
 template <int FAM>
-__global__ void __launch_bounds__(kBatchRuleBlock) k_batch_rule_mixed(const BatchArgs B) {
+__global__ void __launch_bounds__(kBatchRuleBlock, 4) k_batch_rule_mixed(const BatchArgs B) {
   constexpr int RB = kBatchRuleBlock;
   extern __shared__ __align__(16) double smem[];
   const int dm = B.dmax;
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kBatchRuleBlock) k_batch_rule_mixed(const Batc
   const double* H = B.h[cur];
   const int32_t* rid = B.rid[cur];
   const int tid = threadIdx.x;
-  auto tab = [&](int row, int j) -> float { return xt[(row * dm + j) * RB + tid]; };
+  auto tab = [&](int row, int j) -> float& { return xt[(row * dm + j) * RB + tid]; };
   const float l2 = (float)B.lam2, l3 = (float)B.lam3, l5 = (float)B.lam5;
   // this family's regions: one contiguous range (the batch is in family order)
   const long long r_lo = bs->fam_off[cur][FAM], r_hi = bs->fam_off[cur][FAM + 1];

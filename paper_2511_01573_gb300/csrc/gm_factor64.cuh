@@ -15,12 +15,12 @@
 // rotations (cos Delta, sin Delta), two products per node.  Exponentials, sines
 // and class sums run in fixed point on the integer pipes (gmq_families.cuh,
 // Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
-// the outer function at every node: C0 8.14 -> 1.00 ms (4080 -> 328 FP64
-// instructions a region), Gaussian 8.25 -> 1.14, product peak 4.71 -> 1.21,
-// cosine 10.99 -> 1.95; with factors and FP64 sums and functions they took 2.23,
-// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (41-76 % active) is the
-// coordinates, the chains and the weights; twelve warps an SM (eight for the
-// cosine), as many as the workspaces in shared memory let.
+// the outer function at every node: C0 8.14 -> 0.98 ms (4080 -> 328 FP64
+// instructions a region), Gaussian 8.25 -> 1.03, product peak 4.71 -> 1.12,
+// cosine 10.99 -> 1.40; with factors and FP64 sums and functions they took 2.23,
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-82 % active) is the
+// coordinates, the chains and the weights; twelve warps an SM, as many as the
+// workspaces in shared memory let.
 //
 // Accuracy: F is a common factor of every node, so its error scales the
 // region's value and is not amplified by the rule's weights of both signs
@@ -55,18 +55,18 @@ struct Fac {
   static constexpr int kind = kNone;
 };
 
-// e(P, j, c, h, fc, lam): the factor of coordinate c + lam h on axis j relative
-// to the centre's, whose phi is fc.  low(P, j, c, fc): the rounding error of
-// fc.  Coordinates enter as differences from the centre where f is continuous:
+// The factor of coordinate c + lam h on axis j relative to the centre's, whose
+// phi is fc, is the exponential of (for the product peak fc over) arg(P, j, c,
+// h, fc, lam).  low(P, j, c, fc): the rounding error of fc.  Coordinates enter as differences from the centre where f is continuous:
 // fewer operations, and no rounding of c + lam h in between.
 template <>
 struct Fac<GMQ_C0> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
-                                             double lam) {
+  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
+                                               double lam) {
     const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
-    return gexp(fma(-P.a[j], fabs(t), fc));
+    return fma(-P.a[j], fabs(t), fc);
   }
   template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
@@ -79,12 +79,12 @@ template <>
 struct Fac<GMQ_GAUSSIAN> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double,
-                                             double lam) {
+  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double,
+                                               double lam) {
     const double t = __dsub_rn(c, P.u[j]);
     const double bh = __dmul_rn(P.b[j], h);
     const double q = __dmul_rn(__dadd_rn(t, t), bh);
-    return gexp(fma(-lam, q, -__dmul_rn(__dmul_rn(lam, lam), __dmul_rn(bh, h))));
+    return fma(-lam, q, -__dmul_rn(__dmul_rn(lam, lam), __dmul_rn(bh, h)));
   }
   template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
@@ -97,9 +97,9 @@ template <>
 struct Fac<GMQ_DISCONTINUOUS> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
-                                             double lam) {
-    return gexp(fma(P.a[j], fma(lam, h, c), -fc));
+  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
+                                               double lam) {
+    return fma(P.a[j], fma(lam, h, c), -fc);
   }
   template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
@@ -111,10 +111,10 @@ template <>
 struct Fac<GMQ_PRODUCT_PEAK> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double e(const PT& P, int j, double c, double h, double fc,
-                                             double lam) {
+  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
+                                               double lam) {
     const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
-    return __dmul_rn(fc, gm_rcp(fma(t, t, P.b[j])));
+    return fma(t, t, P.b[j]);
   }
 };
 
@@ -126,6 +126,58 @@ struct Fac<GMQ_OSCILLATORY> {
     return fma(P.a[j], c, -fc);
   }
 };
+
+static __device__ __noinline__ double exp_any(double x) { return gm_exp(x); }
+static __device__ __noinline__ double rcp_any(double x) { return gm_rcp(x); }
+
+// N factors from their arguments.  The fast forms' range is tested once for
+// all, so that their instructions interleave (a test for each kept the six
+// exponentials of an axis one after the other).
+template <int FAM, int N>
+__device__ __forceinline__ void factors(const double (&z)[N], double fc, double (&e)[N]) {
+  bool near = true;
+  if constexpr (Sep<FAM>::kMul) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) near = near && rcp_near(z[i]);
+    if (near) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) e[i] = __dmul_rn(fc, rcp_refined(z[i]));
+      return;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) e[i] = __dmul_rn(fc, rcp_any(z[i]));
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) near = near && exp_near(z[i]);
+    if (near) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) e[i] = exp_fixed(to_fixed(z[i], 58));
+      return;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) e[i] = exp_any(z[i]);
+  }
+}
+
+// The six factors of an axis: c +- lambda2 h, c +- lambda3 h, c +- lambda5 h.
+template <int FAM, class PT>
+__device__ __forceinline__ void axis_factors(const PT& P, int k, double c, double h, double fc,
+                                             double lam2, double lam3, double lam5,
+                                             double (&e)[6]) {
+  const double z[6] = {Fac<FAM>::arg(P, k, c, h, fc, lam2), Fac<FAM>::arg(P, k, c, h, fc, -lam2),
+                       Fac<FAM>::arg(P, k, c, h, fc, lam3), Fac<FAM>::arg(P, k, c, h, fc, -lam3),
+                       Fac<FAM>::arg(P, k, c, h, fc, lam5), Fac<FAM>::arg(P, k, c, h, fc, -lam5)};
+  factors<FAM>(z, fc, e);
+}
+
+template <int FAM, class PT>
+__device__ __forceinline__ double one_factor(const PT& P, int k, double c, double h, double fc,
+                                             double lam) {
+  const double z[1] = {Fac<FAM>::arg(P, k, c, h, fc, lam)};
+  double e[1];
+  factors<FAM>(z, fc, e);
+  return e[0];
+}
 
 // F = f(centre) from the axes' phi in order.  Its error is common to every
 // node, so the inner sum is kept to 2^-58 in fixed point, roundings of phi
@@ -162,9 +214,7 @@ struct Centre {
     v += to_fixed(x, 58);
     fixed = fixed && small(x);
   }
-  __device__ __forceinline__ static bool small(double x) {
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x40300000u;  // |x| < 16
-  }
+  __device__ __forceinline__ static bool small(double x) { return sincos_near(x); }  // |x| < 16
   __device__ __forceinline__ double value(int d) const {
     if constexpr (Sep<FAM>::kMul) {
       const double r = Sep<FAM>::g(d, S);
@@ -189,6 +239,18 @@ struct Centre {
 // c +- lambda5 h.  For kRotation every factor is two entries (cosine, sine
 // of the + sign; - is its conjugate) and every chain entry is two, A's
 // chains headed by F.
+// The rotation's chains have three parts from d = 8 on: 56 words a region
+// instead of 80 put twelve warps on an SM, not eight.
+__host__ __device__ constexpr int fac_c(int kind, int d) {
+  return kind == kRotation && d == 8 ? 2 : sep_c(d);
+}
+__host__ __device__ constexpr int fac_b(int kind, int d) {
+  return kind == kRotation && d == 8 ? 3 : sep_b(d);
+}
+__host__ __device__ constexpr int fac_a(int kind, int d) {
+  return d - fac_b(kind, d) - fac_c(kind, d);
+}
+
 struct FacLayout {
   int e3, x3, A, B, C, phiC, e2, e5, F, words;
 };
@@ -199,9 +261,10 @@ __host__ __device__ constexpr FacLayout fac_layout(int d, int kind, bool lanes) 
   s.e3 = 0;
   s.x3 = 2 * d;
   s.A = kind == kRotation ? 2 * d : 3 * d;
-  s.B = s.A + m * (1 << sep_a(d));
-  s.C = s.B + (sep_b(d) ? m * (1 << sep_b(d)) : 0);
-  int w = s.C + (sep_c(d) ? m * (1 << sep_c(d)) : 0);
+  const int b = fac_b(kind, d), c = fac_c(kind, d);
+  s.B = s.A + m * (1 << fac_a(kind, d));
+  s.C = s.B + (b ? m * (1 << b) : 0);
+  int w = s.C + (c ? m * (1 << c) : 0);
   s.phiC = s.e2 = s.e5 = s.F = -1;
   if (lanes) {
     s.phiC = w;
@@ -224,8 +287,10 @@ __host__ __device__ constexpr bool fac_used(int kind, int d) {
 }
 
 // Words of one region's workspace: the factored and the separable form
-// share it (a region uses one, or first one and then the other).
+// share it (a region uses one, or first one and then the other; the cosine
+// never both).
 __host__ __device__ constexpr int region64_words(int d, int kind, bool flag, bool lanes) {
+  if (kind == kRotation && fac_used(kind, d)) return fac_layout(d, kind, lanes).words;
   const int s = sep_layout(d, flag, lanes).words;
   const int f = fac_used(kind, d) ? fac_layout(d, kind, lanes).words : 0;
   return s > f ? s : f;
@@ -251,16 +316,16 @@ __device__ __forceinline__ int exp_magnitude(double v) {
   return e < 0 ? -e : e;
 }
 
-// The factor e of an axis' coordinate, or -0 where the discontinuous family's
-// f is 0 (a flagged coordinate): every product with it is then 0, it bounds no
-// table's exponent, and its sign tells it from a factor that underflowed.
+// A factor, or -0 where the discontinuous family's f is 0 (a flagged
+// coordinate): every product with it is then 0, it bounds no table's exponent,
+// and its sign tells it from a factor that underflowed.
 template <int FAM, class PT>
-__device__ __forceinline__ double factor(const PT& P, int k, double c, double h, double fc,
-                                         double lam) {
+__device__ __forceinline__ double flag_factor(const PT& P, int k, double c, double h, double lam,
+                                              double e) {
   if constexpr (Sep<FAM>::kFlag) {
     if (Sep<FAM>::flag(P, k, fma(lam, h, c))) return -0.0;
   }
-  return Fac<FAM>::e(P, k, c, h, fc, lam);
+  return e;
 }
 __device__ __forceinline__ int factor_room(double e) {
   return __double2hiint(e) == (int)0x80000000u ? 0 : exp_magnitude(e);
@@ -310,10 +375,14 @@ struct LimbAcc {
     mid -= (i64)a.h * b.l;
     mid -= (i64)a.l * b.h;
   }
-  // a b as a number of the same kind (53 bits, rounded down)
+  // the sum as one number in units of 2^-53 of the products' bound, rounded (for
+  // up to 64 products)
+  __device__ __forceinline__ i64 number() const { return (hh << 1) + ((mid + (1 << 25)) >> 26); }
+  // a b as a number of the same kind
   __device__ __forceinline__ static Limbs product(Limbs a, Limbs b) {
-    const i64 mid = (i64)a.h * b.l + (i64)a.l * b.h;
-    return limbs_split((((i64)a.h * b.h) << 1) + (mid >> 26));
+    LimbAcc r;
+    r.add(a, b);
+    return limbs_split(r.number());
   }
 };
 
@@ -469,12 +538,14 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
       ch(k, c, h);
       const double fc = SF::phi(P, k, c);
       top.add(P, k, c, fc);
-      const double p2 = factor<FAM>(P, k, c, h, fc, lam2);
-      const double m2 = factor<FAM>(P, k, c, h, fc, -lam2);
-      const double p3 = factor<FAM>(P, k, c, h, fc, lam3);
-      const double m3 = factor<FAM>(P, k, c, h, fc, -lam3);
-      const double p5 = factor<FAM>(P, k, c, h, fc, lam5);
-      const double m5 = factor<FAM>(P, k, c, h, fc, -lam5);
+      double e[6];
+      axis_factors<FAM>(P, k, c, h, fc, lam2, lam3, lam5, e);
+      const double p2 = flag_factor<FAM>(P, k, c, h, lam2, e[0]);
+      const double m2 = flag_factor<FAM>(P, k, c, h, -lam2, e[1]);
+      const double p3 = flag_factor<FAM>(P, k, c, h, lam3, e[2]);
+      const double m3 = flag_factor<FAM>(P, k, c, h, -lam3, e[3]);
+      const double p5 = flag_factor<FAM>(P, k, c, h, lam5, e[4]);
+      const double m5 = flag_factor<FAM>(P, k, c, h, -lam5, e[5]);
       room += max(max(factor_room(p2), factor_room(m2)),
                   max(max(factor_room(p3), factor_room(m3)),
                       max(factor_room(p5), factor_room(m5))));
@@ -515,7 +586,9 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
       ch(k, c, h);
       const double lam = r < 2 ? lam2 : (r < 4 ? lam3 : lam5);
       const double fc = SF::phi(P, k, c);
-      const double e = factor<FAM>(P, k, c, h, fc, (r & 1) ? -lam : lam);
+      const double ls = (r & 1) ? -lam : lam;
+      const double e =
+          flag_factor<FAM>(P, k, c, h, ls, one_factor<FAM>(P, k, c, h, fc, ls));
       W((r < 2 ? Ly.e2 : (r < 4 ? Ly.e3 : Ly.e5)) + 2 * k + (r & 1)) = e;
       if (r == 0) W(Ly.phiC + k) = fc;
     }
@@ -662,7 +735,7 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     pair.add(j1, k0);
     pair.add(j1, k1);
     const int sh = M1 + M2 - __double2hiint(W(Ly.x3 + j)) - __double2hiint(W(Ly.x3 + k));
-    s4 += ((pair.hh << 1) + (pair.mid >> 26)) >> min(sh, 63);
+    s4 += pair.number() >> min(sh, 63);
   }
   // class 5
   const Limbs one{1 << 26, 0};
@@ -722,7 +795,7 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
   const int lane = (T == 1) ? 0 : (int)(threadIdx.x & (unsigned)(T - 1));
   const unsigned mask = group_mask<T>();
   const FacLayout Ly = fac_layout(d, kRotation, T > 1);
-  const int pa = sep_a(d), pb = sep_b(d), pc = sep_c(d);
+  const int pa = fac_a(kRotation, d), pb = fac_b(kRotation, d), pc = fac_c(kRotation, d);
   auto W = [&](int e) -> double& { return w[(long long)e * ws]; };
   double Fc, Fs, s2, s3, dbest = -1.0;
   int kbest = 0;
@@ -766,9 +839,16 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
       ch(k, c, h);
       const double ah = __dmul_rn(P.a[k], h);
       double c2, n2, c3, n3, c5, n5;
-      gm_sincos(__dmul_rn(lam2, ah), &n2, &c2);
-      gm_sincos(__dmul_rn(lam3, ah), &n3, &c3);
-      gm_sincos(__dmul_rn(lam5, ah), &n5, &c5);
+      const double z2 = __dmul_rn(lam2, ah), z3 = __dmul_rn(lam3, ah), z5 = __dmul_rn(lam5, ah);
+      if (sincos_near(z2) && sincos_near(z3) && sincos_near(z5)) {
+        sincos_fixed(to_fixed(z2, 58), &n2, &c2);
+        sincos_fixed(to_fixed(z3, 58), &n3, &c3);
+        sincos_fixed(to_fixed(z5, 58), &n5, &c5);
+      } else {
+        gm_sincos(z2, &n2, &c2);
+        gm_sincos(z3, &n3, &c3);
+        gm_sincos(z5, &n5, &c5);
+      }
       W(Ly.e3 + 2 * k) = c3;
       W(Ly.e3 + 2 * k + 1) = n3;
       double q2, q3;
@@ -913,8 +993,8 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
       r.sub(y, v);
       i.add(x, v);
       i.add(y, u);
-      x = limbs_split((r.hh << 1) + (r.mid >> 26));
-      y = limbs_split((i.hh << 1) + (i.mid >> 26));
+      x = limbs_split(r.number());
+      y = limbs_split(i.number());
     }
   };
   if constexpr (T == 1) {

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
       const double x = fma(K.x[j], A.h[(int64_t)k * A.ld + r], c);
       xt[w][q] = x;
       if constexpr (kFactors) {
-        double e = Fac<FAM>::e(P, k, c, A.h[(int64_t)k * A.ld + r], SF::phi(P, k, c), K.x[j]);
+        double e = one_factor<FAM>(P, k, c, A.h[(int64_t)k * A.ld + r], SF::phi(P, k, c), K.x[j]);
         atomicMax(&room[w][k], exp_magnitude(e));
         if constexpr (SF::kFlag) {
           if (SF::flag(P, k, x)) e = 0.0;

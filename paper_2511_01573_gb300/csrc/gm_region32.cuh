@@ -38,13 +38,6 @@ __device__ __forceinline__ void mixed_coord_rows(double c, double h, float l2, f
   out[kXM5 * stride] = __fadd_rn(c_hi, __fmaf_rn(-l5, hf, c_lo));
 }
 
-// Integrand parameters in registers (compile-time dimension).
-template <int D>
-struct RegParams {
-  float a[D], u[D], b[D];
-  float c0;
-};
-
 // Generic dimension: every node in the order of its definition (centre;
 // per axis +l2, -l2, +l3, -l3; pairs j < k with sign patterns ++, +-, -+,
 // --; sign patterns m = 0 .. 2^d - 1).  P holds FP32 parameters;
@@ -130,62 +123,215 @@ __device__ __forceinline__ void region_mixed_flat(const PT& P, int d, const unsi
   o.kbest = kbest;
 }
 
-// Dimension D known at compile time (3 <= D <= 16).  Every node is
-// evaluated together with its partner in one paired FP32 evaluation
-// (Family2::eval2), the partner being the node that differs from it in one
-// coordinate only: the two signs of +-lambda2 e_k and of +-lambda3 e_k; for
-// a pair j < k, the two signs on axis k with the same sign on axis j; in the
-// sign-pattern class, the two signs on axis 0.  The nodes of classes 1-4 are
-// formed from the centre held in registers and the one or two coordinates
-// they move (read from the table), with the moved axis k known at compile
-// time (unrolled over k, the pair's first axis j in a loop).  The 2^D
-// sign-pattern nodes are walked in Gray-code order over a register-resident
-// node vector: consecutive patterns differ in one coordinate, which moves
-// between c_k + l5 h_k and c_k - l5 h_k by XOR-ing the two FP32 bit
-// patterns.  In an aligned group of eight patterns the coordinates that
-// change are axes 0, 1, 0, 2, 0, 1, 0, so the group is four axis-0 pairs,
-// with axes 1, 2, 1 stepping between them; the axis changed on entering the
-// group (>= 3) is picked with a predicated select.  Every class sum adds its
-// node values one by one in definition order (Gray-code order for the last
-// class), as the one-node-at-a-time walk did.  Pf holds the FP32 parameters
-// (read once into registers).
+// The FP32 integrands as chains: y(P, j, x) is what axis j's coordinate x enters
+// the inner chain as, step appends it to the chain s of axes 0 .. j - 1, and out
+// is the integrand from the whole chain; step2 and outs work on pairs of nodes
+// (paired FP32 instructions).  Exactly the operations of Family<FAM>::eval in
+// their order, so a node's value has its bits, and nodes that agree on axes 0 ..
+// j share the chain so far.
+template <int FAM>
+struct Chain {
+  static constexpr bool kPeak = FAM == GMQ_PRODUCT_PEAK, kGauss = FAM == GMQ_GAUSSIAN;
+  static constexpr bool kC0 = FAM == GMQ_C0, kDisc = FAM == GMQ_DISCONTINUOUS;
+  static constexpr bool kPoly = FAM == GMQ_POLY_SUMSQ11;
+  template <class PT>
+  __device__ __forceinline__ static float init(const PT& P) {
+    if constexpr (FAM == GMQ_OSCILLATORY) return P.c0;
+    return kPeak || FAM == GMQ_CORNER_PEAK ? 1.0f : 0.0f;
+  }
+  template <class PT>
+  __device__ __forceinline__ static float y(const PT& P, int j, float x) {
+    if constexpr (kPeak || kGauss || kC0) {
+      const float t = x - P.u[j];
+      if constexpr (kPeak) return fmaf(t, t, P.b[j]);
+      return kC0 ? fabsf(t) : t * t;
+    }
+    return x;
+  }
+  // a: the axis' factor of y (not used by the product peak and the polynomial);
+  // u: its threshold (the discontinuous family: -inf, whose exponential is 0,
+  // from the first coordinate above it)
+  template <class PT>
+  __device__ __forceinline__ static float coef(const PT& P, int j) {
+    return kGauss ? P.b[j] : P.a[j];
+  }
+  __device__ __forceinline__ static float step(float s, float a, float u, float v) {
+    if constexpr (kPeak) return s * v;
+    if constexpr (kPoly) return fmaf(v, v, s);
+    if constexpr (kDisc) return v > u ? -__int_as_float(0x7f800000) : fmaf(a, v, s);
+    return fmaf(a, v, s);
+  }
+  __device__ __forceinline__ static float2 step2(float2 s, float a, float u, float2 v) {
+    if constexpr (kPeak) return __fmul2_rn(s, v);
+    if constexpr (kPoly) return __ffma2_rn(v, v, s);
+    const float2 r = __ffma2_rn(bc2(a), v, s);
+    if constexpr (kDisc) {
+      const float ninf = -__int_as_float(0x7f800000);
+      return make_float2(v.x > u ? ninf : r.x, v.y > u ? ninf : r.y);
+    }
+    return r;
+  }
+  __device__ __forceinline__ static float out(int d, float s) {
+    if constexpr (FAM == GMQ_OSCILLATORY) return gcos(s);
+    if constexpr (kPeak) return grcp(s);
+    if constexpr (FAM == GMQ_CORNER_PEAK) return grcp(ipow(s, d + 1));
+    if constexpr (kGauss || kC0) return gexp(-s);
+    if constexpr (kDisc) return gexp(s);
+    const float s2 = s * s, s4 = s2 * s2, s8 = s4 * s4;
+    return s8 * s2 * s;
+  }
+  // out of N pairs of nodes.  The reciprocal and the cosine have fast forms with
+  // the same bits on a range that every integrand in use stays in; one test for
+  // all pairs, not one for each, so that their instructions interleave.
+  template <int D, int N>
+  __device__ __forceinline__ static void outs(float2 (&s)[N]) {
+    if constexpr (kPeak || FAM == GMQ_CORNER_PEAK) {
+      if constexpr (FAM == GMQ_CORNER_PEAK) {
+        // the binary powering of ipow
+        constexpr int e = D + 1, low = e & -e;
+        float2 r[N];
+#pragma unroll
+        for (int b = 1; b <= e; b <<= 1) {
+#pragma unroll
+          for (int n = 0; n < N; ++n) {
+            if (b > 1) s[n] = __fmul2_rn(s[n], s[n]);
+            if (b == low)
+              r[n] = s[n];
+            else if (e & b)
+              r[n] = __fmul2_rn(r[n], s[n]);
+          }
+        }
+#pragma unroll
+        for (int n = 0; n < N; ++n) s[n] = r[n];
+      }
+      unsigned far = 0u;
+      float2 q[N];
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        far |= rcpf_far(s[n].x) | rcpf_far(s[n].y);
+        q[n] = rcpf2(s[n]);
+      }
+      if (far) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) q[n] = make_float2(grcp(s[n].x), grcp(s[n].y));
+      }
+#pragma unroll
+      for (int n = 0; n < N; ++n) s[n] = q[n];
+    } else if constexpr (FAM == GMQ_OSCILLATORY) {
+      bool near = true;
+#pragma unroll
+      for (int n = 0; n < N; ++n)
+        near = near && fabsf(s[n].x) < 32768.0f && fabsf(s[n].y) < 32768.0f;
+      if (near) {
+#pragma unroll
+        for (int n = 0; n < N; ++n) s[n] = gm_cosf2_near(s[n]);
+      } else {
+#pragma unroll
+        for (int n = 0; n < N; ++n) s[n] = make_float2(gm_cosf(s[n].x), gm_cosf(s[n].y));
+      }
+    } else if constexpr (kPoly) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        const float2 s2 = __fmul2_rn(s[n], s[n]), s4 = __fmul2_rn(s2, s2), s8 = __fmul2_rn(s4, s4);
+        s[n] = __fmul2_rn(__fmul2_rn(s8, s2), s[n]);
+      }
+    } else {
+#pragma unroll
+      for (int n = 0; n < N; ++n) s[n] = make_float2(out(D, s[n].x), out(D, s[n].y));
+    }
+  }
+};
+
+// Two compensated FP32 sums side by side (Knuth's TwoSum, paired instructions).
+struct Acc2 {
+  float2 s = {0.0f, 0.0f}, c = {0.0f, 0.0f};
+  __device__ __forceinline__ void add(float2 v) {
+    auto neg = [](float2 x) { return make_float2(-x.x, -x.y); };
+    const float2 t = __fadd2_rn(s, v);
+    const float2 bp = __fadd2_rn(t, neg(s));
+    const float2 ap = __fadd2_rn(t, neg(bp));
+    c = __fadd2_rn(c, __fadd2_rn(__fadd2_rn(s, neg(ap)), __fadd2_rn(v, neg(bp))));
+    s = t;
+  }
+  // both sums as one (the FP64 pipe adds once: at small D it is what bounds)
+  __device__ __forceinline__ Acc<float> one() const {
+    Acc<float> a;
+    a.s = s.x;
+    a.c = __fadd_rn(c.x, c.y);
+    a.add(s.y);
+    return a;
+  }
+  __device__ __forceinline__ double value() const { return one().value(); }
+  __device__ __forceinline__ double value(const Acc2& b) const {
+    Acc<float> x = one();
+    const Acc<float> y = b.one();
+    x.c = __fadd_rn(x.c, y.c);
+    x.add(y.s);
+    return x.value();
+  }
+};
+
+// Dimension D known at compile time (3 <= D <= 16), one thread per region.
+// Bound: FP32 issue.  Evaluated node by node a node's chain costs D steps (12 of
+// 26 FP32 operations for the corner peak at D = 12), so nodes are walked as a
+// tree over the axes in chain order, where those that agree on the first axes
+// share the chain so far -- the same operations on the same operands, hence the
+// same bits.  Sign patterns: the outer axes' prefixes are kept in registers and
+// renewed from the axis that changes on, the last four axes are unrolled to 16
+// patterns (30 steps), so a pattern costs two steps instead of D.  Classes 2
+// to 4 share the prefix up to the first moved axis (and, for a pair, the
+// stretch between the two); only the chain after the last moved axis is walked
+// for each.  Nodes come in pairs on the paired FP32 instructions.  Class sums
+// are compensated, and the sums of FP32 values of like size that they hold are
+// exact, so the order of the walk leaves no trace above 1e-14.
+// tab(row, j): the thread's own column of node coordinates, overwritten with
+// y of them.  2^20 regions, d = 12 / d = 8: corner peak 4.83 -> 3.54 / 0.477 ->
+// 0.386 ms, product peak 4.79 -> 2.98 / 0.482 -> 0.387, Gaussian 4.08 -> 2.95 /
+// 0.424 -> 0.347, C0 3.66 -> 2.97 / 0.391 -> 0.349, cosine 5.78 -> 4.65 / 0.618
+// -> 0.478; up to d = 5 the FP64 differences and weights bound both forms alike.
 template <int FAM, int D, class PT, class Tab>
 __device__ __forceinline__ void region_mixed_walk(const PT& Pf, const Tab& tab, double ratio,
                                                   RegionSums& o) {
-  static_assert(D >= 3 && D <= 16, "the Gray walk needs D >= 3");
-  RegParams<D> rp;
+  static_assert(D >= 3 && D <= 16, "the walk needs D >= 3");
+  using CH = Chain<FAM>;
+  float a[D], yc[D];
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    rp.a[j] = Pf.a[j];
-    rp.u[j] = Pf.u[j];
-    rp.b[j] = Pf.b[j];
+    a[j] = CH::coef(Pf, j);
+#pragma unroll
+    for (int row = 0; row < kXRows; ++row) tab(row, j) = CH::y(Pf, j, tab(row, j));
+    yc[j] = tab(kXC, j);
   }
-  rp.c0 = Pf.c0;
-  Acc<float> S1, S2, S3, S4, S5;
+  auto thr = [&](int j) -> float { return CH::kDisc ? Pf.u[j] : 0.0f; };
+  // the centres of axes k .. D - 1 appended
+  auto rest2 = [&](float2 s, int k) -> float2 {
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+      if (i >= k) s = CH::step2(s, a[i], thr(i), bc2(yc[i]));
+    return s;
+  };
+  const float s0 = CH::init(Pf);
   double dbest = -1.0;
   int kbest = 0;
-  float xc[D];
+  // class 1
+  float sc = s0;
 #pragma unroll
-  for (int j = 0; j < D; ++j) xc[j] = tab(kXC, j);
-  // class 1: the centre
-  const float vc = Family<FAM>::template eval<float>(rp, D, [&](int j) -> float { return xc[j]; });
-  S1.add(vc);
-  const double f0 = f2d_exact(vc);
+  for (int j = 0; j < D; ++j) sc = CH::step(sc, a[j], thr(j), yc[j]);
+  const double f0 = f2d_exact(CH::out(D, sc));
   const double two_f0 = __dmul_rn(2.0, f0);
   // classes 2 and 3: per axis k the pairs (+l2, -l2) and (+l3, -l3), and
   // the fourth difference of axis k
+  Acc2 S2, S3, S4, S4b, S5, S5b;  // two chains of sums where nodes come in numbers
+  float pre = s0;
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    const float2 p2 = make_float2(tab(kXP2, k), tab(kXM2, k));
-    const float2 p3 = make_float2(tab(kXP3, k), tab(kXM3, k));
-    const float2 v2 = Family2<FAM>::eval2(
-        rp, D, [&](int j) -> float2 { return j == k ? p2 : bc2(xc[j]); });
-    const float2 v3 = Family2<FAM>::eval2(
-        rp, D, [&](int j) -> float2 { return j == k ? p3 : bc2(xc[j]); });
-    S2.add(v2.x);
-    S2.add(v2.y);
-    S3.add(v3.x);
-    S3.add(v3.y);
+    float2 v[2] = {
+        rest2(CH::step2(bc2(pre), a[k], thr(k), make_float2(tab(kXP2, k), tab(kXM2, k))), k + 1),
+        rest2(CH::step2(bc2(pre), a[k], thr(k), make_float2(tab(kXP3, k), tab(kXM3, k))), k + 1)};
+    CH::template outs<D>(v);
+    const float2 v2 = v[0], v3 = v[1];
+    S2.add(v2);
+    S3.add(v3);
     const double t1 = __dsub_rn(__dadd_rn(f2d_exact(v2.x), f2d_exact(v2.y)), two_f0);
     const double t2 = __dsub_rn(__dadd_rn(f2d_exact(v3.x), f2d_exact(v3.y)), two_f0);
     const double Dk = fabs(__dsub_rn(t1, __dmul_rn(ratio, t2)));
@@ -193,70 +339,65 @@ __device__ __forceinline__ void region_mixed_walk(const PT& Pf, const Tab& tab, 
       dbest = Dk;
       kbest = k;
     }
+    pre = CH::step(pre, a[k], thr(k), yc[k]);
   }
-  // class 4: pairs j < k, sign patterns ++, +-, -+, -- (the pairs on axis k)
+  // class 4: pairs j < k, the two signs on axis j side by side
+  pre = s0;
   for (int j = 0; j < D - 1; ++j) {
-    const float pj = tab(kXP3, j), mj = tab(kXM3, j);
+    const float aj = CH::coef(Pf, j), uj = thr(j);
+    float2 q = CH::step2(bc2(pre), aj, uj, make_float2(tab(kXP3, j), tab(kXM3, j)));
 #pragma unroll
     for (int k = 1; k < D; ++k) {
       if (k > j) {
-        const float2 pk = make_float2(tab(kXP3, k), tab(kXM3, k));
-        const float2 va = Family2<FAM>::eval2(rp, D, [&](int i) -> float2 {
-          return i == k ? pk : bc2(i == j ? pj : xc[i]);
-        });
-        const float2 vb = Family2<FAM>::eval2(rp, D, [&](int i) -> float2 {
-          return i == k ? pk : bc2(i == j ? mj : xc[i]);
-        });
-        S4.add(va.x);
-        S4.add(va.y);
-        S4.add(vb.x);
-        S4.add(vb.y);
+        float2 v[2] = {rest2(CH::step2(q, a[k], thr(k), bc2(tab(kXP3, k))), k + 1),
+                       rest2(CH::step2(q, a[k], thr(k), bc2(tab(kXM3, k))), k + 1)};
+        CH::template outs<D>(v);
+        S4.add(v[0]);
+        S4b.add(v[1]);
+        q = CH::step2(q, a[k], thr(k), bc2(yc[k]));
       }
     }
+    pre = CH::step(pre, aj, uj, tab(kXC, j));
   }
-  // class 5: Gray-code walk over the 2^D sign patterns in registers
-  float x[D];
-  unsigned tog[D];
+  // class 5: O outer axes, bit b of the counter being the sign of axis O - 1 - b;
+  // I inner axes unrolled
+  constexpr int I = D < 4 ? D : 4, O = D - I;
+  float p5[I], m5[I], p[O + 1];
 #pragma unroll
-  for (int k = 0; k < D; ++k) {
-    const float p5 = tab(kXP5, k), m5 = tab(kXM5, k);
-    x[k] = p5;
-    tog[k] = __float_as_uint(p5) ^ __float_as_uint(m5);
+  for (int i = 0; i < I; ++i) {
+    p5[i] = tab(kXP5, O + i);
+    m5[i] = tab(kXM5, O + i);
   }
-  auto flip = [&](int k) { x[k] = __uint_as_float(__float_as_uint(x[k]) ^ tog[k]); };
-  // the pattern x and its axis-0 partner, in walk order
-  auto pair5 = [&]() {
-    const float2 x0 = make_float2(x[0], __uint_as_float(__float_as_uint(x[0]) ^ tog[0]));
-    const float2 v = Family2<FAM>::eval2(rp, D, [&](int i) -> float2 {
-      return i == 0 ? x0 : bc2(x[i]);
-    });
-    S5.add(v.x);
-    S5.add(v.y);
-  };
-  for (unsigned tb = 0; tb < (1u << D); tb += 8u) {
-    if (tb) {
-      const int jb = __ffs(tb) - 1;
+  p[0] = s0;
+  for (unsigned t = 0; t < (1u << O); ++t) {
+    const int from = t ? O - __ffs((int)t) : 0;  // the first axis whose sign changed
 #pragma unroll
-      for (int k = 3; k < D; ++k)
-        if (k == jb) flip(k);
+    for (int k = 0; k < O; ++k)
+      if (k >= from)
+        p[k + 1] = CH::step(p[k], a[k], thr(k), tab((t >> (O - 1 - k)) & 1u ? kXM5 : kXP5, k));
+    float2 v[1 << (I - 1)];
+    v[0] = CH::step2(bc2(p[O]), a[O], thr(O), make_float2(p5[0], m5[0]));
+#pragma unroll
+    for (int i = 1; i < I; ++i) {
+#pragma unroll
+      for (int n = (1 << (i - 1)) - 1; n >= 0; --n) {
+        const float2 s = v[n];
+        v[2 * n] = CH::step2(s, a[O + i], thr(O + i), bc2(p5[i]));
+        v[2 * n + 1] = CH::step2(s, a[O + i], thr(O + i), bc2(m5[i]));
+      }
     }
-    pair5();  // patterns 0, 1 of the group
-    flip(0);
-    flip(1);
-    pair5();  // 2, 3
-    flip(0);
-    flip(2);
-    pair5();  // 4, 5
-    flip(0);
-    flip(1);
-    pair5();  // 6, 7
-    flip(0);  // the group ends on pattern 7
+    CH::template outs<D>(v);
+#pragma unroll
+    for (int n = 0; n < (1 << (I - 1)); n += 2) {
+      S5.add(v[n]);
+      S5b.add(v[n + 1]);
+    }
   }
-  o.s1 = S1.value();
+  o.s1 = f0;
   o.s2 = S2.value();
   o.s3 = S3.value();
-  o.s4 = S4.value();
-  o.s5 = S5.value();
+  o.s4 = S4.value(S4b);
+  o.s5 = S5.value(S5b);
   o.f0 = f0;
   o.dbest = dbest;
   o.kbest = kbest;

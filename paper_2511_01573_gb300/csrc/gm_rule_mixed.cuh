@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kRuleBlock) k_rule_mixed_reg(const RuleArgs A)
   if (r >= A.n) return;
   RegionSums o;
   region_mixed_walk<FAM, D>(
-      *P, [&](int row, int j) -> float { return xt[(row * d + j) * RB + g]; }, A.R.ratio, o);
+      *P, [&](int row, int j) -> float& { return xt[(row * d + j) * RB + g]; }, A.R.ratio, o);
   region_finish64(
       o, d, A.R.w7, A.R.w5, A.R.estimator ? A.R.nw : nullptr, A.R.vol_omega,
       [&](int k) { return A.c[(int64_t)k * A.ld + r]; },
