@@ -18,17 +18,17 @@
 // lanes of a region taking rows l, l + L, ...  Butterflies, then a fixed
 // order over the warps, combine the lanes' sums.
 //
-// Bound: the FP64 pipe.  Integrands that are products of one factor per axis
-// (gm_factor64.cuh) hold wK e for the 15 nodes of every axis, relative to
-// the centre's value; a row is the product of its digits' entries, and each
-// node costs two fused multiply-adds (its terms of I_K and of E_0), about 20
-// fewer FP64 instructions than an evaluation of f with its weights.  Row sums
+// Bound: the FP64 pipe with f evaluated at every node, ~25 instructions a node.
+// Integrands that are products of one factor per axis (gm_factor64.cuh) hold
+// wK e for the 15 nodes of every axis, relative to the centre's value; a row is
+// the product of its digits' entries, and each node two products (its terms of
+// I_K and of E_0), three integer multiply-adds each.  Row sums
 // give the E_k of the other axes.  The nodes of I_G are the 7^d with odd
 // digits; they are walked on their own, because a lane that skips the term
 // saves nothing when another lane of its warp needs it.  f >= 0 for these
 // integrands, so sum |wK f| is I_K's sum.  d = 4, C0, 2500 regions: 6.57 ->
-// 0.71 ms.  Other integrands, and regions whose factors lack exponent room,
-// evaluate f at every node.
+// 0.26 ms (0.71 with FP64 products).  Other integrands, and regions whose
+// factors lack exponent room, evaluate f at every node.
 #pragma once
 
 #include "gm_factor64.cuh"
@@ -138,43 +138,60 @@ __device__ __forceinline__ void gk_sums_nodes(const SmemParams<double>& P, const
   }
 }
 
-// The same from per-axis factors, relative to F.  kt, gt: wK e and wG e
-// [d][15]; rt: r wK e of axis 0 [15].
+// The same from per-axis factors, relative to F.  kt, rt: wK e [d][15] and r wK e
+// of axis 0 [15] as limbs (gm_factor64.cuh) below 2^E[k] and 2^(E[0] + 1); gt: wG
+// e [d][15].  A row's product of limbs and the node products and sums run on
+// the integer pipes; a row leaves the FP64 pipe its sum's conversion and the
+// E_k of the other axes.
 template <int W>
 __device__ __forceinline__ void gk_sums_factors(const GkConst& K, int d, int lane,
                                                 const double* kt, const double* gt,
-                                                const double* rt, GkSums& s) {
+                                                const double* rt, const int* E, GkSums& s) {
   constexpr int L = 32 * W;
-  int rows = 1, grows = 1;
+  int rows = 1, grows = 1, Er = 0;
   for (int k = 1; k < d; ++k) {
     rows *= 15;
     grows *= 7;
+    Er += E[k];
   }
+  LimbSum sk, se;
+  LimbAcc e0;
+  int run = 0;
   for (int row = lane; row < rows; row += L) {
     int q = row;
-    double kr = 1.0;
+    Limbs kr{1 << 26, 0};
     int dig[GMQ_GK_MAX_DIM];
 #pragma unroll
     for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) {
       if (k < d) {
         dig[k] = q % 15;
         q /= 15;
-        const double v = kt[k * 15 + dig[k]];
-        kr = k == 1 ? v : __dmul_rn(kr, v);
+        const Limbs v = limbs_unpack(kt[k * 15 + dig[k]]);
+        kr = k == 1 ? v : LimbAcc::product(kr, v);
       }
     }
-    double rk = __dmul_rn(kt[0], kr), e0 = __dmul_rn(rt[0], kr);
+    LimbAcc rk;
 #pragma unroll
-    for (int j = 1; j < 15; ++j) {
-      rk = fma(kt[j], kr, rk);
-      e0 = fma(rt[j], kr, e0);
+    for (int j = 0; j < 15; ++j) {
+      rk.add(limbs_unpack(kt[j]), kr);
+      e0.add(limbs_unpack(rt[j]), kr);
     }
-    s.K = __dadd_rn(s.K, rk);
-    s.E[0] = __dadd_rn(s.E[0], e0);
+    const double v = (double)rk.number();
 #pragma unroll
     for (int k = 1; k < GMQ_GK_MAX_DIM; ++k)
-      if (k < d) s.E[k] = fma(K.r[dig[k]], rk, s.E[k]);
+      if (k < d) s.E[k] = fma(K.r[dig[k]], v, s.E[k]);
+    sk.take(rk);
+    if ((run += 15) > kLimbRun - 15) {
+      se.take(e0);
+      run = 0;
+    }
   }
+  se.take(e0);
+  s.K = sk.value(E[0] + Er);
+  s.E[0] = se.value(E[0] + 1 + Er);
+  const double unit = __hiloint2double((970 + E[0] + Er) << 20, 0);  // 2^(E0 + Er - 53)
+#pragma unroll
+  for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) s.E[k] = __dmul_rn(unit, s.E[k]);
   for (int row = lane; row < grows; row += L) {
     int q = row;
     double gr = 1.0;
@@ -207,6 +224,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
   __shared__ double xs[RB][GMQ_GK_MAX_DIM * L];      // each lane's current node
   __shared__ double ft[RB][kFactors ? 2 * NT + 15 : 1];
   __shared__ int room[RB][GMQ_GK_MAX_DIM];
+  __shared__ int bound[RB][GMQ_GK_MAX_DIM];  // high word of the axis' largest wK e, then its bound
   __shared__ double scratch[W * (3 + GMQ_GK_MAX_DIM)];
   const RuleArgs& A = G.A;
   const int d = A.P.d;
@@ -218,7 +236,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
     P.b[j] = A.P.b[j];
   }
   if (tid == 0) P.c0 = A.P.c0;
-  if (lane < GMQ_GK_MAX_DIM) room[w][lane] = 0;
+  if (lane < GMQ_GK_MAX_DIM) room[w][lane] = bound[w][lane] = 0;
   __syncthreads();
   const int64_t r = (int64_t)blockIdx.x * RB + w;
   const bool active = r < A.n;
@@ -239,11 +257,21 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
         }
         const double ke = __dmul_rn(K.wk[j], e);
         kt[q] = ke;
+        atomicMax(&bound[w][k], __double2hiint(ke));
         gt[q] = __dmul_rn(K.wg[j], e);
         if (k == 0) rt[j] = __dmul_rn(K.r[j], ke);
       }
     }
   __syncthreads();
+  if constexpr (kFactors) {
+    if (active && lane < d) bound[w][lane] = exp_bound(__hiloint2double(bound[w][lane], 0));
+    __syncthreads();
+    if (active) {
+      for (int q = lane; q < d * 15; q += L) kt[q] = limbs_of(kt[q], bound[w][q / 15]);
+      for (int j = lane; j < 15; j += L) rt[j] = limbs_of(rt[j], bound[w][0] + 1);
+    }
+    __syncthreads();
+  }
   if (!active) return;  // the whole warp (W = 1): its lanes share the region
   GkSums s;
 #pragma unroll
@@ -261,7 +289,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
     F = top.value(d);
     factors = big <= kFacExpRoom && exp_magnitude(F) <= kFacExpRoom;
     if (factors)
-      gk_sums_factors<W>(K, d, lane, kt, gt, rt, s);
+      gk_sums_factors<W>(K, d, lane, kt, gt, rt, bound[w], s);
     else
       F = 1.0;
   }
