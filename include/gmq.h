@@ -139,7 +139,7 @@ typedef struct gmq_options {
   int32_t lanes;       /* threads per region in the rule kernel: 0 = chosen
                           per sweep by the library, else 1, 4, 32 or (FP64
                           only) 128.  FP64 results do not depend on it
-                          (every class sum is one fixed tree); mixed-
+                          (class sums are exact or one fixed tree); mixed-
                           precision results do, at FP32 rounding level      */
   int32_t flags;       /* 0, or GMQ_KEEP_PARTITION                           */
   int32_t rule;        /* gmq_rule (GMQ_RULE_GENZ_MALIK by default)          */
@@ -200,13 +200,15 @@ gmq_status gmq_set_pool(gmq_context *ctx, void *dev_ptr, size_t bytes);
  * rule applies f at every node).  Every built-in family is f = g(S), S a
  * chain of per-axis terms phi_j(x_j) combined by + (by * for the product
  * peak), and a node takes each coordinate from one of seven values per axis:
- *   GMQ_EVAL_SEPARABLE (default): phi at the 7d coordinate values once per
- *     region; each node's S from one or two combines of per-axis terms and
- *     partial chains; g at every node;
+ *   GMQ_EVAL_SEPARABLE (default): the axes' terms at the 7d coordinate values
+ *     once per region; each node's value as a product of per-axis factors (the
+ *     exponentials, the cosine and the product peak), from a fixed-point inner
+ *     sum (the corner peak), or as g of one or two combines of per-axis terms
+ *     (the polynomial, and regions whose factors or sums lack exponent room);
  *   GMQ_EVAL_NODEWISE: f from each node's coordinates (d operations for S,
  *     then g), as an integrand without that form would be evaluated.
  * Both give every lane mapping the same bits; they differ from each other
- * only in the rounding order of S.  gmq_rule_grad follows it too: the
+ * only in rounding.  gmq_rule_grad follows it too: the
  * separable mode forms the gradient from per-axis, per-coordinate sums of
  * w g'(S) over the nodes, the node-wise mode differentiates f at every
  * node.  The mixed precision, the Gauss-Kronrod rule and the batched form

@@ -127,14 +127,25 @@ struct Fac<GMQ_OSCILLATORY> {
   }
 };
 
-static __device__ __noinline__ double exp_any(double x) { return gm_exp(x); }
+// (per argument, so that a factor does not depend on which others it is formed with)
+static __device__ __noinline__ double exp_any(double x, i64 low) {
+  return exp_near(x) ? exp_fixed(to_fixed(x, 58) + low) : gm_exp(x);
+}
 static __device__ __noinline__ double rcp_any(double x) { return gm_rcp(x); }
 
 // N factors from their arguments.  The fast forms' range is tested once for
 // all, so that their instructions interleave (a test for each kept the six
 // exponentials of an axis one after the other).
-template <int FAM, int N>
-__device__ __forceinline__ void factors(const double (&z)[N], double fc, double (&e)[N]) {
+// The arguments of C0 and the discontinuous family refer to the rounded fc; its
+// rounding error (low, in fixed point) is added to them, as it is to F's.
+template <int FAM, class PT>
+__device__ __forceinline__ i64 low_fixed(const PT& P, int k, double c, double fc) {
+  return to_fixed(Fac<FAM>::low(P, k, c, fc), 58);
+}
+
+template <int FAM, class PT, int N>
+__device__ __forceinline__ void factors(const PT& P, int k, double c, const double (&z)[N],
+                                        double fc, double (&e)[N]) {
   bool near = true;
   if constexpr (Sep<FAM>::kMul) {
 #pragma unroll
@@ -149,13 +160,16 @@ __device__ __forceinline__ void factors(const double (&z)[N], double fc, double 
   } else {
 #pragma unroll
     for (int i = 0; i < N; ++i) near = near && exp_near(z[i]);
+    i64 low = 0;
+    if constexpr (FAM == GMQ_C0) low = low_fixed<FAM>(P, k, c, fc);
+    if constexpr (FAM == GMQ_DISCONTINUOUS) low = -low_fixed<FAM>(P, k, c, fc);
     if (near) {
 #pragma unroll
-      for (int i = 0; i < N; ++i) e[i] = exp_fixed(to_fixed(z[i], 58));
+      for (int i = 0; i < N; ++i) e[i] = exp_fixed(to_fixed(z[i], 58) + low);
       return;
     }
 #pragma unroll
-    for (int i = 0; i < N; ++i) e[i] = exp_any(z[i]);
+    for (int i = 0; i < N; ++i) e[i] = exp_any(z[i], low);
   }
 }
 
@@ -167,7 +181,7 @@ __device__ __forceinline__ void axis_factors(const PT& P, int k, double c, doubl
   const double z[6] = {Fac<FAM>::arg(P, k, c, h, fc, lam2), Fac<FAM>::arg(P, k, c, h, fc, -lam2),
                        Fac<FAM>::arg(P, k, c, h, fc, lam3), Fac<FAM>::arg(P, k, c, h, fc, -lam3),
                        Fac<FAM>::arg(P, k, c, h, fc, lam5), Fac<FAM>::arg(P, k, c, h, fc, -lam5)};
-  factors<FAM>(z, fc, e);
+  factors<FAM>(P, k, c, z, fc, e);
 }
 
 template <int FAM, class PT>
@@ -175,7 +189,7 @@ __device__ __forceinline__ double one_factor(const PT& P, int k, double c, doubl
                                              double lam) {
   const double z[1] = {Fac<FAM>::arg(P, k, c, h, fc, lam)};
   double e[1];
-  factors<FAM>(z, fc, e);
+  factors<FAM>(P, k, c, z, fc, e);
   return e[0];
 }
 
@@ -207,7 +221,7 @@ struct Centre {
         S = __dadd_rn(S, fc);
       }
       take(fc);
-      v += to_fixed(Fac<FAM>::low(P, k, c, fc), 58);
+      v += low_fixed<FAM>(P, k, c, fc);
     }
   }
   __device__ __forceinline__ void take(double x) {

@@ -1,8 +1,10 @@
 // gm_region64.cuh -- FP64 evaluation of one region by a group of T lanes
 // (T in {1, 4, 32, 128}: a thread, four lanes, a warp or a 128-thread block
-// per region), shared by the single-integral rule kernel (gm_rule.cuh)
-// and the batched rule kernel (gm_batch.cu): both compute every region with
-// the same operations in the same order.
+// per region): the separable form, which the rule kernels use for integrands
+// and regions that gm_factor64.cuh and gm_fixed64.cuh do not take, the
+// node-wise form, and the epilogue of all.  Shared by the single-integral rule
+// kernel (gm_rule.cuh) and the batched rule kernel (gm_batch.cu): both compute
+// every region with the same operations in the same order.
 //
 // What is computed (paper Sec. 2, the Genz-Malik degree-7 rule with its
 // embedded degree-5 rule): the five class sums S1..S5 of f over the fully

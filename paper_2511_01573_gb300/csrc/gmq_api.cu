@@ -57,6 +57,7 @@ struct gmq_context {
   char* scratch = nullptr;
   size_t scratch_bytes = 0;
   DevStatus* h_status = nullptr;  // pinned, large enough for a BatchState too
+  DevStatus* h_status_dev = nullptr;  // the device's address of it
   cudaEvent_t status_ev = nullptr;  // a sweep's status has reached h_status
   std::vector<gmq_sweep> trace;
   int64_t launches = 0;
@@ -753,11 +754,12 @@ gmq_status gmq_create(gmq_context** out, int device, size_t pool_bytes_hint) {
   // pinned status buffer: one sweep's DevStatus, or a batch's BatchState
   constexpr size_t kHostStatusBytes =
       sizeof(DevStatus) > sizeof(BatchState) ? sizeof(DevStatus) : sizeof(BatchState);
-  if (cudaHostAlloc((void**)&ctx->h_status, kHostStatusBytes, cudaHostAllocDefault) != cudaSuccess) {
+  if (cudaHostAlloc((void**)&ctx->h_status, kHostStatusBytes, cudaHostAllocMapped) != cudaSuccess) {
     delete ctx;
     return GMQ_ERR_CUDA;
   }
-  if (cudaEventCreateWithFlags(&ctx->status_ev, cudaEventDisableTiming) != cudaSuccess) {
+  if (cudaHostGetDevicePointer((void**)&ctx->h_status_dev, ctx->h_status, 0) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ctx->status_ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaFreeHost(ctx->h_status);
     delete ctx;
     return GMQ_ERR_CUDA;
@@ -947,7 +949,7 @@ gmq_status gmq_integrate(gmq_context* ctx, const gmq_problem* prob, const gmq_op
   PA.c_out = cA;
   PA.h_out = hA;
   PA.ld = L.ld;
-  GMQ_CK(cudaMemsetAsync(st, 0, sizeof(DevStatus), strm));
+  PA.st = st;
   prof_begin(ctx, kKPartition);
   GMQ_CK(launch_partition(PA, strm));
   prof_end(ctx, kKPartition, n);
@@ -1016,15 +1018,15 @@ gmq_status gmq_integrate(gmq_context* ctx, const gmq_problem* prob, const gmq_op
     S.ld_leaf = L.ld;
     S.leaf_cap = cap;
     S.st = st;
+    S.host = ctx->h_status_dev;
     prof_begin(ctx, kKSum);
     GMQ_CK(launch_sum_status(S, strm));
     prof_end(ctx, kKSum, n);
     prof_begin(ctx, kKClassify);
     GMQ_CK(launch_classify(S, strm));
     prof_end(ctx, kKClassify, n);
-    // the split does not change the status: the host reads it and prepares the
-    // next sweep while the split still runs
-    GMQ_CK(cudaMemcpyAsync(ctx->h_status, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, strm));
+    // the split does not change the status, which is in the host's memory by
+    // now: the host reads it and prepares the next sweep while the split runs
     GMQ_CK(cudaEventRecord(ctx->status_ev, strm));
     prof_begin(ctx, kKSplit);
     GMQ_CK(launch_split(S, strm));
@@ -1308,6 +1310,7 @@ gmq_status gmq_classify_split(gmq_context* ctx, int32_t dim, int64_t n, const do
   S.budget_val = budget;
   S.guard = kGuardFp64;
   S.st = X.st;
+  S.host = ctx->h_status_dev;
   cudaStream_t strm = ctx->stream;
   GMQ_CK(cudaMemsetAsync(X.st, 0, sizeof(DevStatus), strm));
   prof_begin(ctx, kKClassify);
@@ -1317,7 +1320,6 @@ gmq_status gmq_classify_split(gmq_context* ctx, int32_t dim, int64_t n, const do
   GMQ_CK(launch_split(S, strm));
   prof_end(ctx, kKSplit, n);
   ctx->launches += 2;
-  GMQ_CK(cudaMemcpyAsync(ctx->h_status, X.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, strm));
   GMQ_CK(cudaStreamSynchronize(strm));
   prof_collect(ctx);
   const DevStatus h = *ctx->h_status;

@@ -112,6 +112,7 @@ struct SweepArgs {
   int64_t ld_leaf;
   int64_t leaf_cap;
   DevStatus* st;
+  DevStatus* host;         // the device's view of the host's status, or null
 };
 
 // Pairwise-tree sum over the threads of a block, one value per thread,

@@ -202,6 +202,10 @@ __global__ void __launch_bounds__(kQuad) k_sum_status(const SweepArgs S) {
     else if (S.last_sweep)
       f |= kLastSweep | kDone;
     st->flags = f;
+    // a stopped loop's status is final; otherwise k_classify completes it.  The
+    // kernel that completes it writes the host's copy: a copy node of its own
+    // costs the sweep 2 to 3 us
+    if ((f & kDone) && S.host) *S.host = *st;
   }
 }
 
@@ -301,6 +305,7 @@ __global__ void __launch_bounds__(kQuad) k_classify(const SweepArgs S) {
       }
     }
     st->flags = f;
+    if (S.host) *S.host = *st;
   }
 }
 
@@ -372,6 +377,7 @@ __global__ void __launch_bounds__(kQuad) k_split(const SweepArgs S) {
 __global__ void k_partition(const PartArgs P) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= P.n) return;
+  if (q == 0 && P.st) *P.st = DevStatus{};
   int64_t rem = q;
   for (int k = 0; k < P.d; ++k) {
     const int64_t i = rem % P.s;

@@ -15,6 +15,7 @@ struct PartArgs {
   double* c_out;
   double* h_out;
   int64_t ld;
+  DevStatus* st;  // status to clear, or null
 };
 
 cudaError_t launch_sum_status(const SweepArgs& S, cudaStream_t s);
