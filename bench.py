@@ -116,7 +116,7 @@ RULE_EXEC_FP64_FLOPS_D8 = {0: 526.0, 1: 802.0, 2: 231.0, 3: 443.0, 4: 433.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "65d03437758577ae"
+RULE_COUNTS_SHA16 = "6ae9366f23930517"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -130,7 +130,7 @@ RULE_COUNTS_SHA16 = "65d03437758577ae"
 MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "c53349b5712a45ee"
+MIXED_COUNTS_SHA16 = "1d4c067d54e444a7"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):
