@@ -15,10 +15,10 @@
 // rotations (cos Delta, sin Delta), two products per node.  Exponentials, sines
 // and class sums run in fixed point on the integer pipes (gmq_families.cuh,
 // Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
-// the outer function at every node: C0 8.14 -> 0.98 ms (4080 -> 328 FP64
+// the outer function at every node: C0 8.14 -> 0.96 ms (4080 -> 278 FP64
 // instructions a region), Gaussian 8.25 -> 1.03, product peak 4.71 -> 1.12,
 // cosine 10.99 -> 1.40; with factors and FP64 sums and functions they took 2.23,
-// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-82 % active) is the
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-81 % active) is the
 // coordinates, the chains and the weights; twelve warps an SM, as many as the
 // workspaces in shared memory let.
 //
@@ -55,55 +55,125 @@ struct Fac {
   static constexpr int kind = kNone;
 };
 
-// The factor of coordinate c + lam h on axis j relative to the centre's, whose
-// phi is fc, is the exponential of (for the product peak fc over) arg(P, j, c,
-// h, fc, lam).  low(P, j, c, fc): the rounding error of fc.  Coordinates enter as differences from the centre where f is continuous:
-// fewer operations, and no rounding of c + lam h in between.
+// Relative to the centre's, the factor of coordinate c + lam h on axis j is, for
+// the product peak, fc over arg(P, j, c, h, lam); for the others, whose phi at the
+// centre is fc, it is the exponential of a difference z(lam), |lam| < 1, which is
+// formed in fixed point: rounded relative to its own size it would put a factor
+// far from 1 (and the F that makes up for it) further from f than the node's own
+// inner sum, small where f is large, does.  terms<q>: what z takes from the axis,
+// in units of 2^-q (m) and 2^-(q+1) (lin, quad), each an FP64 value and its
+// rounding error (low: that of fc); z<q>(x, l): z in units of 2^-q, l = |lam|
+// 2^63, neg: lam < 0.  size: the two values whose size limits q.
+// Differences c - u enter as they are rounded: no rounding of c + lam h.
+struct FacTerms {
+  i64 m, lin, quad;
+  bool neg, aneg;  // c < u, a < 0 (the kink)
+};
+
+// a l 2^-64 for 0 <= l < 2^63; within 1 unit for q = 54, 3 for q = 58
+template <int q>
+__device__ __forceinline__ i64 lam_mul(i64 a, u64 l) {
+  if constexpr (q < 58) return __mul64hi(a, (i64)l);
+  return fixed_mul_signed(a, l);
+}
+template <int q>
+__device__ __forceinline__ i64 to_fixed2(double hi, double lo) {
+  return to_fixed(hi, q) + to_fixed(lo, q);
+}
+
+// z = a |t| - a |t + lam h|
 template <>
 struct Fac<GMQ_C0> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
-                                               double lam) {
-    const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
-    return fma(-P.a[j], fabs(t), fc);
-  }
-  template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
     return fma(P.a[j], fabs(__dsub_rn(c, P.u[j])), -fc);
   }
+  template <class PT>
+  __device__ __forceinline__ static void size(const PT& P, int j, double, double h, double fc,
+                                              double& x, double& y) {
+    x = fc;
+    y = __dmul_rn(P.a[j], h);
+  }
+  template <int q, class PT>
+  __device__ __forceinline__ static FacTerms terms(const PT& P, int j, double c, double h,
+                                                   double fc) {
+    FacTerms t;
+    const double ah = __dmul_rn(P.a[j], h);
+    t.m = to_fixed2<q>(fc, low(P, j, c, fc));
+    t.lin = to_fixed2<q + 1>(ah, fma(P.a[j], h, -ah));
+    t.neg = __double2hiint(__dsub_rn(c, P.u[j])) < 0;
+    t.aneg = __double2hiint(P.a[j]) < 0;
+    return t;
+  }
+  template <int q>
+  __device__ __forceinline__ static i64 z(const FacTerms& t, u64 l, bool neg) {
+    const i64 g = lam_mul<q>(t.lin, l);
+    i64 v = (t.neg ? -t.m : t.m) + (neg ? -g : g);  // a (t + lam h)
+    if ((v < 0) != t.aneg) v = -v;                  // a |t + lam h|
+    return t.m - v;
+  }
 };
 
-// b ((t + lam h)^2 - t^2) = lam^2 b h^2 + lam 2 b h t, t = c - u
+// z = -b ((t + lam h)^2 - t^2) = -(lam 2 b h t + lam^2 b h^2), t = c - u
 template <>
 struct Fac<GMQ_GAUSSIAN> {
   static constexpr int kind = kReal;
-  template <class PT>
-  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double,
-                                               double lam) {
-    const double t = __dsub_rn(c, P.u[j]);
-    const double bh = __dmul_rn(P.b[j], h);
-    const double q = __dmul_rn(__dadd_rn(t, t), bh);
-    return fma(-lam, q, -__dmul_rn(__dmul_rn(lam, lam), __dmul_rn(bh, h)));
-  }
   template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
     const double t = __dsub_rn(c, P.u[j]), t2 = __dmul_rn(t, t);
     return fma(P.b[j], fma(t, t, -t2), fma(P.b[j], t2, -fc));
   }
+  template <class PT>
+  __device__ __forceinline__ static void size(const PT& P, int j, double c, double h, double,
+                                              double& x, double& y) {
+    const double t = __dsub_rn(c, P.u[j]), bh = __dmul_rn(P.b[j], h);
+    x = __dmul_rn(__dadd_rn(t, t), bh);
+    y = __dmul_rn(bh, h);
+  }
+  template <int q, class PT>
+  __device__ __forceinline__ static FacTerms terms(const PT& P, int j, double c, double h,
+                                                   double) {
+    FacTerms t;
+    const double t1 = __dsub_rn(c, P.u[j]), tt = __dadd_rn(t1, t1);
+    const double bh = __dmul_rn(P.b[j], h), bl = fma(P.b[j], h, -bh);
+    const double x = __dmul_rn(tt, bh), y = __dmul_rn(bh, h);
+    t.lin = to_fixed2<q + 1>(x, fma(tt, bl, fma(tt, bh, -x)));
+    t.quad = to_fixed2<q + 1>(y, fma(bl, h, fma(bh, h, -y)));
+    return t;
+  }
+  template <int q>
+  __device__ __forceinline__ static i64 z(const FacTerms& t, u64 l, bool neg) {
+    const i64 g = lam_mul<q>(t.lin, l);
+    const i64 s = lam_mul<q>(t.quad, (u64)__umul64hi(l, l) << 1);
+    return (neg ? g : -g) - s;
+  }
 };
 
+// z = lam a h
 template <>
 struct Fac<GMQ_DISCONTINUOUS> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
-                                               double lam) {
-    return fma(P.a[j], fma(lam, h, c), -fc);
-  }
-  template <class PT>
   __device__ __forceinline__ static double low(const PT& P, int j, double c, double fc) {
     return fma(P.a[j], c, -fc);
+  }
+  template <class PT>
+  __device__ __forceinline__ static void size(const PT& P, int j, double, double h, double,
+                                              double& x, double& y) {
+    x = y = __dmul_rn(P.a[j], h);
+  }
+  template <int q, class PT>
+  __device__ __forceinline__ static FacTerms terms(const PT& P, int j, double, double h, double) {
+    FacTerms t;
+    const double ah = __dmul_rn(P.a[j], h);
+    t.lin = to_fixed2<q + 1>(ah, fma(P.a[j], h, -ah));
+    return t;
+  }
+  template <int q>
+  __device__ __forceinline__ static i64 z(const FacTerms& t, u64 l, bool neg) {
+    const i64 g = lam_mul<q>(t.lin, l);
+    return neg ? -g : g;
   }
 };
 
@@ -111,7 +181,7 @@ template <>
 struct Fac<GMQ_PRODUCT_PEAK> {
   static constexpr int kind = kReal;
   template <class PT>
-  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h, double fc,
+  __device__ __forceinline__ static double arg(const PT& P, int j, double c, double h,
                                                double lam) {
     const double t = fma(lam, h, __dsub_rn(c, P.u[j]));
     return fma(t, t, P.b[j]);
@@ -127,29 +197,52 @@ struct Fac<GMQ_OSCILLATORY> {
   }
 };
 
-// (per argument, so that a factor does not depend on which others it is formed with)
-static __device__ __noinline__ double exp_any(double x, i64 low) {
-  return exp_near(x) ? exp_fixed(to_fixed(x, 58) + low) : gm_exp(x);
-}
 static __device__ __noinline__ double rcp_any(double x) { return gm_rcp(x); }
 
-// N factors from their arguments.  The fast forms' range is tested once for
-// all, so that their instructions interleave (a test for each kept the six
-// exponentials of an axis one after the other).
-// The arguments of C0 and the discontinuous family refer to the rounded fc; its
-// rounding error (low, in fixed point) is added to them, as it is to F's.
 template <int FAM, class PT>
 __device__ __forceinline__ i64 low_fixed(const PT& P, int k, double c, double fc) {
   return to_fixed(Fac<FAM>::low(P, k, c, fc), 58);
 }
 
+// |lam| in units of 2^-63
+__device__ __forceinline__ u64 lam_fixed(double lam) { return (u64)to_fixed(fabs(lam), 63); }
+
+// z and exp(z) of one factor whose terms are not below 16: in units of 2^-54 while
+// they are below 256 (|z| < 512), in FP64 from the coordinate above (such a factor
+// has no exponent room, and only its size matters).
+template <int FAM, class PT>
+static __device__ __noinline__ double factor_far(const PT& P, int k, double c, double h, double fc,
+                                                 double lam, bool wide) {
+  using F = Fac<FAM>;
+  if (wide) {
+    const i64 z = F::template z<54>(F::template terms<54>(P, k, c, h, fc), lam_fixed(lam),
+                                    __double2hiint(lam) < 0);
+    return exp_wide(z << 4, round_shifted(z));
+  }
+  const double p = Sep<FAM>::phi(P, k, fma(lam, h, c));
+  return gm_exp(FAM == GMQ_DISCONTINUOUS ? __dsub_rn(p, fc) : __dsub_rn(fc, p));
+}
+// |x| < 256, tested on the high word
+__device__ __forceinline__ bool below_256(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x40700000u;
+}
+
+// The factors of N coordinates c + lam[i] h.  Which form they take is decided
+// for the axis, not for a factor: one test, so that the instructions of N
+// exponentials interleave (a test for each kept them one after the other), and a
+// factor does not depend on which others it is formed with.
 template <int FAM, class PT, int N>
-__device__ __forceinline__ void factors(const PT& P, int k, double c, const double (&z)[N],
-                                        double fc, double (&e)[N]) {
-  bool near = true;
+__device__ __forceinline__ void factors(const PT& P, int k, double c, double h, double fc,
+                                        const double (&lam)[N], double (&e)[N]) {
+  using F = Fac<FAM>;
   if constexpr (Sep<FAM>::kMul) {
+    double z[N];
+    bool near = true;
 #pragma unroll
-    for (int i = 0; i < N; ++i) near = near && rcp_near(z[i]);
+    for (int i = 0; i < N; ++i) {
+      z[i] = F::arg(P, k, c, h, lam[i]);
+      near = near && rcp_near(z[i]);
+    }
     if (near) {
 #pragma unroll
       for (int i = 0; i < N; ++i) e[i] = __dmul_rn(fc, rcp_refined(z[i]));
@@ -158,18 +251,18 @@ __device__ __forceinline__ void factors(const PT& P, int k, double c, const doub
 #pragma unroll
     for (int i = 0; i < N; ++i) e[i] = __dmul_rn(fc, rcp_any(z[i]));
   } else {
+    double x, y;
+    F::size(P, k, c, h, fc, x, y);
+    if (sincos_near(x) && sincos_near(y)) {  // both below 16: |z| < 31
+      const FacTerms t = F::template terms<58>(P, k, c, h, fc);
 #pragma unroll
-    for (int i = 0; i < N; ++i) near = near && exp_near(z[i]);
-    i64 low = 0;
-    if constexpr (FAM == GMQ_C0) low = low_fixed<FAM>(P, k, c, fc);
-    if constexpr (FAM == GMQ_DISCONTINUOUS) low = -low_fixed<FAM>(P, k, c, fc);
-    if (near) {
-#pragma unroll
-      for (int i = 0; i < N; ++i) e[i] = exp_fixed(to_fixed(z[i], 58) + low);
+      for (int i = 0; i < N; ++i)
+        e[i] = exp_fixed(F::template z<58>(t, lam_fixed(lam[i]), __double2hiint(lam[i]) < 0));
       return;
     }
-#pragma unroll
-    for (int i = 0; i < N; ++i) e[i] = exp_any(z[i], low);
+    const bool wide = below_256(x) && below_256(y);
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) e[i] = factor_far<FAM>(P, k, c, h, fc, lam[i], wide);
   }
 }
 
@@ -178,25 +271,24 @@ template <int FAM, class PT>
 __device__ __forceinline__ void axis_factors(const PT& P, int k, double c, double h, double fc,
                                              double lam2, double lam3, double lam5,
                                              double (&e)[6]) {
-  const double z[6] = {Fac<FAM>::arg(P, k, c, h, fc, lam2), Fac<FAM>::arg(P, k, c, h, fc, -lam2),
-                       Fac<FAM>::arg(P, k, c, h, fc, lam3), Fac<FAM>::arg(P, k, c, h, fc, -lam3),
-                       Fac<FAM>::arg(P, k, c, h, fc, lam5), Fac<FAM>::arg(P, k, c, h, fc, -lam5)};
-  factors<FAM>(P, k, c, z, fc, e);
+  const double lam[6] = {lam2, -lam2, lam3, -lam3, lam5, -lam5};
+  factors<FAM>(P, k, c, h, fc, lam, e);
 }
 
 template <int FAM, class PT>
 __device__ __forceinline__ double one_factor(const PT& P, int k, double c, double h, double fc,
                                              double lam) {
-  const double z[1] = {Fac<FAM>::arg(P, k, c, h, fc, lam)};
+  const double l[1] = {lam};
   double e[1];
-  factors<FAM>(P, k, c, z, fc, e);
+  factors<FAM>(P, k, c, h, fc, l, e);
   return e[0];
 }
 
 // F = f(centre) from the axes' phi in order.  Its error is common to every
-// node, so the inner sum is kept to 2^-58 in fixed point, roundings of phi
-// included (for |S| < 16 and every |phi| < 16; in FP64 otherwise), and the
-// product peak's product as a sum of two doubles.
+// node, so the inner sum is kept in units of 2^-58, roundings of phi included, as
+// a 64-bit integer modulo 2^64 (for |S| < 512 and every |phi| < 512, where the
+// rounded S tells the multiple of 64; in FP64 otherwise; the cosine's below 16),
+// and the product peak's product as a sum of two doubles.
 template <int FAM>
 struct Centre {
   double S, lo = 0.0;
@@ -228,18 +320,23 @@ struct Centre {
     v += to_fixed(x, 58);
     fixed = fixed && small(x);
   }
-  __device__ __forceinline__ static bool small(double x) { return sincos_near(x); }  // |x| < 16
+  __device__ __forceinline__ static bool small(double x) {  // |x| < 512
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x40800000u;
+  }
   __device__ __forceinline__ double value(int d) const {
     if constexpr (Sep<FAM>::kMul) {
       const double r = Sep<FAM>::g(d, S);
       return fma(-__dmul_rn(r, lo), r, r);
     } else {
       if (!fixed || !small(S)) return Sep<FAM>::g(d, S);
-      return exp_fixed(FAM == GMQ_DISCONTINUOUS ? v : -v);
+      const i64 x = FAM == GMQ_DISCONTINUOUS ? v : -v;
+      if (sincos_near(S)) return exp_fixed(x);  // |S| < 16
+      const int n = round_mul_int(S, 1.44269504f);
+      return exp_wide(x, FAM == GMQ_DISCONTINUOUS ? n : -n);
     }
   }
   __device__ __forceinline__ void sincos(double& sn, double& cs) const {
-    if (!fixed || !small(S))
+    if (!fixed || !sincos_near(S))
       gm_sincos(S, &sn, &cs);
     else
       sincos_fixed(v, &sn, &cs);

@@ -33,3 +33,88 @@ def test_cosine_factors_at_the_ends_of_the_reduction(gpu_ctx, lanes):
                            lanes=lanes)[0].cpu().numpy()
     err = np.abs((i7 * 2.0 ** 39).astype(LD) - np.cos(x.astype(LD)))
     assert np.max(err) <= 2.2 * EPS
+
+
+def _factor(fam, a, u, b, x):
+    """One axis' factor of f in long double (a scalar's worth of the family)."""
+    t = x - u
+    if fam == G.GAUSSIAN:
+        return np.exp(-b * t * t)
+    if fam == G.C0:
+        return np.exp(-a * np.abs(t))
+    if fam == G.PRODUCT_PEAK:
+        return 1 / (t * t + b)
+    return np.where(t > 0, LD(0), np.exp(a * x))
+
+
+def _exact_i7(fam, a, u, c, h):
+    """The degree-7 rule's value on one region and the sum of its terms'
+    magnitudes, unit volume, in long double: class sums of products of factors."""
+    d = len(a)
+    a, u, c, h = (np.asarray(v, dtype=LD) for v in (a, u, c, h))
+    b = (1 / (a * a) if fam == G.PRODUCT_PEAK else a * a).astype(np.float64).astype(LD)
+    l2, l3, l5 = (LD(np.sqrt(v)) for v in (9 / 70, 9 / 10, 9 / 19))
+    f = lambda lam: _factor(fam, a, u, b, c + lam * h)
+    f0 = f(LD(0))
+    p = [f(l) + f(-l) for l in (l2, l3, l5)]
+    others = [np.prod(np.delete(f0, k)) for k in range(d)]
+    s4 = LD(0)
+    for j in range(d):
+        for k in range(j + 1, d):
+            s4 += p[1][j] * p[1][k] * np.prod(np.delete(f0, [j, k]))
+    s = [np.prod(f0), sum(o * v for o, v in zip(others, p[0])),
+         sum(o * v for o, v in zip(others, p[1])), s4, np.prod(p[2])]
+    w = [LD(v) for v in (12824 - 9120 * d + 400 * d * d, 2940, 1820 - 400 * d, 200)]
+    w = [v / 19683 for v in w] + [LD(6859) / 19683 / 2 ** d]
+    return sum(x * y for x, y in zip(w, s)), sum(abs(x * y) for x, y in zip(w, s))
+
+
+def _cases(fam, d, n, lo, hi, whole, seed):
+    rng = np.random.default_rng(seed)
+    for _ in range(n):
+        a, u = rng.uniform(lo, hi, d), rng.uniform(0, 1, d)
+        if fam == G.DISCONTINUOUS:
+            u = 0.4 + 0.6 * u
+        x = rng.uniform(0, 1, (2, d))
+        c, h = 0.5 * (x[0] + x[1]), 0.5 * np.abs(x[0] - x[1])
+        if whole:
+            c, h = np.full(d, 0.5), np.full(d, 0.5)
+        yield a, u, c, h
+
+
+def _rms_errors(gpu_ctx, fam, cases, exact):
+    """rms over the cases of I7's error relative to its terms: the default form's
+    and the node-wise form's."""
+    from paper_2511_01573_gb300 import gmq
+    out = np.zeros(2)
+    n = 0
+    for a, u, c, h in cases:
+        ref, terms = exact(fam, a, u, c, h)
+        if terms == 0:
+            continue
+        vol = np.prod((2 * h).astype(LD))
+        for i, mode in enumerate((gmq.EVAL_SEPARABLE, gmq.EVAL_NODEWISE)):
+            gpu_ctx.set_eval_mode(mode)
+            try:
+                i7 = gpu_ctx.eval_rule(fam, a, u, _soa(c[None]), _soa(h[None]), lanes=32)[0]
+            finally:
+                gpu_ctx.set_eval_mode(gmq.EVAL_SEPARABLE)
+            out[i] += float((LD(i7.item()) / vol - ref) / terms) ** 2
+        n += 1
+    return np.sqrt(out / n)
+
+
+@pytest.mark.parametrize("whole", [False, True])
+@pytest.mark.parametrize("fam,lo,hi,d", [(G.C0, 4, 12, 4), (G.C0, 4, 12, 8), (G.C0, 20, 60, 8),
+                                         (G.C0, 0.5, 3, 5), (G.GAUSSIAN, 5, 15, 4),
+                                         (G.GAUSSIAN, 0.5, 3, 6), (G.GAUSSIAN, 5, 15, 8),
+                                         (G.DISCONTINUOUS, 5, 15, 6)])
+def test_steep_factors(gpu_ctx, fam, lo, hi, d, whole):
+    """Factors far from 1: the difference that a factor is the exponential of is
+    kept to 2^-57 (2^-53 where it is 15 and more), not rounded relative to its own
+    size, so that products of factors are as near as the node-wise form, which
+    rounds every node's inner sum, small where f is large: at most 1.25 of its
+    error, and half an eps for the products' own roundings."""
+    mine, node = _rms_errors(gpu_ctx, fam, _cases(fam, d, 48, lo, hi, whole, 11 * d + int(lo)),
+                             _exact_i7)
+    assert mine <= 1.25 * node + 0.5 * EPS
