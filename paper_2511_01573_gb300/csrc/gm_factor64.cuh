@@ -15,18 +15,20 @@
 // rotations (cos Delta, sin Delta), two products per node.  Exponentials, sines
 // and class sums run in fixed point on the integer pipes (gmq_families.cuh,
 // Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
-// the outer function at every node: C0 8.14 -> 0.96 ms (4080 -> 278 FP64
-// instructions a region), Gaussian 8.25 -> 1.03, product peak 4.71 -> 1.12,
+// the outer function at every node: C0 8.14 -> 0.97 ms (4080 -> 278 FP64
+// instructions a region), Gaussian 8.25 -> 1.04, product peak 4.71 -> 1.14,
 // cosine 10.99 -> 1.40; with factors and FP64 sums and functions they took 2.23,
-// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-81 % active) is the
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-80 % active) is the
 // coordinates, the chains and the weights; twelve warps an SM, as many as the
 // workspaces in shared memory let.
 //
 // Accuracy: F is a common factor of every node, so its error scales the
 // region's value and is not amplified by the rule's weights of both signs
 // (sum |w| is 5.8 at d = 8), and it is formed beyond FP64 (Centre); the factors
-// carry an error near 2^-53 each.  Against quad precision I7 is within 0.5 to 1.1
-// times, the error estimate within 0.1 to 1 times the separable form's error.
+// carry an error near 2^-53 each, whatever their size.  Against 113-bit arithmetic
+// (d = 2..16, slopes 0.5 to 300, random boxes and the whole domain) the rms error of
+// I7 is 0.15 to 1.2 times the separable form's, or, where both are below 2^-53 of
+// the terms, up to 1.9 times.
 // Factors may over- or underflow where f does not (a factor is relative to
 // the centre): regions whose factors' exponents do not leave room are
 // evaluated by region_sums64, decided from the region alone, so that every
@@ -446,10 +448,12 @@ __device__ __forceinline__ int factor_room(double e) {
 // is v 2^(53 - E) rounded, in two signed limbs h 2^27 + l (|h| <= 2^26, |l| <=
 // 2^26); 2^E bounds the table it comes from, so its error is at most 2^-54 of
 // the table's largest entry, an FP64 rounding of that entry.  A product is
-// h h' 2^54 + (h l' + l h') 2^27, three multiply-adds to 64 bits (12 cycles of
-// an SM quarter against 76 for an FP64 instruction); l l', below 2^-54 of the
-// largest product and of either sign, is left out.  Sums are exact integers:
-// no order of the nodes and no lane mapping changes a bit.
+// h h' 2^54 + (h l' + l h') 2^27 + l l'; the first two terms are three
+// multiply-adds to 64 bits (12 cycles of an SM quarter against 76 for an FP64
+// instruction), the third, up to 2^-54 of the largest product, is added for all
+// products of two tables at once (sum l times sum l': left out, 2^12 products
+// with a few large ones are 1e-15 off).  Sums are exact integers: no order of
+// the nodes and no lane mapping changes a bit.
 struct Limbs {
   int h, l;
 };
@@ -489,7 +493,15 @@ struct LimbAcc {
   // the sum as one number in units of 2^-53 of the products' bound, rounded (for
   // up to 64 products)
   __device__ __forceinline__ i64 number() const { return (hh << 1) + ((mid + (1 << 25)) >> 26); }
-  // a b as a number of the same kind
+  // a b as a number of the same kind; what was rounded off, in units of 2^-37 of
+  // its last place, is added to rest
+  __device__ __forceinline__ static Limbs product(Limbs a, Limbs b, i64& rest) {
+    LimbAcc r;
+    r.add(a, b);
+    const i64 up = (r.mid + (1 << 25)) >> 26;
+    rest += (((r.mid - (up << 26)) << 27) + (i64)a.l * b.l) >> 16;
+    return limbs_split((r.hh << 1) + up);
+  }
   __device__ __forceinline__ static Limbs product(Limbs a, Limbs b) {
     LimbAcc r;
     r.add(a, b);
@@ -510,6 +522,12 @@ struct LimbSum {
     add(a.mid >> 63, (u64)a.mid);
     a.hh = 0;
     a.mid = 0;
+  }
+  // x y 2^-k, 0 < k < 64
+  __device__ __forceinline__ void add_product(i64 x, i64 y, int k) {
+    const i64 h = __mul64hi(x, y);
+    const u64 l = (u64)x * (u64)y;
+    add(h >> k, (l >> k) | ((u64)h << (64 - k)));
   }
   // times 2^(E - 79): E the sum of the two tables' bounds
   __device__ __forceinline__ double value(int E) const {
@@ -542,6 +560,41 @@ __device__ __forceinline__ void lanes_add(LimbSum& x, unsigned mask) {
   }
 }
 
+// Two 64-bit sums over the group, in every lane.
+template <int T>
+__device__ __forceinline__ void lanes_add(i64& x, i64& y, unsigned mask) {
+  if constexpr (T > 32) {
+    __shared__ i64 sx[T], sy[T];
+    const int l = threadIdx.x & (T - 1);
+#pragma unroll
+    for (int off = T / 2; off >= 32; off >>= 1) {
+      __syncthreads();
+      sx[l] = x;
+      sy[l] = y;
+      __syncthreads();
+      x += sx[l ^ off];
+      y += sy[l ^ off];
+    }
+  }
+  constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+  for (int off = W / 2; off > 0; off >>= 1) {
+    x += __shfl_xor_sync(mask, x, off, W);
+    y += __shfl_xor_sync(mask, y, off, W);
+  }
+}
+
+// What is left out of a class-5 sum, from sums over its tables: the products of
+// low limbs, and above d = 8 what the products B C were rounded by times the A
+// they are multiplied with (its high limbs: the rest is 2^-27 of that).
+struct LimbRest {
+  i64 la = 0, lb = 0, ha = 0, rb = 0;  // sums of A's l, B's l, A's h, B C's rests
+  __device__ __forceinline__ void add_to(LimbSum& s) const {
+    s.add_product(la, lb, 27);
+    s.add_product(ha, rb, 37);
+  }
+};
+
 // Exponent E with v < 2^E; a zero (a flagged factor), below every factor with
 // room, gets one that leaves its fixed-point value 0.
 __device__ __forceinline__ int exp_bound(double v) {
@@ -570,27 +623,60 @@ __device__ __forceinline__ void lane_leaves(int lane, int lg, int& p0, int& cnt)
 
 __device__ __forceinline__ int lg_ceil(int n) { return n <= 1 ? 0 : 32 - __clz(n - 1); }
 
-// Class 5 of the real factors by one thread: pattern m = (m_A, hi), value
-// A[m_A] B[hi] (A[m_A] (B[.] C[.]) above d = 8); CH entries of A stay in
-// registers while hi runs, so a product costs one shared-memory read in CH.
+// Class 5 of the real factors by one thread: pattern m = (m_A, hi), value A[m_A]
+// B[hi] (above d = 8 A[m_A] (B[.] C[.])); CH entries of A stay in registers while
+// hi runs, so a product costs one shared-memory read in CH.
 template <int CH, class WF>
-__device__ __forceinline__ void fac_class5(const WF& W, const FacLayout& Ly, int pa, int pb, int pc,
+__device__ __forceinline__ void fac_class5(const WF& W, const FacLayout& Ly, int pa, int pb,
                                            LimbSum& sum) {
-  const int nA = 1 << pa, nhi = 1 << (pb + pc), bm = (1 << pb) - 1;
+  const int nA = 1 << pa, nB = 1 << pb;
+  int la = 0, lb = 0;  // at most 16 entries each
+  LimbAcc acc;         // at most 256 products
   for (int lo = 0; lo < nA; lo += CH) {
     Limbs a[CH];
 #pragma unroll
-    for (int i = 0; i < CH; ++i) a[i] = limbs_unpack(W(Ly.A + lo + i));
+    for (int i = 0; i < CH; ++i) {
+      a[i] = limbs_unpack(W(Ly.A + lo + i));
+      la += a[i].l;
+    }
+    lb = 0;  // the same for every stretch of A
+    for (int hi = 0; hi < nB; ++hi) {
+      const Limbs b = limbs_unpack(W(Ly.B + hi));
+      lb += b.l;
+#pragma unroll
+      for (int i = 0; i < CH; ++i) acc.add(a[i], b);
+    }
+  }
+  acc.mid += ((i64)la * lb) >> 27;
+  sum.take(acc);
+}
+// above d = 8
+template <int CH, class WF>
+__device__ __forceinline__ void fac_class5c(const WF& W, const FacLayout& Ly, int pa, int pb,
+                                            int pc, LimbSum& sum) {
+  const int nA = 1 << pa, nhi = 1 << (pb + pc), bm = (1 << pb) - 1;
+  LimbRest rest;
+  for (int lo = 0; lo < nA; lo += CH) {
+    Limbs a[CH];
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+      a[i] = limbs_unpack(W(Ly.A + lo + i));
+      rest.la += a[i].l;
+      rest.ha += a[i].h;
+    }
     LimbAcc acc;
+    rest.lb = rest.rb = 0;
     for (int hi = 0; hi < nhi; ++hi) {
-      Limbs b = limbs_unpack(W(Ly.B + (hi & bm)));
-      if (pc) b = LimbAcc::product(b, limbs_unpack(W(Ly.C + (hi >> pb))));
+      const Limbs b = LimbAcc::product(limbs_unpack(W(Ly.B + (hi & bm))),
+                                       limbs_unpack(W(Ly.C + (hi >> pb))), rest.rb);
+      rest.lb += b.l;
 #pragma unroll
       for (int i = 0; i < CH; ++i) acc.add(a[i], b);
       if (((hi + 1) & (kLimbRun / CH - 1)) == 0) sum.take(acc);
     }
     sum.take(acc);
   }
+  rest.add_to(sum);
 }
 
 // Class sums and split axis of one region from per-axis factors (kReal);
@@ -826,8 +912,8 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
       }
     }
   }
-  // class 4: the four nodes of the pairs j < k, a pair's exact sum cut to 2^-55
-  // of the largest product that two axes can have
+  // class 4: the four nodes of the pairs j < k, a pair's exact sum rounded to
+  // 2^-54 of the largest product that two axes can have
   LimbSum s5;
   LimbAcc acc;
   i64 s4 = 0;
@@ -845,8 +931,10 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     pair.add(j0, k1);
     pair.add(j1, k0);
     pair.add(j1, k1);
-    const int sh = M1 + M2 - __double2hiint(W(Ly.x3 + j)) - __double2hiint(W(Ly.x3 + k));
-    s4 += pair.number() >> min(sh, 63);
+    pair.mid += ((i64)(j0.l + j1.l) * (k0.l + k1.l)) >> 27;
+    const int sh = min(
+        M1 + M2 - __double2hiint(W(Ly.x3 + j)) - __double2hiint(W(Ly.x3 + k)), 62);
+    s4 += (pair.number() + (((i64)1 << sh) >> 1)) >> sh;
   }
   // class 5
   const Limbs one{1 << 26, 0};
@@ -854,19 +942,32 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     if (pb == 0) {  // d = 1
       for (int q = 0; q < nA; ++q) acc.add(limbs_unpack(W(Ly.A + q)), one);
       s5.take(acc);
+    } else if (pc) {
+      fac_class5c<8>(W, Ly, pa, pb, pc, s5);
     } else if (nA >= 8) {
-      fac_class5<8>(W, Ly, pa, pb, pc, s5);
+      fac_class5<8>(W, Ly, pa, pb, s5);
     } else if (nA >= 4) {
-      fac_class5<4>(W, Ly, pa, pb, pc, s5);
+      fac_class5<4>(W, Ly, pa, pb, s5);
     } else {
-      fac_class5<2>(W, Ly, pa, pb, pc, s5);
+      fac_class5<2>(W, Ly, pa, pb, s5);
     }
   } else {
     int run = 0;
+    LimbRest rest;
+    for (int q = lane; q < nA; q += T) {
+      const Limbs a = limbs_unpack(W(Ly.A + q));
+      rest.la += a.l;
+      rest.ha += a.h;
+    }
     for (int m = lane; m < (1 << d); m += T) {
       const int hi = m >> pa;
       Limbs b = pb ? limbs_unpack(W(Ly.B + (hi & (nB - 1)))) : one;
-      if (pc) b = LimbAcc::product(b, limbs_unpack(W(Ly.C + (hi >> pb))));
+      i64 rb = 0;
+      if (pc) b = LimbAcc::product(b, limbs_unpack(W(Ly.C + (hi >> pb))), rb);
+      if ((m & (nA - 1)) == 0) {  // once for every hi
+        rest.lb += b.l;
+        rest.rb += rb;
+      }
       acc.add(limbs_unpack(W(Ly.A + (m & (nA - 1)))), b);
       if (++run == kLimbRun) {
         s5.take(acc);
@@ -879,6 +980,9 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     lanes_add<T>(t4, mask);
     s4 = (i64)t4.lo;
     lanes_add<T>(s5, mask);
+    lanes_add<T>(rest.la, rest.lb, mask);
+    if (pc) lanes_add<T>(rest.ha, rest.rb, mask);
+    rest.add_to(s5);
   }
   double f0 = F;
   if constexpr (SF::kFlag) f0 = zc ? 0.0 : F;

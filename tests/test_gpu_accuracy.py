@@ -118,3 +118,17 @@ def test_steep_factors(gpu_ctx, fam, lo, hi, d, whole):
     mine, node = _rms_errors(gpu_ctx, fam, _cases(fam, d, 48, lo, hi, whole, 11 * d + int(lo)),
                              _exact_i7)
     assert mine <= 1.25 * node + 0.5 * EPS
+
+
+@pytest.mark.parametrize("fam,lo,hi,d", [(G.GAUSSIAN, 2.8, 3.2, 12), (G.GAUSSIAN, 2.8, 3.2, 14),
+                                         (G.GAUSSIAN, 0.5, 3, 14), (G.GAUSSIAN, 2.8, 3.2, 16),
+                                         (G.PRODUCT_PEAK, 4.5, 5.5, 14),
+                                         (G.PRODUCT_PEAK, 4.5, 5.5, 16),
+                                         (G.PRODUCT_PEAK, 10, 60, 16), (G.C0, 4, 12, 14)])
+def test_class_sums_of_many_products(gpu_ctx, fam, lo, hi, d):
+    """2^12 and more products of tables whose largest entries dominate (the whole
+    domain): the sums of integer products are exact but for the tables' entries,
+    each within half an eps of its table's largest, so the node-wise form's error
+    is met up to a quarter and half an eps."""
+    mine, node = _rms_errors(gpu_ctx, fam, _cases(fam, d, 24, lo, hi, True, d), _exact_i7)
+    assert mine <= 1.25 * node + 0.5 * EPS
