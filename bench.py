@@ -116,7 +116,7 @@ RULE_EXEC_FP64_FLOPS_D8 = {0: 526.0, 1: 802.0, 2: 231.0, 3: 423.0, 4: 295.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "c1e44ef04cc69d9b"
+RULE_COUNTS_SHA16 = "58f33d2cf7ab3e97"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per

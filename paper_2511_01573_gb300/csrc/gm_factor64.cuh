@@ -485,6 +485,12 @@ struct LimbAcc {
     mid += (i64)a.h * b.l;
     mid += (i64)a.l * b.h;
   }
+  // the same for a b that was just split from a product (mad_wide)
+  __device__ __forceinline__ void add_split(Limbs a, Limbs b) {
+    mad_wide(hh, a.h, b.h);
+    mad_wide(mid, a.h, b.l);
+    mad_wide(mid, a.l, b.h);
+  }
   __device__ __forceinline__ void sub(Limbs a, Limbs b) {
     hh -= (i64)a.h * b.h;
     mid -= (i64)a.h * b.l;
@@ -501,11 +507,6 @@ struct LimbAcc {
     const i64 up = (r.mid + (1 << 25)) >> 26;
     rest += (((r.mid - (up << 26)) << 27) + (i64)a.l * b.l) >> 16;
     return limbs_split((r.hh << 1) + up);
-  }
-  __device__ __forceinline__ static Limbs product(Limbs a, Limbs b) {
-    LimbAcc r;
-    r.add(a, b);
-    return limbs_split(r.number());
   }
 };
 
@@ -528,6 +529,11 @@ struct LimbSum {
     const i64 h = __mul64hi(x, y);
     const u64 l = (u64)x * (u64)y;
     add(h >> k, (l >> k) | ((u64)h << (64 - k)));
+  }
+  // x 2^(48 - k), k >= 0
+  __device__ __forceinline__ void add_scaled(i64 x, int k) {
+    const int r = k - 48;
+    add(x >> min(16 + k, 63), r < 0 ? (u64)x << -r : (u64)(x >> min(r, 63)));
   }
   // times 2^(E - 79): E the sum of the two tables' bounds
   __device__ __forceinline__ double value(int E) const {
@@ -671,7 +677,7 @@ __device__ __forceinline__ void fac_class5c(const WF& W, const FacLayout& Ly, in
                                        limbs_unpack(W(Ly.C + (hi >> pb))), rest.rb);
       rest.lb += b.l;
 #pragma unroll
-      for (int i = 0; i < CH; ++i) acc.add(a[i], b);
+      for (int i = 0; i < CH; ++i) acc.add_split(a[i], b);
       if (((hi + 1) & (kLimbRun / CH - 1)) == 0) sum.take(acc);
     }
     sum.take(acc);

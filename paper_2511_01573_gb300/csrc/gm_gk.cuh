@@ -27,7 +27,7 @@
 // digits; they are walked on their own, because a lane that skips the term
 // saves nothing when another lane of its warp needs it.  f >= 0 for these
 // integrands, so sum |wK f| is I_K's sum.  d = 4, C0, 2500 regions: 6.57 ->
-// 0.26 ms (0.71 with FP64 products).  Other integrands, and regions whose
+// 0.27 ms (0.71 with FP64 products).  Other integrands, and regions whose
 // factors lack exponent room, evaluate f at every node.
 #pragma once
 
@@ -61,16 +61,18 @@ struct GkSums {
 };
 
 // Combine the sums of the region's 32 W lanes in a fixed order: every lane
-// of the region's first warp returns the total.  scratch: [W][9].
+// of the region's first warp returns the total (of A unless it is K's).  scratch:
+// [W][9].
 template <int W>
-__device__ __forceinline__ void gk_combine(GkSums& s, double* scratch) {
+__device__ __forceinline__ void gk_combine(GkSums& s, int d, bool a_is_k, double* scratch) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     s.K += __shfl_xor_sync(0xffffffffu, s.K, off);
     s.G += __shfl_xor_sync(0xffffffffu, s.G, off);
-    s.A += __shfl_xor_sync(0xffffffffu, s.A, off);
+    if (!a_is_k) s.A += __shfl_xor_sync(0xffffffffu, s.A, off);
 #pragma unroll
-    for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] += __shfl_xor_sync(0xffffffffu, s.E[k], off);
+    for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
+      if (k < d) s.E[k] += __shfl_xor_sync(0xffffffffu, s.E[k], off);
   }
   if constexpr (W > 1) {
     const int w = threadIdx.x >> 5;
@@ -79,7 +81,9 @@ __device__ __forceinline__ void gk_combine(GkSums& s, double* scratch) {
       o[0] = s.K;
       o[1] = s.G;
       o[2] = s.A;
-      for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) o[3 + k] = s.E[k];
+#pragma unroll
+      for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
+        if (k < d) o[3 + k] = s.E[k];
     }
     __syncthreads();
     if (w == 0) {
@@ -87,8 +91,10 @@ __device__ __forceinline__ void gk_combine(GkSums& s, double* scratch) {
         const double* o = scratch + v * (3 + GMQ_GK_MAX_DIM);
         s.K += o[0];
         s.G += o[1];
-        s.A += o[2];
-        for (int k = 0; k < GMQ_GK_MAX_DIM; ++k) s.E[k] += o[3 + k];
+        if (!a_is_k) s.A += o[2];
+#pragma unroll
+        for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
+          if (k < d) s.E[k] += o[3 + k];
       }
     }
   }
@@ -138,11 +144,23 @@ __device__ __forceinline__ void gk_sums_nodes(const SmemParams<double>& P, const
   }
 }
 
-// The same from per-axis factors, relative to F.  kt, rt: wK e [d][15] and r wK e
-// of axis 0 [15] as limbs (gm_factor64.cuh) below 2^E[k] and 2^(E[0] + 1); gt: wG
-// e [d][15].  A row's product of limbs and the node products and sums run on
-// the integer pipes; a row leaves the FP64 pipe its sum's conversion and the
-// E_k of the other axes.
+// An axis entry of a row's product: 64-bit mantissa (the 53 bits of a double at
+// the top) and its biased exponent in the low eleven bits; 0 for 0.  Kept in
+// integer registers throughout: as a double it can be a signalling NaN, which a
+// select of doubles was seen to quieten.
+__device__ __forceinline__ u64 gk_word(double v) {
+  const u64 b = (u64)__double_as_longlong(v);
+  if (b << 1 == 0) return 0;
+  return ((b << 11) | 0x8000000000000000ull) + ((b >> 52) & 0x7ff);
+}
+
+// The same from per-axis factors, relative to F.  kt: wK e [d][15], axis 0's and
+// rt's (r wK e of axis 0 [15]) as limbs (gm_factor64.cuh) below 2^E[0] and 2^(E[0]
+// + 1), the other axes' as gk_word; gt: wG e [d][15].  Every row's product has its
+// own exponent: rounded to one bound for all, 15^5 rows of which a few are large
+// put I_K of d = 6 up to 3e-12 off.  A row's product, the node products and sums
+// run on the integer pipes; a row leaves the FP64 pipe its sum's conversion and
+// the E_k of the other axes.
 template <int W>
 __device__ __forceinline__ void gk_sums_factors(const GkConst& K, int d, int lane,
                                                 const double* kt, const double* gt,
@@ -154,42 +172,57 @@ __device__ __forceinline__ void gk_sums_factors(const GkConst& K, int d, int lan
     grows *= 7;
     Er += E[k];
   }
+  int lk = 0, lr = 0;  // sums of the low limbs, whose products a row adds at once
+#pragma unroll
+  for (int j = 0; j < 15; ++j) {
+    lk += limbs_unpack(kt[j]).l;
+    lr += limbs_unpack(rt[j]).l;
+  }
   LimbSum sk, se;
-  LimbAcc e0;
-  int run = 0;
   for (int row = lane; row < rows; row += L) {
-    int q = row;
-    Limbs kr{1 << 26, 0};
+    int q = row, x = 0;
+    u64 m = 0;
     int dig[GMQ_GK_MAX_DIM];
 #pragma unroll
     for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) {
       if (k < d) {
         dig[k] = q % 15;
         q /= 15;
-        const Limbs v = limbs_unpack(kt[k * 15 + dig[k]]);
-        kr = k == 1 ? v : LimbAcc::product(kr, v);
+        const u64 w = reinterpret_cast<const u64*>(kt)[k * 15 + dig[k]];
+        const u64 v = w & ~0x7ffull;
+        x += (int)(w & 0x7ff) - 1022;
+        m = k == 1 ? v : fixed_mul(m, v);
       }
     }
-    LimbAcc rk;
+    // m 2^(x - 64) as limbs times 2^x (at most d - 2 <= 4 leading zeros)
+    Limbs kr{1 << 26, 0};
+    if (d > 1) {
+      const int lz = __clz((int)(m >> 32));
+      m <<= lz;
+      x -= lz;
+      kr = limbs_split((i64)(m >> 11) + (i64)((m >> 10) & 1));
+    }
+    LimbAcc rk, re;
 #pragma unroll
     for (int j = 0; j < 15; ++j) {
-      rk.add(limbs_unpack(kt[j]), kr);
-      e0.add(limbs_unpack(rt[j]), kr);
+      rk.add_split(limbs_unpack(kt[j]), kr);
+      re.add_split(limbs_unpack(rt[j]), kr);
     }
-    const double v = (double)rk.number();
+    rk.mid += ((i64)lk * kr.l) >> 27;
+    re.mid += ((i64)lr * kr.l) >> 27;
+    const i64 nk = rk.number();
+    double v = (double)nk;
+    if (nk != 0) v = __hiloint2double(__double2hiint(v) + (int)((unsigned)x << 20), __double2loint(v));
 #pragma unroll
     for (int k = 1; k < GMQ_GK_MAX_DIM; ++k)
       if (k < d) s.E[k] = fma(K.r[dig[k]], v, s.E[k]);
-    sk.take(rk);
-    if ((run += 15) > kLimbRun - 15) {
-      se.take(e0);
-      run = 0;
-    }
+    sk.add_scaled(nk, Er - x);
+    se.add_scaled(re.number(), Er - x);
   }
-  se.take(e0);
-  s.K = sk.value(E[0] + Er);
-  s.E[0] = se.value(E[0] + 1 + Er);
-  const double unit = __hiloint2double((970 + E[0] + Er) << 20, 0);  // 2^(E0 + Er - 53)
+  // numbers are in units of 2^(E0 + x - 53), sums in 2^(E0 + Er - 101)
+  s.K = sk.value(E[0] + Er - 22);
+  s.E[0] = se.value(E[0] + 1 + Er - 22);
+  const double unit = __hiloint2double((970 + E[0]) << 20, 0);  // 2^(E0 - 53)
 #pragma unroll
   for (int k = 1; k < GMQ_GK_MAX_DIM; ++k) s.E[k] = __dmul_rn(unit, s.E[k]);
   for (int row = lane; row < grows; row += L) {
@@ -208,7 +241,6 @@ __device__ __forceinline__ void gk_sums_factors(const GkConst& K, int d, int lan
     for (int j = 3; j < 15; j += 2) rg = fma(gt[j], gr, rg);
     s.G = __dadd_rn(s.G, rg);
   }
-  s.A = s.K;
 }
 
 // W warps per region, kGkBlock / (32 W) regions per block.
@@ -267,7 +299,9 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
     if (active && lane < d) bound[w][lane] = exp_bound(__hiloint2double(bound[w][lane], 0));
     __syncthreads();
     if (active) {
-      for (int q = lane; q < d * 15; q += L) kt[q] = limbs_of(kt[q], bound[w][q / 15]);
+      for (int q = lane; q < 15; q += L) kt[q] = limbs_of(kt[q], bound[w][0]);
+      for (int q = 15 + lane; q < d * 15; q += L)
+        reinterpret_cast<u64*>(kt)[q] = gk_word(kt[q]);
       for (int j = lane; j < 15; j += L) rt[j] = limbs_of(rt[j], bound[w][0] + 1);
     }
     __syncthreads();
@@ -294,8 +328,9 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
       F = 1.0;
   }
   if (!factors) gk_sums_nodes<FAM, W>(P, K, d, lane, xt[w], xs[w] + lane, s);
-  gk_combine<W>(s, scratch);
+  gk_combine<W>(s, d, factors, scratch);
   if (lane != 0) return;
+  if (factors) s.A = s.K;
   s.K = __dmul_rn(F, s.K);
   s.G = __dmul_rn(F, s.G);
   s.A = __dmul_rn(F, s.A);

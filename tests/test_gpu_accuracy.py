@@ -132,3 +132,36 @@ def test_class_sums_of_many_products(gpu_ctx, fam, lo, hi, d):
     is met up to a quarter and half an eps."""
     mine, node = _rms_errors(gpu_ctx, fam, _cases(fam, d, 24, lo, hi, True, d), _exact_i7)
     assert mine <= 1.25 * node + 0.5 * EPS
+
+
+@pytest.mark.parametrize("fam,lo,hi", [(G.PRODUCT_PEAK, 10, 20), (G.PRODUCT_PEAK, 30, 60),
+                                       (G.PRODUCT_PEAK, 100, 300), (G.C0, 5, 20), (G.C0, 0.5, 3),
+                                       (G.GAUSSIAN, 3, 9)])
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 6])
+def test_gauss_kronrod_far_factors(gpu_ctx, oracle, fam, lo, hi, d):
+    """I_K of the tensor rule on the whole domain, where a few of the 15^d terms
+    make the sum: the product over the axes of the sums of 15 terms in long
+    double.  A factor is within 1.5 eps, the centre within 2, the entries of axis
+    0 within half an eps of its largest, row products and sums below: 1.5 sqrt(d) +
+    4 eps rms, and the coordinates' rounding, half an eps of |x - u| <= 1, which
+    moves f by a for the exponentials and, worst, by 2 a^2 |x - u| <= a for the
+    peak, times sqrt(d)."""
+    K = np.asarray(oracle.gk_table())
+    rng = np.random.default_rng(100 * d + int(lo))
+    sq = []
+    for _ in range(12):
+        a, u = rng.uniform(lo, hi, d), rng.uniform(0, 1, d)
+        if fam == G.GAUSSIAN:
+            u = 0.25 + 0.5 * u
+        la, lu = a.astype(LD), u.astype(LD)
+        b = (1 / (la * la) if fam == G.PRODUCT_PEAK else la * la).astype(np.float64).astype(LD)
+        from paper_2511_01573_gb300 import gmq
+        T = np.asarray(gmq.gk_table()).astype(LD)
+        x = LD(0.5) + LD(0.5) * T[:15]
+        ref = LD(1)
+        for k in range(d):
+            ref *= np.sum(T[15:30] * _factor(fam, la[k], lu[k], b[k], x)) / 2
+        half = _soa(np.full((1, d), 0.5))
+        ik = gpu_ctx.eval_rule_gk(fam, a, u, half, half)[0].item()
+        sq.append(float((LD(ik) - ref) / ref) ** 2)
+    assert np.sqrt(np.mean(sq)) <= (1.5 * d ** 0.5 + 4 + 0.5 * d ** 0.5 * hi / 4) * EPS
