@@ -8,17 +8,20 @@
 // product (two or three multiply-adds) is some five times cheaper than an
 // FP64 one.  A corner-peak node costs 12 FP64 instructions in the separable
 // form, ~900 cycles; here it costs about 85 instructions, one of them an FP32
-// reciprocal.  d = 8, 2^20 regions, one thread per region: 9.41 -> 1.54 ms (4829
-// -> 241 FP64 instructions a region; issue slots 60 % busy, twelve warps an SM).
+// reciprocal.  d = 8, 2^20 regions, one thread per region: 9.41 -> 1.57 ms (4829
+// -> 222 FP64 instructions a region; issue slots 60 % busy, twelve warps an SM).
 //
-// Scaling: with inv about 1 / min S over the region (8 significant bits, so
-// that its powers are nearly exact), s = S inv lies in (1, 4) and f =
-// inv^(d+1) s^-(d+1).  S is linear in the coordinates, so every node's s is
-// an integer sum of the centre's and of +-lambda a_k h_k inv in units of
-// 2^-58: exact, whatever the order.  Values u = s^-(d+1) < 1 are in units of
-// 2^-64 and class sums are exact 96-bit integers, so no lane mapping can
-// change a bit.  Errors: 2^-59 per term of s and 2^-60 of 1 / s, both times
-// d + 1, and 2^-63 per product, against 2^-53 per operation before.
+// Scaling: with inv about 1 / (the smallest S of the nodes) (8 significant bits),
+// s = S inv lies in (1, 4) and f = inv^(d+1) s^-(d+1).  S is linear in the
+// coordinates, so every node's s is an integer sum of the centre's and of
+// +-lambda a_k h_k inv in units of 2^-58: exact, whatever the order.  Values u =
+// s^-(d+1) < 1 are in units of 2^-64 and class sums are exact 96-bit integers, so
+// no lane mapping can change a bit.  Classes 1 to 4, whose nodes move one axis or
+// two, and class 5 have an inv each, so that the largest u of the sums is near 1:
+// u is rounded to 2^-64 and not to its own size, which with one inv for the whole
+// box (S down to a corner that is no node) left f(centre) at d = 16 with 30 bits.
+// Errors relative to the sums: 2^-59 per term of s and 2^-60 of 1 / s, both times
+// d + 1; of a power 2^-64 per node, whose mean is added back (pow_bias).
 // Regions where S is not positive, spans a factor of about 4 or more, or
 // leaves no exponent room are evaluated by region_sums64.
 #pragma once
@@ -65,6 +68,44 @@ __device__ __forceinline__ void fixed_pow(u64 (&u)[N], int e) {
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) u[i] = r[i];
+}
+
+// |x| in FP32 by integer operations, rounded towards zero; 0 below 2^-126, infinity
+// above FP32's range and for NaN.
+__device__ __forceinline__ float abs_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, e = hi >> 20;
+  const unsigned b = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) |
+                     ((unsigned)__double2loint(x) >> 29);
+  return __uint_as_float(e < 897u ? 0u : (e < 1151u ? b : 0x7f800000u));
+}
+
+// What n powers u^e of fixed_pow lack in the mean, in units of 2^-64: the last
+// product drops 5/4 of them (a square 5/6).
+__device__ __forceinline__ u64 pow_bias(int n, int e) {
+  return (u64)((e & (e - 1)) ? (5 * n + 2) >> 2 : (5 * n + 3) / 6);
+}
+
+// inv^e rounded to FP64 (2^-59 beside), inv positive and normal: the classes'
+// factors, whose errors do not cancel between them.
+__device__ __forceinline__ double pow_rounded(double inv, int e) {
+  const int hi = __double2hiint(inv);
+  const u64 u = ((u64)((hi & 0xfffff) | 0x100000) << 43) | ((u64)(unsigned)__double2loint(inv) << 11);
+  const int x = ((hi >> 20) & 0x7ff) - 1022;  // inv = u 2^(x - 64)
+  u64 r = u;
+  int rx = x;
+  auto times = [&](u64 v, int vx) {
+    r = fixed_mul(r, v);
+    rx += vx;
+    if ((i64)r >= 0) {
+      r <<= 1;
+      --rx;
+    }
+  };
+  for (int b = 30 - __clz(e); b >= 0; --b) {
+    times(r, rx);
+    if ((e >> b) & 1) times(u, x);
+  }
+  return __longlong_as_double((i64)(((u64)(rx + 1021) << 52) + (((r >> 10) + 1) >> 1)));
 }
 
 // Sum of 64-bit values in 96 bits.
@@ -117,8 +158,7 @@ __device__ __forceinline__ void lanes_add(FixedAcc& x, unsigned mask) {
 // Class sums and split axis of one region of the corner peak; arguments as
 // region_sums64 (the workspace fits the separable form's: [d] steps of
 // lambda3, the class-5 chains, with T > 1 lanes [2d] steps of lambda2 and
-// lambda5 and the centre's s).  False: the region's S does not fit, and
-// nothing was written to `o` (every lane of the group returns the same).
+// lambda5).  False: the region's S does not fit, and nothing was written to `o` (every lane of the group returns the same).
 template <int T, class PT, class CH>
 __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
                                                      const unsigned short* pairs, const CH& ch,
@@ -132,9 +172,11 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
   const int e2 = eC + (pc ? 1 << pc : 0), e5 = e2 + d;
   auto W = [&](int e) -> i64& { return reinterpret_cast<i64*>(w)[(long long)e * ws]; };
   // S at the centre as a sum of two doubles (f moves by d + 1 times the
-  // relative error of S, all nodes alike, and the FP64 pipe has room) and the
-  // reach of the nodes, by every lane
-  double S = 1.0, Slo = 0.0, reach = 0.0;
+  // relative error of S, all nodes alike, and the FP64 pipe has room) and, in
+  // FP32, the reach of the nodes that move one axis or two and of those that move
+  // all, by every lane
+  double S = 1.0, Slo = 0.0;
+  float all = 0.0f, m1 = 0.0f, m2 = 0.0f;  // sum of |a h| and the two largest
   for (int k = 0; k < d; ++k) {
     double c, h;
     ch(k, c, h);
@@ -142,20 +184,30 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
     const double t = __dadd_rn(S, p);
     Slo = __dadd_rn(Slo, __dadd_rn(fma(P.a[k], c, -p), __dsub_rn(p, __dsub_rn(t, S))));
     S = t;
-    reach = fma(fabs(P.a[k]), fabs(h), reach);
+    const float ah = abs_f32(P.a[k]) * abs_f32(h);
+    all += ah;
+    m2 = fmaxf(m2, fminf(m1, ah));
+    m1 = fmaxf(m1, ah);
   }
-  reach = __dmul_rn(lam3, reach);
-  // inv: the leading 8 bits of 1 / min S, rounded up, so that s > 1
-  const double smin = __dsub_rn(S, reach);
-  const unsigned ex = ((unsigned)__double2hiint(smin) >> 20);  // sign and exponent
-  if (ex - (1023u - 40u) > 80u) return false;                  // not in [2^-40, 2^41): negative, 0, NaN
-  // (two units of the eighth bit above the truncated quotient put the
-  // smallest s between 1 + 2^-8 and 1 + 2^-6)
-  const float q = __fdiv_rn(1.0f, __double2float_rn(smin));
-  const double inv = (double)__uint_as_float((__float_as_uint(q) & 0xffff0000u) + 0x20000u);
-  const double s0 = __dmul_rn(S, inv);
-  if (!(fma(reach, inv, s0) < 3.99)) return false;
-  const i64 v0 = to_fixed(s0, 58) + to_fixed(fma(Slo, inv, fma(S, inv, -s0)), 58);
+  const float Sf = __double2float_rn(S);
+  // inv: the leading 8 bits of 1 / (S - reach), rounded up, so that s > 1; v: s of
+  // the centre.  False: s does not fit.
+  auto scale = [&](float reach, double& inv, i64& v) -> bool {
+    const float smin = Sf - reach;
+    const unsigned ex = __float_as_uint(smin) >> 23;  // sign and exponent
+    if (ex - (127u - 40u) > 80u) return false;  // not in [2^-40, 2^41): negative, 0, NaN
+    // (two units of the eighth bit above the truncated quotient put the
+    // smallest s between 1 + 2^-8 and 1 + 2^-6, less 2^-20 for the reach)
+    const float q =
+        __uint_as_float((__float_as_uint(__fdiv_rn(1.0f, smin)) & 0xffff0000u) + 0x20000u);
+    inv = f2d_exact(q);
+    const double s0 = __dmul_rn(S, inv);
+    v = to_fixed(s0, 58) + to_fixed(fma(Slo, inv, fma(S, inv, -s0)), 58);
+    return (Sf + reach) * q < 3.98f;
+  };
+  double inv, inv5;
+  i64 v0, v05;
+  if (!scale((float)lam3 * (m1 + m2), inv, v0) || !scale((float)lam5 * all, inv5, v05)) return false;
   const int e = d + 1;
   // 2^64 s^-(d+1) of the nodes at s = v 2^-58
   auto nodes = [&](auto& v) {
@@ -163,13 +215,14 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
     for (auto& x : v) x = fixed_rcp((i64)x);
     fixed_pow(v, e);
   };
+  const double l2 = __dmul_rn(lam2, inv), l3 = __dmul_rn(lam3, inv), l5 = __dmul_rn(lam5, inv5);
   auto steps = [&](int k, i64& g2, i64& g3, i64& g5) {
     double c, h;
     ch(k, c, h);
-    const double t = __dmul_rn(__dmul_rn(P.a[k], h), inv);
-    g2 = to_fixed(__dmul_rn(lam2, t), 58);
-    g3 = to_fixed(__dmul_rn(lam3, t), 58);
-    g5 = to_fixed(__dmul_rn(lam5, t), 58);
+    const double t = __dmul_rn(P.a[k], h);
+    g2 = to_fixed(__dmul_rn(l2, t), 58);
+    g3 = to_fixed(__dmul_rn(l3, t), 58);
+    g5 = to_fixed(__dmul_rn(l5, t), 58);
   };
   u64 c0[1] = {(u64)v0};
   nodes(c0);
@@ -204,7 +257,7 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
       const int e0 = k < pa ? eA : (k < pa + pb ? eB : eC);
       const int i = k < pa ? k : (k < pa + pb ? k - pa : k - pa - pb);
       if (i == 0) {
-        const i64 head = k ? 0 : v0;
+        const i64 head = k ? 0 : v05;
         W(e0) = head + g5;
         W(e0 + 1) = head - g5;
       } else {
@@ -229,7 +282,7 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
     const int nA = 1 << pa, nB = pb ? 1 << pb : 0, nC = pc ? 1 << pc : 0;
     for (int t = lane; t < nA + nB + nC; t += T) {
       int q0 = t, e0 = eA, j0 = 0, nb = pa;
-      i64 v = v0;
+      i64 v = v05;
       if (q0 >= nA) {
         q0 -= nA;
         e0 = eB;
@@ -311,12 +364,16 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
     lanes_add<T>(s4, mask);
     lanes_add<T>(s5, mask);
   }
-  const double F = ipow(inv, e);
-  o.s1 = __dmul_rn(F, __dmul_rn((double)u0, 0x1p-64));
+  s2.add(pow_bias(2 * d, e));
+  s3.add(pow_bias(2 * d, e));
+  s4.add(pow_bias(4 * np, e));
+  s5.add(pow_bias(1 << d, e));
+  const double F = pow_rounded(inv, e), F5 = pow_rounded(inv5, e);
+  o.s1 = __dmul_rn(F, __dmul_rn((double)(u0 + 1), 0x1p-64));
   o.s2 = __dmul_rn(F, s2.value());
   o.s3 = __dmul_rn(F, s3.value());
   o.s4 = __dmul_rn(F, s4.value());
-  o.s5 = __dmul_rn(F, s5.value());
+  o.s5 = __dmul_rn(F5, s5.value());
   o.f0 = o.s1;
   o.dbest = __dmul_rn(__dmul_rn(F, 0x1p-62), dbest);
   o.kbest = kbest;

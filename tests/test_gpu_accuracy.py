@@ -165,3 +165,40 @@ def test_gauss_kronrod_far_factors(gpu_ctx, oracle, fam, lo, hi, d):
         ik = gpu_ctx.eval_rule_gk(fam, a, u, half, half)[0].item()
         sq.append(float((LD(ik) - ref) / ref) ** 2)
     assert np.sqrt(np.mean(sq)) <= (1.5 * d ** 0.5 + 4 + 0.5 * d ** 0.5 * hi / 4) * EPS
+
+
+def _exact_corner(fam, a, u, c, h):
+    d = len(a)
+    a, c, h = (np.asarray(v, dtype=LD) for v in (a, c, h))
+    l2, l3, l5 = (LD(np.sqrt(v)) for v in (9 / 70, 9 / 10, 9 / 19))
+    s0, ah = 1 + np.sum(a * c), a * h
+    f = lambda s: 1 / s ** (d + 1)
+    s4 = LD(0)
+    for j in range(d):
+        for k in range(j + 1, d):
+            for sj in (1, -1):
+                for sk in (1, -1):
+                    s4 += f(s0 + l3 * (sj * ah[j] + sk * ah[k]))
+    s = np.array([s0], dtype=LD)
+    for k in range(d):
+        s = np.concatenate([s + l5 * ah[k], s - l5 * ah[k]])
+    S = [f(s0), np.sum(f(s0 + l2 * ah) + f(s0 - l2 * ah)), np.sum(f(s0 + l3 * ah) + f(s0 - l3 * ah)),
+         s4, np.sum(f(s))]
+    w = [LD(v) for v in (12824 - 9120 * d + 400 * d * d, 2940, 1820 - 400 * d, 200)]
+    w = [v / 19683 for v in w] + [LD(6859) / 19683 / 2 ** d]
+    return sum(x * y for x, y in zip(w, S)), sum(abs(x * y) for x, y in zip(w, S))
+
+
+@pytest.mark.parametrize("d,total", [(4, 3.3), (8, 2.4), (8, 3.3), (12, 1.85), (12, 3.3),
+                                     (14, 2.4), (14, 3.3), (16, 1.2), (16, 2.4), (16, 3.3)])
+def test_corner_powers(gpu_ctx, d, total):
+    """The corner peak on the whole domain, S spanning up to a factor of almost 4,
+    whose powers d + 1 lie up to 2^34 apart: at most the node-wise form's error and
+    half an eps."""
+    def cases():
+        rng = np.random.default_rng(d)
+        for _ in range(24 if d < 14 else 8):
+            a = rng.uniform(0.1, 1.0, d)
+            yield a * (total / a.sum()), np.zeros(d), np.full(d, 0.5), np.full(d, 0.5)
+    mine, node = _rms_errors(gpu_ctx, G.CORNER_PEAK, cases(), _exact_corner)
+    assert mine <= node + 0.5 * EPS
