@@ -130,7 +130,7 @@ RULE_COUNTS_SHA16 = "6a2bd317ab4ef726"
 MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "df2f645a88873b26"
+MIXED_COUNTS_SHA16 = "1218f4801747e460"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kBatchRuleBlock, 4) k_batch_rule_mixed(const B
     auto cval = [&](int k) { return C[(int64_t)k * B.ld + r]; };
     auto hval = [&](int k) { return H[(int64_t)k * B.ld + r]; };
     RegionSums o;
-    switch (FAM == GMQ_POLY_SUMSQ11 ? 0 : d) {  // the polynomial: node by node
+    switch (d) {
       case 3: region_mixed_walk<FAM, 3>(it.Pf, tab, B.ratio, o); break;
       case 4: region_mixed_walk<FAM, 4>(it.Pf, tab, B.ratio, o); break;
       case 5: region_mixed_walk<FAM, 5>(it.Pf, tab, B.ratio, o); break;

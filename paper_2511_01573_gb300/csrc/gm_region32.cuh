@@ -233,7 +233,10 @@ struct Chain {
 #pragma unroll
       for (int n = 0; n < N; ++n) {
         const float2 s2 = __fmul2_rn(s[n], s[n]), s4 = __fmul2_rn(s2, s2), s8 = __fmul2_rn(s4, s4);
-        s[n] = __fmul2_rn(__fmul2_rn(s8, s2), s[n]);
+        const float2 p = __fmul2_rn(s8, s2);
+        // scalar: the assembler fuses a paired product into the paired addition
+        // that takes it (Acc2), rounding mode or not, and the node loses its rounding
+        s[n] = make_float2(__fmul_rn(p.x, s[n].x), __fmul_rn(p.y, s[n].y));
       }
     } else {
 #pragma unroll
@@ -288,7 +291,7 @@ struct Acc2 {
 // y of them.  2^20 regions, d = 12 / d = 8: corner peak 4.83 -> 3.54 / 0.477 ->
 // 0.386 ms, product peak 4.79 -> 2.98 / 0.482 -> 0.387, Gaussian 4.08 -> 2.95 /
 // 0.424 -> 0.347, C0 3.66 -> 2.97 / 0.391 -> 0.349, cosine 5.78 -> 4.65 / 0.618
-// -> 0.478; up to d = 5 the FP64 differences and weights bound both forms alike.
+// -> 0.478, polynomial 3.19 -> 2.32 / 0.417 -> 0.396; up to d = 5 the FP64 differences and weights bound both forms alike.
 template <int FAM, int D, class PT, class Tab>
 __device__ __forceinline__ void region_mixed_walk(const PT& Pf, const Tab& tab, double ratio,
                                                   RegionSums& o) {

@@ -338,9 +338,7 @@ cudaError_t launch_mixed(int T, const RuleArgs& A, cudaStream_t s) {
   cudaError_t launch_rule_family<FAMV>(int precision, int T, const RuleArgs& A,         \
                                        cudaStream_t s) {                                \
     if (precision == GMQ_FP64) return launch_rule64<FAMV>(T, A, s);                    \
-    /* the polynomial's values are (sum x^2)^11: node by node */                          \
-    if (precision == GMQ_MIXED && T == 1 && A.P.d >= 3 && A.P.d <= 12 &&                \
-        FAMV != GMQ_POLY_SUMSQ11)                                                       \
+    if (precision == GMQ_MIXED && T == 1 && A.P.d >= 3 && A.P.d <= 12)                 \
       return launch_mixed_reg<FAMV>(A, s);                                             \
     if (precision == GMQ_MIXED) return launch_mixed<FAMV>(T, A, s);                    \
     return cudaErrorInvalidValue;                                                      \
