@@ -300,32 +300,52 @@ int auto_splits(int d, int64_t cap) {
 
 // Lanes per region for a sweep of n regions (a launch choice: FP64 results do
 // not depend on it).
-// FP64: what a region costs on the FP64 pipe outside its nodes (centre, volume,
-// weights) is paid once per warp, so few lanes per region waste least; more
-// lanes shorten the chain of one region while warps are few.  Measured, rule
-// call in us for 4 / 1 lanes (d = 8, C0 and corner peak): n = 8192: 81 / 111 and
-// 89 / 103, 16384: 114 / 111 and 101 / 106; for 32 / 4 lanes: n = 512: 61 / 75
-// and 64 / 72, 2048: 77 / 75 and 77 / 73, 8192: 143 / 81; d = 10: n = 2048 (the
-// cosine) 98 / 117, 4096: 134 / 115; a block per region only pays for a region
-// or less per SM.
+// FP64, from factors or in fixed point: what a region costs on the FP64 pipe
+// outside its nodes (centre, volume, weights) is paid once per warp, so few lanes
+// per region waste least; more lanes shorten the chain of one region while warps
+// are few.  Measured (rule calls in us, 152 SMs; real factors / cosine / corner
+// peak).  A block or a warp a region: d = 12, n = 600: 73 / 74 / 85 and 79 / 84 /
+// 94, 1200: 100 / 104 / 108 and 87 / 107 / 106; d = 14, 1200: 133 / 158 / 193 and
+// 144 / 223 / 234.  Up to d = 8, 32 or 4 lanes, n = 1200: 65 / 62 / 65 and 77 / 77 /
+// 80, 3000: 80 / 79 / 79 and 76 / 78 / 76; 4 or one, 8000: 85 / 89 / 84 and 86 / 104 /
+// 103, 15000: 100 / 105 / 103 and 85 / 104 / 105.  Above, 32 lanes last longer (d =
+// 10, 3000: 88 / 92 / 96 against 106 / 113 / 132 with 4) and real factors go to one
+// lane at once (d = 11, 8000: 126 against 160 with 4 and 176 with 32), the others by
+// way of 4 up to d = 10 (d = 10, 8000: 144, 148) and of 32 above (d = 12, 8000: 252,
+// 277, with one 320, 596).
+// FP64, an inner sum and its function at every node (the polynomial, the cosine
+// above d = 14, node-wise evaluation): more threads, the more the costlier a node
+// (polynomial / node-wise C0, d = 8: n = 2000 with 32 or 4 lanes 95 / 104 and 122 /
+// 166, 8000 212 / 239 and 140 / 202, 15000 with 4 or one 225 / 335 and 196 / 470; d =
+// 14, 300 with a block or a warp a region 133 / 341 and 214 / 814).  With the rule
+// above they took up to 2.4 times as long.
 // Mixed: the register walk of one lane (3 <= d <= 12) wins over 32 lanes from
 // some 2000 regions on at 401 nodes (d = 8, C0: n = 512: 68 / 62, 2048: 69 /
 // 75, 32768: 72 / 302), at once below 130 nodes (d = 5: 58 / 70 at 2048) and
 // from about 5000 at 1245 nodes (d = 10: 93 / 97 at 2048, 92 / 159 at 8192; the
 // corner peak 139 / 98 and 141 / 171); 4 lanes never do (111 to 265 us).
-int choose_lanes(int req, int64_t n, int d, int sms, int precision) {
+int choose_lanes(int req, int64_t n, int d, int sms, int precision, int family, bool nodewise) {
   if (req) return req;
   const int64_t nodes = num_nodes(d);
   if (precision != GMQ_FP64) {
-    if (d < 3 || d > 12) {
-      const int64_t want = (int64_t)sms * 256;
+    const int64_t want = (int64_t)sms * 256;
+    if (d < 3 || d > 12)
       return n >= want || nodes < 16 ? 1 : (n * 4 >= want || nodes < 128 ? 4 : 32);
-    }
     return nodes < 256 || n * 256 >= (int64_t)sms * 8 * nodes ? 1 : 32;
   }
-  if (n >= (int64_t)sms * 96 || nodes < 16) return 1;
-  if (n >= (int64_t)sms * (nodes < 1024 ? 8 : 20) || nodes < 128) return 4;
-  return n > sms || nodes < 1024 ? 32 : 128;
+  if (nodes < 16) return 1;
+  const bool cosine = family == GMQ_OSCILLATORY;
+  if (nodewise || family == GMQ_POLY_SUMSQ11 || (cosine && d > kFacRotationMaxDim)) {
+    if (n >= (int64_t)sms * (nodewise && nodes >= 256 ? 256 : 96)) return 1;
+    const int per4 = nodes < 256 ? 24 : (nodewise ? (nodes < 1024 ? 40 : 64) : (nodes < 2048 ? 24 : 64));
+    if (n >= (int64_t)sms * per4 || nodes < 128) return 4;
+    return n < (int64_t)sms * 6 && nodes >= 512 ? 128 : 32;
+  }
+  if (n * 600 <= sms * nodes) return 128;
+  if (d <= 8) return n >= (int64_t)sms * 96 ? 1 : (n >= (int64_t)sms * 8 || nodes < 128 ? 4 : 32);
+  if (n * 512 <= sms * (24 * 512 + nodes)) return 32;
+  if (n >= (int64_t)sms * 96 || !(cosine || family == GMQ_CORNER_PEAK)) return 1;
+  return d <= 10 ? 4 : 32;
 }
 
 cudaError_t launch_rule(int fam, int precision, int T, const RuleArgs& A, cudaStream_t s) {
@@ -962,7 +982,8 @@ gmq_status gmq_integrate(gmq_context* ctx, const gmq_problem* prob, const gmq_op
     std::snprintf(sweep_name, sizeof(sweep_name), "sweep %d: %lld regions", iters + 1,
                   (long long)n);
     NvtxRange sweep_range(sweep_name);
-    const int T = choose_lanes(opt->lanes, n, d, ctx->sm_count, opt->precision);
+    const int T = choose_lanes(opt->lanes, n, d, ctx->sm_count, opt->precision, prob->family,
+                               ctx->eval_mode == GMQ_EVAL_NODEWISE);
     RuleArgs A;
     A.c = cA;
     A.h = hA;
@@ -1138,7 +1159,8 @@ gmq_status gmq_eval_rule(gmq_context* ctx, const gmq_problem* prob, int32_t prec
   A.P = fam_params(prob);
   A.R = rule_const(prob->dim, prob->lo, prob->hi, estimator);
   A.nodewise = ctx->eval_mode == GMQ_EVAL_NODEWISE ? 1 : 0;
-  const int T = choose_lanes(lanes, n, prob->dim, ctx->sm_count, precision);
+  const int T = choose_lanes(lanes, n, prob->dim, ctx->sm_count, precision, prob->family,
+                             ctx->eval_mode == GMQ_EVAL_NODEWISE);
   prof_begin(ctx, kKRule);
   GMQ_CK(launch_rule(prob->family, precision, T, A, ctx->stream));
   prof_end(ctx, kKRule, n);
