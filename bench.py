@@ -97,9 +97,9 @@ CAP = 1 << 24
 # FP64 work of the rule at d = 8 (401 nodes) per region and family, as FP64
 # thread-instructions and flops (FMA = 2): what the separable form, which
 # evaluates the integrand's outer function at every node, spends on it (ncu,
-# sm__thread_inst_executed_pipe_fp64_pred_on over 2^20 regions).  A fixed unit
-# of work.  Family codes: 0 oscillatory, 1 product peak, 2 corner peak,
-# 3 Gaussian, 4 C0.
+# sm__thread_inst_executed_pipe_fp64_pred_on over 2^20 regions).  The roofline
+# line names the instructions beside those executed.  Family codes: 0
+# oscillatory, 1 product peak, 2 corner peak, 3 Gaussian, 4 C0.
 RULE_FP64_INST_D8 = {0: 5631.0, 1: 2476.0, 2: 4829.0, 3: 4136.0, 4: 4080.0}
 RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
 
@@ -113,6 +113,8 @@ RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
 # then the roofline reports no fraction.
 RULE_EXEC_FP64_INST_D8 = {0: 393.0, 1: 533.0, 2: 222.0, 3: 358.0, 4: 278.0}
 RULE_EXEC_FP64_FLOPS_D8 = {0: 526.0, 1: 802.0, 2: 205.0, 3: 423.0, 4: 295.0}
+# all thread instructions a region (smsp__inst_executed x 32), of the same launches
+RULE_EXEC_INST_D8 = {0: 21762.0, 1: 10203.0, 2: 35602.0, 3: 17387.0, 4: 16916.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
@@ -129,8 +131,9 @@ RULE_COUNTS_SHA16 = "6a2bd317ab4ef726"
 # mixed kernel's sources as the FP64 counts are to the FP64 kernel's.
 MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
-                        "gmq_families.cuh", "gm_math_tables.cuh", "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "1218f4801747e460"
+                        "gmq_families.cuh", "gm_int64.cuh", "gm_math_tables.cuh",
+                        "gmq_common.cuh")
+MIXED_COUNTS_SHA16 = "2bb8666dc10ff75d"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):
@@ -1074,13 +1077,15 @@ def main():
     if rank != 0:
         return
     rule = prof["rule"]
-    # FP64 roofline of the rule kernel: FP64 instructions (and flops) per
-    # region of each family at d = 8 (a fixed count: the integrand at 401
-    # nodes plus one accumulation each and the per-region epilogue) times the
-    # regions of that family in the timed steps, over the rule kernel's
-    # event-timed launches.  Peak: the measured FP64 FMA issue rate (probe
-    # kernel, same process); beside it the nominal 2 FP64 lanes per clock per
-    # SM (1.25 TFLOP/s / 2 / 152 SMs / 2.07 GHz) at the median SM clock.
+    # FP64 roofline of the rule kernel: FP64 instructions (and flops) executed
+    # per region of each family at d = 8 (a fixed count) times the regions of
+    # that family in the timed steps, over the rule kernel's event-timed
+    # launches.  Peak: the measured FP64 FMA issue rate (probe kernel, same
+    # process); beside it the nominal 2 FP64 lanes per clock per SM (1.25
+    # TFLOP/s / 2 / 152 SMs / 2.07 GHz) at the median SM clock.  Most of the
+    # kernel's arithmetic runs on the integer pipes, so the fraction alone does
+    # not say how far the kernel is from its bound: issue_view gives all of its
+    # instructions against the four warp instructions that an SM issues a clock.
     roof = None
     clocks = clk.summary()
     counts_current = rule_source_fingerprint() == RULE_COUNTS_SHA16
@@ -1093,6 +1098,8 @@ def main():
         peak_nominal = 2 * 152 * mhz * 1e6 / 1e9  # G FP64 lane-inst/s
         peak = probe64 / 1e9
         ach = inst / avg_s / 1e9
+        issued = sum(RULE_EXEC_INST_D8[f] * n for f, n in timed_fam_regions.items()) / 32 / n_launch
+        issue_peak = 4 * 152 * mhz * 1e6 / 1e9  # G warp-inst/s
         roof = {"bound": "alu", "achieved": ach, "peak": peak,
                 "unit": "G FP64 lane-inst/s", "frac": ach / peak if counts_current else None,
                 "traffic": (RULE_DRAM_BYTES_PER_REGION_D8 * rule["regions"] / n_launch
@@ -1108,8 +1115,13 @@ def main():
                 "counts_match_source": counts_current,
                 "flops_view": {"achieved_gflops": flops / avg_s / 1e9,
                                "peak_gflops_measured_fma": 2 * probe_ops["fma"] / 1e9},
+                "issue_view": {"achieved_G_warp_inst_per_s": issued / avg_s / 1e9,
+                               "peak_G_warp_inst_per_s": issue_peak,
+                               "frac": issued / avg_s / 1e9 / issue_peak if counts_current else None},
                 "inst_per_region": {G.FAMILY_NAMES[f]: RULE_EXEC_FP64_INST_D8[f]
                                     for f in sorted(timed_fam_regions)},
+                "inst_per_region_at_every_node": {G.FAMILY_NAMES[f]: RULE_FP64_INST_D8[f]
+                                                  for f in sorted(timed_fam_regions)},
                 "regions_by_family": {G.FAMILY_NAMES[f]: n // args.steps
                                       for f, n in sorted(timed_fam_regions.items())}}
     line = {
