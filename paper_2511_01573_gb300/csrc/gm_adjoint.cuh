@@ -397,6 +397,7 @@ __device__ __forceinline__ bool grad_region_factors(const GradArgs& A, const Sme
   double s2 = 0.0, s3 = 0.0, vol = 1.0;
   int room = 0;
   for (int k = 0; k < d; ++k) {
+    if (!SF::kMul && room > kFacExpRoom) continue;
     double c, h;
     ch(k, c, h);
     vol = __dmul_rn(vol, __dmul_rn(2.0, h));

@@ -15,10 +15,10 @@
 // rotations (cos Delta, sin Delta), two products per node.  Exponentials, sines
 // and class sums run in fixed point on the integer pipes (gmq_families.cuh,
 // Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
-// the outer function at every node: C0 8.14 -> 0.97 ms (4080 -> 278 FP64
-// instructions a region), Gaussian 8.25 -> 1.04, product peak 4.71 -> 1.14,
+// the outer function at every node: C0 8.14 -> 0.94 ms (4080 -> 278 FP64
+// instructions a region), Gaussian 8.25 -> 1.04, product peak 4.71 -> 1.12,
 // cosine 10.99 -> 1.40; with factors and FP64 sums and functions they took 2.23,
-// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-80 % active) is the
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-82 % active) is the
 // coordinates, the chains and the weights; twelve warps an SM, as many as the
 // workspaces in shared memory let.
 //
@@ -209,24 +209,16 @@ __device__ __forceinline__ i64 low_fixed(const PT& P, int k, double c, double fc
 // |lam| in units of 2^-63
 __device__ __forceinline__ u64 lam_fixed(double lam) { return (u64)to_fixed(fabs(lam), 63); }
 
-// z and exp(z) of one factor whose terms are not below 16: in units of 2^-54 while
-// they are below 256 (|z| < 512), in FP64 from the coordinate above (such a factor
-// has no exponent room, and only its size matters).
-template <int FAM, class PT>
-static __device__ __noinline__ double factor_far(const PT& P, int k, double c, double h, double fc,
-                                                 double lam, bool wide) {
-  using F = Fac<FAM>;
-  if (wide) {
-    const i64 z = F::template z<54>(F::template terms<54>(P, k, c, h, fc), lam_fixed(lam),
-                                    __double2hiint(lam) < 0);
-    return exp_wide(z << 4, round_shifted(z));
-  }
-  const double p = Sep<FAM>::phi(P, k, fma(lam, h, c));
-  return gm_exp(FAM == GMQ_DISCONTINUOUS ? __dsub_rn(p, fc) : __dsub_rn(fc, p));
-}
 // |x| < 256, tested on the high word
 __device__ __forceinline__ bool below_256(double x) {
   return ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x40700000u;
+}
+// The largest |z| of an axis' six factors, from the values of size(), in FP32.
+template <int FAM>
+__device__ __forceinline__ float largest_z(double x, double y) {
+  constexpr float l3 = 0.9486833f;
+  if constexpr (FAM == GMQ_GAUSSIAN) return l3 * (abs_f32(x) + l3 * abs_f32(y));
+  return l3 * abs_f32(y);
 }
 
 // The factors of N coordinates c + lam[i] h.  Which form they take is decided
@@ -262,9 +254,25 @@ __device__ __forceinline__ void factors(const PT& P, int k, double c, double h, 
         e[i] = exp_fixed(F::template z<58>(t, lam_fixed(lam[i]), __double2hiint(lam[i]) < 0));
       return;
     }
+    // Beyond exp(+-345) = 2^+-498 the axis has no exponent room (kFacExpRoom): 0
+    // says so, without an exponential.  In units of 2^-54 below 256; what is left
+    // has an exponent near the limit, and its size is all that matters.
+    const bool none = !(largest_z<FAM>(x, y) < 345.0f);
     const bool wide = below_256(x) && below_256(y);
+    FacTerms t{};
+    if (wide) t = F::template terms<54>(P, k, c, h, fc);
 #pragma unroll 1
-    for (int i = 0; i < N; ++i) e[i] = factor_far<FAM>(P, k, c, h, fc, lam[i], wide);
+    for (int i = 0; i < N; ++i) {
+      double v = 0.0;
+      if (wide) {
+        const i64 z = F::template z<54>(t, lam_fixed(lam[i]), __double2hiint(lam[i]) < 0);
+        v = exp_wide(z << 4, round_shifted(z));
+      } else if (!none) {
+        const double p = Sep<FAM>::phi(P, k, fma(lam[i], h, c));
+        v = gm_exp(FAM == GMQ_DISCONTINUOUS ? __dsub_rn(p, fc) : __dsub_rn(fc, p));
+      }
+      e[i] = none ? 0.0 : v;
+    }
   }
 }
 
@@ -737,6 +745,10 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     PairTree t2, t3;
     Centre<FAM> top;
     for (int k = 0; k < d; ++k) {
+      // (no return from here: lanes that left the loop at different axes would
+      // run what follows one group after the other; the product peak's factors
+      // hardly ever lack room, and the test costs it 6 %)
+      if (!SF::kMul && room > kFacExpRoom) continue;
       double c, h;
       ch(k, c, h);
       const double fc = SF::phi(P, k, c);

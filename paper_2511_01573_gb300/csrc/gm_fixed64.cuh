@@ -70,15 +70,6 @@ __device__ __forceinline__ void fixed_pow(u64 (&u)[N], int e) {
   for (int i = 0; i < N; ++i) u[i] = r[i];
 }
 
-// |x| in FP32 by integer operations, rounded towards zero; 0 below 2^-126, infinity
-// above FP32's range and for NaN.
-__device__ __forceinline__ float abs_f32(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, e = hi >> 20;
-  const unsigned b = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) |
-                     ((unsigned)__double2loint(x) >> 29);
-  return __uint_as_float(e < 897u ? 0u : (e < 1151u ? b : 0x7f800000u));
-}
-
 // What n powers u^e of fixed_pow lack in the mean, in units of 2^-64: the last
 // product drops 5/4 of them (a square 5/6).
 __device__ __forceinline__ u64 pow_bias(int n, int e) {

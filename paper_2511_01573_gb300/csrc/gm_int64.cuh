@@ -49,6 +49,15 @@ __device__ __forceinline__ i64 fixed_mul_signed(i64 a, u64 b) {
   return (i64)ah * bh + (((i64)ah * (int)(bl >> 1)) >> 31) + (i64)(wide_mul(al, (unsigned)bh) >> 32);
 }
 
+// |x| in FP32 by integer operations, rounded towards zero; 0 below 2^-126, infinity
+// above FP32's range and for NaN.
+__device__ __forceinline__ float abs_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, e = hi >> 20;
+  const unsigned b = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) |
+                     ((unsigned)__double2loint(x) >> 29);
+  return __uint_as_float(e < 897u ? 0u : (e < 1151u ? b : 0x7f800000u));
+}
+
 // v 2^-q rounded to nearest (ties away from zero), for q < 1000
 __device__ __forceinline__ double fixed_to_double(i64 v, int q) {
   if (v == 0) return 0.0;
