@@ -349,7 +349,7 @@ struct Centre {
     if (!fixed || !sincos_near(S))
       gm_sincos(S, &sn, &cs);
     else
-      sincos_fixed(v, &sn, &cs);
+      sincos_fixed(v, 58, &sn, &cs);
   }
 };
 
@@ -1074,9 +1074,9 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
       double c2, n2, c3, n3, c5, n5;
       const double z2 = __dmul_rn(lam2, ah), z3 = __dmul_rn(lam3, ah), z5 = __dmul_rn(lam5, ah);
       if (sincos_near(z2) && sincos_near(z3) && sincos_near(z5)) {
-        sincos_fixed(to_fixed(z2, 58), &n2, &c2);
-        sincos_fixed(to_fixed(z3, 58), &n3, &c3);
-        sincos_fixed(to_fixed(z5, 58), &n5, &c5);
+        sincos_fixed(to_fixed(z2, 58), 58, &n2, &c2);
+        sincos_fixed(to_fixed(z3, 58), 58, &n3, &c3);
+        sincos_fixed(to_fixed(z5, 58), 58, &n5, &c5);
       } else {
         gm_sincos(z2, &n2, &c2);
         gm_sincos(z3, &n3, &c3);

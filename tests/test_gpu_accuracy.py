@@ -202,3 +202,18 @@ def test_corner_powers(gpu_ctx, d, total):
             yield a * (total / a.sum()), np.zeros(d), np.full(d, 0.5), np.full(d, 0.5)
     mine, node = _rms_errors(gpu_ctx, G.CORNER_PEAK, cases(), _exact_corner)
     assert mine <= node + 0.5 * EPS
+
+
+@pytest.mark.parametrize("lanes", [1, 32])
+def test_cosine_from_sixteen_on(gpu_ctx, lanes):
+    """The same for arguments in units of 2^-54 (16 <= |x| < 256: within 1.4 eps) and
+    on both sides of the two limits."""
+    rng = np.random.default_rng(5)
+    x = np.concatenate([np.arange(1305, 20861, 2) * np.pi / 256 + 1e-7, rng.uniform(16, 256, 4000),
+                        16 + np.arange(-8, 9) * 2.0 ** -49, 256 + np.arange(-8, 9) * 2.0 ** -45])
+    x = x[np.abs(np.cos(x)) < 0.5]
+    h = np.full((len(x), 1), 2.0 ** -40)
+    i7 = gpu_ctx.eval_rule(G.OSCILLATORY, np.ones(1), np.zeros(1), _soa(x[:, None]), _soa(h),
+                           lanes=lanes)[0].cpu().numpy()
+    err = np.abs((i7 * 2.0 ** 39).astype(LD) - np.cos(x.astype(LD)))
+    assert np.max(err) <= 2.4 * EPS
