@@ -62,17 +62,18 @@ struct GkSums {
 
 // Combine the sums of the region's 32 W lanes in a fixed order: every lane
 // of the region's first warp returns the total (of A unless it is K's).  scratch:
-// [W][9].
-template <int W>
+// [W][9].  SOME: leave out the sums that a dimension lacks (with f at every node
+// the adds cost nothing that the tests for them would not).
+template <int W, bool SOME>
 __device__ __forceinline__ void gk_combine(GkSums& s, int d, bool a_is_k, double* scratch) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     s.K += __shfl_xor_sync(0xffffffffu, s.K, off);
     s.G += __shfl_xor_sync(0xffffffffu, s.G, off);
-    if (!a_is_k) s.A += __shfl_xor_sync(0xffffffffu, s.A, off);
+    if (!SOME || !a_is_k) s.A += __shfl_xor_sync(0xffffffffu, s.A, off);
 #pragma unroll
     for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
-      if (k < d) s.E[k] += __shfl_xor_sync(0xffffffffu, s.E[k], off);
+      if (!SOME || k < d) s.E[k] += __shfl_xor_sync(0xffffffffu, s.E[k], off);
   }
   if constexpr (W > 1) {
     const int w = threadIdx.x >> 5;
@@ -83,7 +84,7 @@ __device__ __forceinline__ void gk_combine(GkSums& s, int d, bool a_is_k, double
       o[2] = s.A;
 #pragma unroll
       for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
-        if (k < d) o[3 + k] = s.E[k];
+        if (!SOME || k < d) o[3 + k] = s.E[k];
     }
     __syncthreads();
     if (w == 0) {
@@ -91,10 +92,10 @@ __device__ __forceinline__ void gk_combine(GkSums& s, int d, bool a_is_k, double
         const double* o = scratch + v * (3 + GMQ_GK_MAX_DIM);
         s.K += o[0];
         s.G += o[1];
-        if (!a_is_k) s.A += o[2];
+        if (!SOME || !a_is_k) s.A += o[2];
 #pragma unroll
         for (int k = 0; k < GMQ_GK_MAX_DIM; ++k)
-          if (k < d) s.E[k] += o[3 + k];
+          if (!SOME || k < d) s.E[k] += o[3 + k];
       }
     }
   }
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
       F = 1.0;
   }
   if (!factors) gk_sums_nodes<FAM, W>(P, K, d, lane, xt[w], xs[w] + lane, s);
-  gk_combine<W>(s, d, factors, scratch);
+  gk_combine<W, kFactors>(s, d, factors, scratch);
   if (lane != 0) return;
   if (factors) s.A = s.K;
   s.K = __dmul_rn(F, s.K);
