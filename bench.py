@@ -118,7 +118,7 @@ RULE_EXEC_INST_D8 = {0: 21845.0, 1: 10203.0, 2: 35602.0, 3: 18265.0, 4: 17747.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "451e1b7c3e7c2315"
+RULE_COUNTS_SHA16 = "b4b63ead73701254"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -133,7 +133,7 @@ MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_int64.cuh", "gm_math_tables.cuh",
                         "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "8695991e1a5f44ea"
+MIXED_COUNTS_SHA16 = "11dcf89af4dc8890"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):
