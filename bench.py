@@ -118,7 +118,7 @@ RULE_EXEC_INST_D8 = {0: 21845.0, 1: 10203.0, 2: 35602.0, 3: 18265.0, 4: 17747.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "b4b63ead73701254"
+RULE_COUNTS_SHA16 = "f4a667cb5e9e549d"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per

@@ -38,8 +38,8 @@ size_t batch_rule_smem(int dmax) {
 }
 
 // Dynamic shared memory from which a launch opts in: the 48 KB that need no
-// opt-in hold the kernel's static arrays (at most 4 KB) too.
-constexpr size_t kBatchOptInSmem = 44 * 1024;
+// opt-in hold the kernel's static arrays (5.5 KB at most) too.
+constexpr size_t kBatchOptInSmem = 40 * 1024;
 
 template <int FAM, int T>
 __device__ __forceinline__ void batch_rule64_lanes(const BatchArgs& B, double* smem,

@@ -196,7 +196,7 @@ cudaError_t launch_rule64_t(const RuleArgs& A, cudaStream_t s) {
     return cudaGetLastError();
   }
   const size_t smem = rule64_smem_bytes<FAM>(A.P.d, T);
-  if (smem > 44 * 1024) {  // with the static arrays of T = 128, below 4 KB, the 48 KB limit
+  if (smem > 40 * 1024) {  // with the static arrays of T = 128, below 8 KB, the 48 KB limit
     cudaError_t e = cudaFuncSetAttribute(k_rule64<FAM, T>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
