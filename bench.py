@@ -114,11 +114,11 @@ RULE_FP64_FLOPS_D8 = {0: 8882.0, 1: 3778.0, 2: 6075.0, 3: 6184.0, 4: 6128.0}
 RULE_EXEC_FP64_INST_D8 = {0: 393.0, 1: 533.0, 2: 222.0, 3: 358.0, 4: 278.0}
 RULE_EXEC_FP64_FLOPS_D8 = {0: 526.0, 1: 802.0, 2: 205.0, 3: 423.0, 4: 295.0}
 # all thread instructions a region (smsp__inst_executed x 32), of the same launches
-RULE_EXEC_INST_D8 = {0: 21845.0, 1: 10203.0, 2: 35602.0, 3: 18265.0, 4: 17747.0}
+RULE_EXEC_INST_D8 = {0: 21845.0, 1: 10592.0, 2: 35602.0, 3: 18662.0, 4: 18171.0}
 RULE_COUNTS_SOURCES = ("gm_rule.cuh", "gm_factor64.cuh", "gm_fixed64.cuh", "gm_int64.cuh",
                        "gm_region64.cuh", "gmq_families.cuh", "gm_math_tables.cuh",
                        "gmq_common.cuh")
-RULE_COUNTS_SHA16 = "f4a667cb5e9e549d"
+RULE_COUNTS_SHA16 = "9453a3c4f3f88f51"
 
 
 # FP32 work of the mixed rule kernel (k_rule_mixed_reg, one thread per
@@ -133,7 +133,7 @@ MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_int64.cuh", "gm_math_tables.cuh",
                         "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "11dcf89af4dc8890"
+MIXED_COUNTS_SHA16 = "b89debc12819b097"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):

@@ -11,8 +11,9 @@
 //                     that family's regions, persistent grid, dimension per
 //                     region; 1, 4, 32 or 128 lanes per region, chosen per
 //                     sweep from the list length (the per-region work is
-//                     gm_region64.cuh's, so the choice never changes a
-//                     result); the mixed form's k_batch_rule_mixed likewise
+//                     region_sums of gm_factor64.cuh, so the choice never
+//                     changes a result); the mixed form's k_batch_rule_mixed
+//                     likewise
 //   k_batch_sums      tiles of 4096 regions of one integral each
 //                     (persistent grid): pairwise-tree sums per tile; the
 //                     integral's last tile adds the tile sums and tests the

@@ -3,9 +3,8 @@
 // per-family kernels in gm_rule_inst.cu).  The batch is in family order, so
 // each family's regions are one contiguous range of the list; a launch walks
 // its family's range on a persistent grid, one thread per region, with the
-// single-integral mixed path's
-// per-region code (gm_region32.cuh): the Gray-code register walk for
-// 3 <= d <= 12, the generic one-thread form otherwise.  So every region gets
+// single-integral mixed path's per-region code (gm_region32.cuh): the tree walk
+// for 3 <= d <= 12, the generic one-thread form otherwise.  So every region gets
 // the bits gmq_integrate's mixed path with one lane per region gives it.
 #pragma once
 

@@ -5,7 +5,7 @@
 // family's range on a persistent grid with T = bs->lanes lanes per region
 // (1, 4, 32 or a 128-thread block; chosen per sweep, never changing a
 // result) and the single-integral FP64 path's per-region code
-// (gm_region64.cuh) specialised for the family, so every region gets the
+// (region_sums, gm_factor64.cuh) specialised for the family, so every region gets the
 // bits gmq_integrate gives it, from a kernel whose registers and code are
 // those of its own integrand rather than of all seven.
 #pragma once

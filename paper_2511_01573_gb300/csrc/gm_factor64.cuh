@@ -3,7 +3,7 @@
 // real part of such a product (the cosine): node values from per-axis
 // factors.  Shared by the single-integral and the batched FP64 rule kernels.
 //
-// Bound: the FP64 pipe (one warp instruction in 64 cycles per SM quarter;
+// Bound: the FP64 pipe (one warp instruction in 76 cycles per SM quarter;
 // integer and shared-memory instructions beside it are nearly free), so the
 // design counts FP64 instructions.  With S = S_0 + Delta_j (+ Delta_k) an
 // exponential node is f = F e_j (e_k): F = f(centre), e = exp(-Delta) one of
@@ -27,8 +27,9 @@
 // (sum |w| is 5.8 at d = 8), and it is formed beyond FP64 (Centre); the factors
 // carry an error near 2^-53 each, whatever their size.  Against 113-bit arithmetic
 // (d = 2..16, slopes 0.5 to 300, random boxes and the whole domain) the rms error of
-// I7 is 0.15 to 1.2 times the separable form's, or, where both are below 2^-53 of
+// I7 is 0.14 to 1.4 times the separable form's, or, where both are below 2^-53 of
 // the terms, up to 1.9 times.
+//
 // Factors may over- or underflow where f does not (a factor is relative to
 // the centre): regions whose factors' exponents do not leave room are
 // evaluated by region_sums64, decided from the region alone, so that every
@@ -479,9 +480,25 @@ __device__ __forceinline__ Limbs limbs_unpack(double w) {
   r.l = __double2loint(w);
   return r;
 }
-// |v| <= 2^E
+// |v| <= 2^E; ties away from zero, for the rotation's entries of both signs
 __device__ __forceinline__ double limbs_of(double v, int E) {
   return limbs_pack(limbs_split(to_fixed(v, 53 - E)));
+}
+// x 2^-k rounded to nearest, to even on ties (for k < 32), 0 <= k <= 62
+__device__ __forceinline__ i64 shift_even(i64 x, int k) {
+  const i64 r = x + (((i64)1 << k) >> 1);
+  const i64 q = r >> k;
+  const bool tie = k > 0 && ((unsigned)r & ((1u << min(k, 31)) - 1u)) == 0u;
+  return tie ? q & ~(i64)1 : q;
+}
+// |v| < 2^E; ties to even: entries of one sign lose the one or two bits by which
+// they are below the table's largest, and ties rounded up put 0.6 to 0.9 of 2^-53
+// on the class sums
+__device__ __forceinline__ double limbs_even(double v, int E) {
+  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff, k = E + 1022 - e;
+  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+  const i64 q = k < 56 ? shift_even(m, k) : 0;
+  return limbs_pack(limbs_split(hi < 0 ? -q : q));
 }
 
 constexpr int kLimbRun = 512;  // products that a LimbAcc takes before it may overflow
@@ -869,18 +886,7 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
       t2.push(q2);
       t3.push(q3);
     }
-    // argmax over the lanes: larger D wins, the lower axis on ties (T = 128:
-    // the d <= 16 leaves sit in warp 0, whose lane 0 alone uses the axis)
-    constexpr int WL = T < 32 ? T : 32;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(mask, dbest, off, WL);
-      const int ok = __shfl_xor_sync(mask, kbest, off, WL);
-      if (od > dbest || (od == dbest && ok < kbest)) {
-        dbest = od;
-        kbest = ok;
-      }
-    }
+    lanes_argmax<T>(dbest, kbest, mask);
     bool pr2, pr3;
     const double x2 = t2.flush(pr2), x3 = t3.flush(pr3);
     s2 = lanes_tree<T>(x2, pr2, mask);
@@ -900,14 +906,14 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
   for (int k = lane; k < d; k += T) {
     const double p3 = W(Ly.e3 + 2 * k), m3 = W(Ly.e3 + 2 * k + 1);
     const int E = max(exp_bound(p3), exp_bound(m3));
-    W(Ly.e3 + 2 * k) = limbs_of(p3, E);
-    W(Ly.e3 + 2 * k + 1) = limbs_of(m3, E);
+    W(Ly.e3 + 2 * k) = limbs_even(p3, E);
+    W(Ly.e3 + 2 * k + 1) = limbs_even(m3, E);
     W(Ly.x3 + k) = __hiloint2double(E, 0);
     M2 = max(M2, min(M1, E));
     M1 = max(M1, E);
   }
   for (int q = lane; q < nA + nB + nC; q += T)
-    W(Ly.A + q) = limbs_of(W(Ly.A + q), q < nA ? EA : (q < nA + nB ? EB : EC));
+    W(Ly.A + q) = limbs_even(W(Ly.A + q), q < nA ? EA : (q < nA + nB ? EB : EC));
   if constexpr (T > 1) group_sync<T>(mask);
   if constexpr (T > 1 || SF::kFlag) {
     // (a flagged centre leaves the pairs that move its axis)
@@ -952,7 +958,7 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
     pair.mid += ((i64)(j0.l + j1.l) * (k0.l + k1.l)) >> 27;
     const int sh = min(
         M1 + M2 - __double2hiint(W(Ly.x3 + j)) - __double2hiint(W(Ly.x3 + k)), 62);
-    s4 += (pair.number() + (((i64)1 << sh) >> 1)) >> sh;
+    s4 += shift_even(pair.number(), sh);
   }
   // class 5
   const Limbs one{1 << 26, 0};
@@ -1186,16 +1192,7 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
       t2.push(q2);
       t3.push(q3);
     }
-    constexpr int WL = T < 32 ? T : 32;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(mask, dbest, off, WL);
-      const int ok = __shfl_xor_sync(mask, kbest, off, WL);
-      if (od > dbest || (od == dbest && ok < kbest)) {
-        dbest = od;
-        kbest = ok;
-      }
-    }
+    lanes_argmax<T>(dbest, kbest, mask);
     bool pr2, pr3;
     const double x2 = t2.flush(pr2), x3 = t3.flush(pr3);
     s2 = lanes_tree<T>(x2, pr2, mask);

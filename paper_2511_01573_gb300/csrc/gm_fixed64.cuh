@@ -294,18 +294,7 @@ __device__ __forceinline__ bool region_sums64_corner(const PT& P, int d,
       W(e0 + q0) = v;
     }
     group_sync<T>(mask);
-    // argmax over the lanes: larger D wins, the lower axis on ties (T = 128:
-    // the d <= 16 axes sit in warp 0, whose lane 0 alone uses the axis)
-    constexpr int WL = T < 32 ? T : 32;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(mask, dbest, off, WL);
-      const int ok = __shfl_xor_sync(mask, kbest, off, WL);
-      if (od > dbest || (od == dbest && ok < kbest)) {
-        dbest = od;
-        kbest = ok;
-      }
-    }
+    lanes_argmax<T>(dbest, kbest, mask);
   }
   // class 4
   const int np = d * (d - 1) / 2;

@@ -300,10 +300,10 @@ __global__ void __launch_bounds__(kGkBlock) k_rule_gk(const GkArgs G) {
     if (active && lane < d) bound[w][lane] = exp_bound(__hiloint2double(bound[w][lane], 0));
     __syncthreads();
     if (active) {
-      for (int q = lane; q < 15; q += L) kt[q] = limbs_of(kt[q], bound[w][0]);
+      for (int q = lane; q < 15; q += L) kt[q] = limbs_even(kt[q], bound[w][0]);
       for (int q = 15 + lane; q < d * 15; q += L)
         reinterpret_cast<u64*>(kt)[q] = gk_word(kt[q]);
-      for (int j = lane; j < 15; j += L) rt[j] = limbs_of(rt[j], bound[w][0] + 1);
+      for (int j = lane; j < 15; j += L) rt[j] = limbs_even(rt[j], bound[w][0] + 1);
     }
     __syncthreads();
   }

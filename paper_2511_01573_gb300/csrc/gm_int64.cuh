@@ -21,7 +21,8 @@ __device__ __forceinline__ void mad_wide(i64& acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
 
-// round(x 2^q) for |x| < 2^(62 - q), by integer operations
+// round(x 2^q) for |x| < 2^(63 - q), modulo 2^64 for |x| < 2^(68 - q), by integer
+// operations
 __device__ __forceinline__ i64 to_fixed(double x, int q) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) & 0x7ff;

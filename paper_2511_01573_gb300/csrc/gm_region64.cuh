@@ -157,6 +157,22 @@ __device__ __forceinline__ double lanes_tree(double x, bool present, unsigned ma
   return present ? x : 0.0;
 }
 
+// Largest fourth difference over the group and its axis, the lower one on ties
+// (T = 128: the d <= 16 axes sit in warp 0, whose lane 0 alone uses the axis).
+template <int T>
+__device__ __forceinline__ void lanes_argmax(double& dbest, int& kbest, unsigned mask) {
+  constexpr int W = T < 32 ? T : 32;
+#pragma unroll
+  for (int off = W / 2; off > 0; off >>= 1) {
+    const double od = __shfl_xor_sync(mask, dbest, off, W);
+    const int ok = __shfl_xor_sync(mask, kbest, off, W);
+    if (od > dbest || (od == dbest && ok < kbest)) {
+      dbest = od;
+      kbest = ok;
+    }
+  }
+}
+
 // One class sum over n nodes, val(q) = f at the class's node q.
 template <int T, class Val>
 __device__ __forceinline__ double class_sum(int n, int lane, unsigned mask, Val val) {
@@ -506,19 +522,7 @@ __device__ __forceinline__ void region_sums64(const PT& P, int d, const unsigned
         kbest = k;
       }
     }
-    // argmax over the lanes: larger D wins, the lower axis on ties (for
-    // T = 128 every axis k < d <= 16 sits in warp 0, which holds the answer
-    // for lane 0, the only lane that uses it)
-    constexpr int WL = T < 32 ? T : 32;
-#pragma unroll
-    for (int off = WL / 2; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(mask, dbest, off, WL);
-      const int ok = __shfl_xor_sync(mask, kbest, off, WL);
-      if (od > dbest || (od == dbest && ok < kbest)) {
-        dbest = od;
-        kbest = ok;
-      }
-    }
+    lanes_argmax<T>(dbest, kbest, mask);
     // classes 2 and 3 hold 2d <= 32 nodes: one node per chunk
     PairTree t2, t3;
     const int p0 = lane_first_chunk<T>(lane), p1 = min(p0 + kChunks / T, 2 * d);
@@ -684,19 +688,7 @@ __device__ __forceinline__ void region_sums64_nodewise(const PT& P, int d,
         kbest = k;
       }
     }
-    // argmax over the lanes: larger D wins, the lower axis on ties (for
-    // T = 128 every axis k < d <= 16 sits in warp 0, which holds the answer
-    // for lane 0, the only lane that uses it)
-    constexpr int W = T < 32 ? T : 32;
-#pragma unroll
-    for (int off = W / 2; off > 0; off >>= 1) {
-      const double od = __shfl_xor_sync(mask, dbest, off, W);
-      const int ok = __shfl_xor_sync(mask, kbest, off, W);
-      if (od > dbest || (od == dbest && ok < kbest)) {
-        dbest = od;
-        kbest = ok;
-      }
-    }
+    lanes_argmax<T>(dbest, kbest, mask);
     // classes 2 and 3 hold 2d <= 32 nodes: one node per chunk
     PairTree t2, t3;
     const int p0 = lane_first_chunk<T>(lane), p1 = min(p0 + kChunks / T, 2 * d);

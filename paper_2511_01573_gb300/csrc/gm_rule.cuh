@@ -16,13 +16,15 @@
 //      decoded from the bits of its index (centre; 4d axis nodes; 4 sign
 //      patterns per axis pair; the 2^d sign patterns of the last class are
 //      the bits of the index itself).  Every node's value is formed and
-//      added: one fused multiply-add of two factors, or the outer function
-//      of its inner sum and an add;
+//      added: a product of two factors as two-limb integers (an FP64 add on
+//      the axes), a power in fixed point (the corner peak), or the outer
+//      function of its inner sum and an add;
 //   3. combines the class sums over the T lanes, finds the split axis
 //      (argmax of the fourth differences) and writes I7, the error estimate,
 //      vol / vol(Omega) and the axis byte.
 // The per-region work is region_sums (gm_factor64.cuh) and region_finish64
-// (gm_region64.cuh), whose fixed summation tree makes the results bit-identical for every T.
+// (gm_region64.cuh); exact integer sums and fixed summation trees make the
+// results bit-identical for every T.
 #pragma once
 
 #include "gm_factor64.cuh"
@@ -55,7 +57,7 @@ inline size_t rule64_smem_bytes(int d, int T) {
 }
 
 // FP64 rule kernel; per-region work shared with the batched kernel
-// (gm_region64.cuh).
+// (region_sums, gm_factor64.cuh).
 template <int FAM, int T>
 __global__ void __launch_bounds__(kRuleBlock) k_rule64(const RuleArgs A) {
   constexpr int RB = kRuleBlock / T;

@@ -8,8 +8,8 @@
 //   k_rule_mixed      any dimension, T = 1, 4 or 32 lanes per region (the
 //                     lanes' compensated sums combined by a butterfly)
 //   k_rule_mixed_reg  one thread per region, 3 <= d <= 12 known at compile
-//                     time: the 2^d sign-pattern nodes walked in Gray-code
-//                     order in registers (region_mixed_walk)
+//                     time: the nodes walked as a tree over the axes, prefixes
+//                     of the chains in registers (region_mixed_walk)
 #pragma once
 
 #include "gm_region32.cuh"
@@ -222,11 +222,10 @@ __global__ void __launch_bounds__(kRuleBlock) k_rule_mixed(const RuleArgs A) {
 }
 
 // Mixed form, one thread per region, dimension D known at compile time:
-// the sign-pattern nodes are walked in Gray-code order in registers
-// (region_mixed_walk).
+// the nodes are walked as a tree over the axes (region_mixed_walk).
 template <int FAM, int D>
 __global__ void __launch_bounds__(kRuleBlock) k_rule_mixed_reg(const RuleArgs A) {
-  static_assert(D >= 3 && D <= 16, "gray walk needs D >= 3");
+  static_assert(D >= 3 && D <= 16, "the walk needs D >= 3");
   constexpr int RB = kRuleBlock;
   constexpr int d = D;
   // shared memory: the FP32 coordinate table and the FP32 parameters only
