@@ -133,7 +133,7 @@ MIXED_FP32_OPS_D12 = {2: 85007.0, 3: 71949.0}
 MIXED_COUNTS_SOURCES = ("gm_rule_mixed.cuh", "gm_region32.cuh", "gm_region64.cuh",
                         "gmq_families.cuh", "gm_int64.cuh", "gm_math_tables.cuh",
                         "gmq_common.cuh")
-MIXED_COUNTS_SHA16 = "b89debc12819b097"
+MIXED_COUNTS_SHA16 = "a56e1e2ec571dacc"
 
 
 def rule_source_fingerprint(files=RULE_COUNTS_SOURCES):

@@ -151,8 +151,11 @@ struct Chain {
   // a: the axis' factor of y (not used by the product peak and the polynomial);
   // u: its threshold (the discontinuous family: -inf, whose exponential is 0,
   // from the first coordinate above it)
+  // (a slope beyond FP32's range is kept finite there: infinity times a coordinate
+  // would make a NaN of the -inf)
   template <class PT>
   __device__ __forceinline__ static float coef(const PT& P, int j) {
+    if constexpr (kDisc) return fminf(fmaxf(P.a[j], -3.402823466e38f), 3.402823466e38f);
     return kGauss ? P.b[j] : P.a[j];
   }
   __device__ __forceinline__ static float step(float s, float a, float u, float v) {

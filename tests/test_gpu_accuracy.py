@@ -241,3 +241,17 @@ def test_mean_error_of_table_roundings(gpu_ctx, fam, lo, hi):
             ref, terms = _exact_i7(fam, a, u, c[i], h[i])
             err.append(float((LD(i7[i]) / np.prod((2 * h[i]).astype(LD)) - ref) / terms) / EPS)
     assert abs(np.mean(err)) <= 0.1
+
+
+@pytest.mark.parametrize("lanes", [1, 4, 32])
+@pytest.mark.parametrize("d", [3, 6, 12])
+def test_mixed_flagged_region_with_a_slope_beyond_fp32(gpu_ctx, lanes, d):
+    """A region above the discontinuous integrand's threshold on its first axis is 0,
+    whatever the slopes on the axes after it."""
+    from paper_2511_01573_gb300 import gmq
+    a, u = np.ones(d), np.full(d, 2.0)
+    a[1:], u[0] = 1e39, -1.0
+    c = np.random.default_rng(d).uniform(0.3, 0.7, (9, d))
+    i7, err, _, _ = gpu_ctx.eval_rule(G.DISCONTINUOUS, a, u, _soa(c), _soa(np.full((9, d), 0.1)),
+                                      precision=gmq.MIXED, lanes=lanes)
+    assert torch.all(i7 == 0.0) and torch.all(err == 0.0)
