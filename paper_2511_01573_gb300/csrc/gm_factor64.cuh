@@ -17,8 +17,8 @@
 // Limbs below).  Measured at d = 8, 2^20 regions, one thread per region, against
 // the outer function at every node: C0 8.14 -> 0.94 ms (4080 -> 278 FP64
 // instructions a region), Gaussian 8.25 -> 1.04, product peak 4.71 -> 1.12,
-// cosine 10.99 -> 1.40; with factors and FP64 sums and functions they took 2.23,
-// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (48-82 % active) is the
+// cosine 10.99 -> 1.42; with factors and FP64 sums and functions they took 2.23,
+// 2.34, 2.00 and 3.31 ms.  What is left on the FP64 pipe (46-82 % active) is the
 // coordinates, the chains and the weights; twelve warps an SM, as many as the
 // workspaces in shared memory let.
 //
@@ -27,7 +27,7 @@
 // (sum |w| is 5.8 at d = 8), and it is formed beyond FP64 (Centre); the factors
 // carry an error near 2^-53 each, whatever their size.  Against 113-bit arithmetic
 // (d = 2..16, slopes 0.5 to 300, random boxes and the whole domain) the rms error of
-// I7 is 0.14 to 1.4 times the separable form's, or, where both are below 2^-53 of
+// I7 is 0.01 (cosine) to 1.4 times the separable form's, or, where both are below 2^-53 of
 // the terms, up to 1.9 times.
 //
 // Factors may over- or underflow where f does not (a factor is relative to
@@ -298,8 +298,8 @@ __device__ __forceinline__ double one_factor(const PT& P, int k, double c, doubl
 // F = f(centre) from the axes' phi in order.  Its error is common to every
 // node, so the inner sum is kept in units of 2^-58, roundings of phi included, as
 // a 64-bit integer modulo 2^64 (for |S| < 512 and every |phi| < 512, where the
-// rounded S tells the multiple of 64; in FP64 otherwise; the cosine's below 16),
-// and the product peak's product as a sum of two doubles.
+// rounded S tells the multiple of 64; in FP64 otherwise), and the product peak's
+// product as a sum of two doubles.
 template <int FAM>
 struct Centre {
   double S, lo = 0.0;
@@ -347,10 +347,15 @@ struct Centre {
     }
   }
   __device__ __forceinline__ void sincos(double& sn, double& cs) const {
-    if (!fixed || !sincos_near(S))
+    if (!fixed || !small(S)) {
       gm_sincos(S, &sn, &cs);
-    else
-      sincos_fixed(v, 58, &sn, &cs);
+      return;
+    }
+    // less the whole turns (2 pi 2^58 = L + L1 2^-32) that a rounded S of 16 and
+    // more tells
+    const i64 L = 0x1921fb54442d1846ll;
+    const int n = sincos_near(S) ? 0 : round_mul_int(S, 0.159154943f);
+    sincos_fixed(v - n * L - (((i64)n * 0x9898cc51ll) >> 32), 58, &sn, &cs);
   }
 };
 
@@ -1022,6 +1027,27 @@ __device__ __forceinline__ bool region_sums64_real(const PT& P, int d, const uns
   return true;
 }
 
+// cos and sin of lam a h, |lam| < 1, for N lam: the angle in units of 2^-58 (2^-54
+// where |a h| is 16 and more), a h and its rounding error times lam; in FP64 where
+// |a h| is 256 and more.  An angle is shared by half of the nodes: rounded
+// relative to its own size it moved I7 of steep integrands by twice what nodes'
+// own inner sums, rounded each for itself, do.
+template <class PT, int N>
+__device__ __forceinline__ void rotations(const PT& P, int k, double h, const double (&lam)[N],
+                                          double (&cs)[N], double (&sn)[N]) {
+  const double ah = __dmul_rn(P.a[k], h);
+  if (below_256(ah)) {
+    const int q = sincos_near(ah) ? 58 : 54;
+    const i64 lin = to_fixed(ah, q + 1) + to_fixed(fma(P.a[k], h, -ah), q + 1);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      sincos_fixed(fixed_mul_signed(lin, lam_fixed(lam[i])), q, &sn[i], &cs[i]);
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) gm_sincos(__dmul_rn(lam[i], ah), &sn[i], &cs[i]);
+  }
+}
+
 // The same for the cosine: f = Re(F prod (cos Delta_k +- i sin Delta_k)),
 // F = cos S_0 + i sin S_0, Delta = a lambda h.
 template <int FAM, int T, class PT, class CH>
@@ -1076,18 +1102,10 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
     for (int k = 0; k < d; ++k) {
       double c, h;
       ch(k, c, h);
-      const double ah = __dmul_rn(P.a[k], h);
-      double c2, n2, c3, n3, c5, n5;
-      const double z2 = __dmul_rn(lam2, ah), z3 = __dmul_rn(lam3, ah), z5 = __dmul_rn(lam5, ah);
-      if (sincos_near(z2) && sincos_near(z3) && sincos_near(z5)) {
-        sincos_fixed(to_fixed(z2, 58), 58, &n2, &c2);
-        sincos_fixed(to_fixed(z3, 58), 58, &n3, &c3);
-        sincos_fixed(to_fixed(z5, 58), 58, &n5, &c5);
-      } else {
-        gm_sincos(z2, &n2, &c2);
-        gm_sincos(z3, &n3, &c3);
-        gm_sincos(z5, &n5, &c5);
-      }
+      const double lam[3] = {lam2, lam3, lam5};
+      double cs[3], sn[3];
+      rotations(P, k, h, lam, cs, sn);
+      const double c2 = cs[0], n2 = sn[0], c3 = cs[1], n3 = sn[1], c5 = cs[2], n5 = sn[2];
       W(Ly.e3 + 2 * k) = c3;
       W(Ly.e3 + 2 * k + 1) = n3;
       double q2, q3;
@@ -1122,12 +1140,12 @@ __device__ __forceinline__ void region_sums64_rotation(const PT& P, int d,
       const int k = t / 3, r = t - 3 * k;
       double c, h;
       ch(k, c, h);
-      const double ah = __dmul_rn(P.a[k], h);
-      double sn, cs;
-      gm_sincos(__dmul_rn(r == 0 ? lam2 : (r == 1 ? lam3 : lam5), ah), &sn, &cs);
+      const double lam[1] = {r == 0 ? lam2 : (r == 1 ? lam3 : lam5)};
+      double cs[1], sn[1];
+      rotations(P, k, h, lam, cs, sn);
       const int e = (r == 0 ? Ly.e2 : (r == 1 ? Ly.e3 : Ly.e5)) + 2 * k;
-      W(e) = cs;
-      W(e + 1) = sn;
+      W(e) = cs[0];
+      W(e + 1) = sn[0];
       if (r == 0) W(Ly.phiC + k) = SF::phi(P, k, c);
     }
     group_sync<T>(mask);

@@ -255,3 +255,28 @@ def test_mixed_flagged_region_with_a_slope_beyond_fp32(gpu_ctx, lanes, d):
     i7, err, _, _ = gpu_ctx.eval_rule(G.DISCONTINUOUS, a, u, _soa(c), _soa(np.full((9, d), 0.1)),
                                       precision=gmq.MIXED, lanes=lanes)
     assert torch.all(i7 == 0.0) and torch.all(err == 0.0)
+
+
+def _exact_cosine(fam, a, u, c, h):
+    d = len(a)
+    c0 = LD(2.0 * np.pi * u[0])
+    a, c, h = (np.asarray(v, dtype=LD) for v in (a, c, h))
+    f0 = np.cos(c0 + np.sum(a * c))
+    z = [2 * np.cos(LD(np.sqrt(v)) * a * h) for v in (9 / 70, 9 / 10, 9 / 19)]
+    s4 = (np.sum(z[1]) ** 2 - np.sum(z[1] ** 2)) / 2
+    s = [LD(1), np.sum(z[0]), np.sum(z[1]), s4, np.prod(z[2])]
+    n = [1, 2 * d, 2 * d, 2 * d * (d - 1), 2 ** d]
+    w = [LD(v / 19683) for v in (12824 - 9120 * d + 400 * d * d, 2940, 1820 - 400 * d, 200,
+                                 6859 / 2 ** d)]
+    return f0 * sum(x * y for x, y in zip(w, s)), sum(abs(x) * y for x, y in zip(w, n))
+
+
+@pytest.mark.parametrize("whole", [False, True])
+@pytest.mark.parametrize("lo,hi,d", [(5, 15, 4), (5, 15, 8), (5, 15, 14), (30, 90, 3), (0.5, 3, 6)])
+def test_steep_cosine(gpu_ctx, lo, hi, d, whole):
+    """Angles and the centre's sum in fixed point, half a unit of 2^-57 each: what is
+    left is the roundings of the products, below half an eps of the terms, whatever
+    the sum's size, which the node-wise form's error grows with."""
+    mine, node = _rms_errors(gpu_ctx, G.OSCILLATORY, _cases(G.OSCILLATORY, d, 48, lo, hi, whole, d),
+                             _exact_cosine)
+    assert mine <= 0.5 * EPS + 0.25 * node
